@@ -163,7 +163,13 @@ const char *nb_last_error(void);
 void nb_params_default(nb_params *p);
 
 /* Create a context for up to n_capacity particles (1 <= n_capacity <= 2^26)
- * on p->device.  Allocates all device memory the context will use.
+ * on p->device.  Allocates the device memory of its state; the pair kernels'
+ * partial sums are allocated by the first nb_load and may grow in a later
+ * nb_load, nb_set_precision, nb_set_cluster_params or nb_tune (24 bytes per
+ * body and slot; the kernels that evaluate each pair once use about N / 1024
+ * slots, up to 4 GB in all, beyond which, or where the device has no room, the
+ * N x N kernels run with a few dozen).  Nothing is allocated by a step or an
+ * evaluation.
  * *out receives the context.  Errors: NB_EINVAL (bad parameters),
  * NB_ENOMEM, NB_ECUDA. */
 int nb_create(const nb_params *p, int64_t n_capacity, nb_ctx **out);
@@ -441,7 +447,8 @@ typedef struct {
     double hbm_budget_bytes;  /* device memory for resident state (> 0);
                                  about 436 bytes per body slot, plus the
                                  groups' partial sums beyond that share (at
-                                 most ~67 MB per group of the twelve) */
+                                 most ~67 MB or a 32nd of the budget,
+                                 whichever is more, per group of the twelve) */
     int max_jobs;             /* resident jobs at most, 1..65536 */
     double G;                 /* as nb_params */
     int ext_on;

@@ -31,33 +31,35 @@ const char *last_error() { return g_err.c_str(); }
 
 // ---- pool --------------------------------------------------------------------
 
-int64_t part_elems_for(const Pool &P, int64_t n)
+int device_sms(int device)
 {
-    const int64_t giw = (int64_t)P.num_sms * MAX_WAVES * 3072;
+    int v = 0;
+    if (cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, device) != cudaSuccess) return 0;
+    return v;
+}
+
+// Partial sums of the full decomposition: a set of n bodies needs about
+// G * ipb / n + 2 slots per body, where G * ipb <= SMs * MAX_WAVES *
+// (resident blocks * i-block width) and the last factor is at most 3072 for
+// every compiled variant (8 x 256, 6 x 512, 3 x 1024).  The planes are laid
+// out per set (stride n, linear body index), so 3 (giw + 2 n) doubles give
+// its n bodies (giw + 2 n) / n slots whatever the pool's size.  make_decomp
+// shrinks a grid that would need more than a set has.
+int64_t part_elems_for(int sms, int64_t n)
+{
+    const int64_t giw = (int64_t)sms * MAX_WAVES * 3072;
     const int64_t slots_n = giw + 2 * n, cap_n = MAX_PART_SLOTS * n;
     return 3 * (slots_n < cap_n ? slots_n : cap_n);
 }
 
-int pool_create(Pool &P, int device, int64_t cap, bool own_part)
+int pool_create(Pool &P, int device, int64_t cap)
 {
     P.device = device;
     P.cap = cap;
-    if (cudaDeviceGetAttribute(&P.num_sms, cudaDevAttrMultiProcessorCount, device) !=
-        cudaSuccess)
-        return set_error(NB_ECUDA, "cudaDeviceGetAttribute failed");
+    P.num_sms = device_sms(device);
+    if (P.num_sms < 1) return set_error(NB_ECUDA, "cudaDeviceGetAttribute failed");
     DevState &s = P.s;
     s.cap = cap;
-    // partial sums: a set of n bodies needs about G * ipb / n + 2 slots per
-    // body, where G * ipb <= SMs * MAX_WAVES * (resident blocks * i-block
-    // width) and the last factor is at most 3072 for every compiled variant
-    // (8 x 256, 6 x 512, 3 x 1024).  The planes are laid out per set (stride
-    // n, linear body index), so 3 (giw + 2 cap) doubles give a set of n
-    // bodies (giw + 2 cap) / n slots: a small set in a large pool (a serving
-    // group) gets as many as a context of its own size.  make_decomp
-    // shrinks a grid that would need more than a set has.  Sets that run
-    // concurrently in one pool (the serving loop's groups) cannot share this
-    // storage: such a pool has none, and each set reserves its own.
-    s.part_elems = own_part ? part_elems_for(P, cap) : 0;
     s.part_slots = 0;
     s.pstride = 0;
     s.red_len = 0;
@@ -75,7 +77,6 @@ int pool_create(Pool &P, int device, int64_t cap, bool own_part)
     A((void **)&s.xl, c4); A((void **)&s.yl, c4); A((void **)&s.zl, c4);
     A((void **)&s.jd, 2 * (size_t)cap * sizeof(float4));
     A((void **)&s.jl, 2 * (size_t)cap * sizeof(float4));
-    if (s.part_elems > 0) A((void **)&s.part, (size_t)s.part_elems * 8);
     A((void **)&s.corr, 3 * c8);
     A((void **)&P.stage, 7 * c8);
     if (!ok) {
@@ -113,7 +114,7 @@ int set_create(ClusterSet &C, int32_t kcap, int64_t body_cap, int priority)
     const size_t bytes = al(k8) * 2 + al(k81) * 3 + al((size_t)kcap * 4) * 2 + al(k8) * 2 +
                          al((size_t)C.scap * 4) + al((size_t)C.scap * 8) * 2 +
                          al((size_t)(kcap + 1) * 4) + al((size_t)kcap * sizeof(Frame)) +
-                         al((size_t)kcap * DIAG_STRIDE * 8) + al(k8);
+                         al((size_t)kcap * DIAG_STRIDE * 8) + al(k8) * 3;
     if (cudaMalloc(&C.dmem, bytes) != cudaSuccess) {
         cudaGetLastError();
         C.dmem = nullptr;
@@ -162,18 +163,23 @@ int set_reserve_part(ClusterSet &C, int64_t elems, cudaStream_t st)
     const int64_t want = C.part ? (elems > C.part_elems * 3 / 2 ? elems : C.part_elems * 3 / 2)
                                 : elems;
     if (C.part) {
-        NB_TRY(cudaFreeAsync(C.part, st));
+        NB_TRY(C.part_ordered ? cudaFreeAsync(C.part, st) : cudaFree(C.part));
         C.part = nullptr;
         C.part_elems = 0;
     }
     void *q = nullptr;
-    if (cudaMallocAsync(&q, (size_t)want * 8, st) != cudaSuccess) {
-        cudaGetLastError();
+    for (const int64_t e : {want, elems})
+        if (!q && (C.part_ordered ? cudaMallocAsync(&q, (size_t)e * 8, st)
+                                  : cudaMalloc(&q, (size_t)e * 8)) == cudaSuccess) {
+            C.part_elems = e;
+        } else if (!q) {
+            cudaGetLastError();
+            q = nullptr;
+        }
+    if (!q)
         return set_error(NB_ENOMEM, "partial-sum storage: %lld bytes not available",
-                         (long long)want * 8);
-    }
+                         (long long)elems * 8);
     C.part = static_cast<double *>(q);
-    C.part_elems = want;
     return NB_OK;
 }
 
@@ -224,7 +230,7 @@ int set_define(ClusterSet &C, int32_t K, const int64_t *boff, const int64_t *nk,
     return NB_OK;
 }
 
-int set_layout(ClusterSet &C, int ipb, cudaStream_t st, int jt)
+int set_units(ClusterSet &C, int ipb, int jt, bool sym)
 {
     if (jt < 32 || jt > TILE || TILE % jt != 0)
         return set_error(NB_EINVAL, "j-range width %d must divide %d and be >= 32", jt, TILE);
@@ -233,18 +239,29 @@ int set_layout(ClusterSet &C, int ipb, cudaStream_t st, int jt)
     C.ipb = ipb;
     C.ntiles.resize(K);
     C.uoff.assign(K + 1, 0);
-    C.uoff_pot.assign(K + 1, 0);
+    C.poff.assign(K, 0);
+    C.poff_pot.assign(K, 0);
     C.max_ntiles = 0;
-    C.seg_off.assign(K + 1, 0);
-    C.seg_k.clear();
-    C.seg_lo.clear();
-    C.seg_hi.clear();
     for (int32_t k = 0; k < K; ++k) {
         const int64_t nt = (C.nk[k] + TILE - 1) / TILE;
         C.ntiles[k] = (int32_t)nt;
         if (nt > C.max_ntiles) C.max_ntiles = nt;
         C.uoff[k + 1] = C.uoff[k] + ((C.nk[k] + ipb - 1) / ipb) * nt * per_tile;
-        C.uoff_pot[k + 1] = C.uoff_pot[k] + nt * nt;
+    }
+    if (sym) sym_units(C.nk.data(), K, ipb, jt, C.uoff.data());
+    C.uoff_pot.assign(K + 1, 0);
+    sym_units(C.nk.data(), K, TILE * POT_I, POT_JT, C.uoff_pot.data());
+    return NB_OK;
+}
+
+int set_layout(ClusterSet &C, cudaStream_t st)
+{
+    const int32_t K = C.K;
+    C.seg_off.assign(K + 1, 0);
+    C.seg_k.clear();
+    C.seg_lo.clear();
+    C.seg_hi.clear();
+    for (int32_t k = 0; k < K; ++k) {
         for (int64_t lo = C.noff[k]; lo < C.noff[k + 1]; lo += SEG_BODIES) {
             C.seg_k.push_back(k);
             C.seg_lo.push_back(lo);
@@ -278,6 +295,8 @@ int set_layout(ClusterSet &C, int ipb, cudaStream_t st, int jt)
     C.frame = (Frame *)take((size_t)C.kcap * sizeof(Frame));
     C.diag = (double *)take((size_t)C.kcap * DIAG_STRIDE * 8);
     double *d_mu = (double *)take(k8);
+    int64_t *d_poff = (int64_t *)take(k8);
+    int64_t *d_poffp = (int64_t *)take(k8);
     if ((int32_t)C.mu.size() != K) C.mu.assign(K, 0.0);
     auto up = [&](void *dst, const void *src, size_t bytes) {
         return bytes ? cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, st)
@@ -293,6 +312,8 @@ int set_layout(ClusterSet &C, int ipb, cudaStream_t st, int jt)
     NB_TRY(up(d_eps2d, C.eps2d.data(), K * 8));
     NB_TRY(up(d_dts, C.dts.data(), K * 8));
     NB_TRY(up(d_mu, C.mu.data(), K * 8));
+    NB_TRY(up(d_poff, C.poff.data(), K * 8));
+    NB_TRY(up(d_poffp, C.poff_pot.data(), K * 8));
     NB_TRY(up(d_segk, C.seg_k.data(), S * 4));
     NB_TRY(up(d_seglo, C.seg_lo.data(), S * 8));
     NB_TRY(up(d_seghi, C.seg_hi.data(), S * 8));
@@ -308,6 +329,7 @@ int set_layout(ClusterSet &C, int ipb, cudaStream_t st, int jt)
     c.eps2d = d_eps2d;
     c.dts = d_dts;
     c.mu = d_mu;
+    c.poff = d_poff;
     c.frame = C.frame;
     c.S = (int32_t)S;
     c.seg_k = d_segk;
@@ -321,6 +343,7 @@ int set_layout(ClusterSet &C, int ipb, cudaStream_t st, int jt)
     NB_TRY(cudaStreamSynchronize(st));
     C.cl_pot = c;
     C.cl_pot.uoff = d_uoffp;
+    C.cl_pot.poff = d_poffp;
     return NB_OK;
 }
 
@@ -399,13 +422,44 @@ void block_order(ClusterSet &C, const Decomp &d, int I, bool partial)
     C.bperm_ipb = d.ipb;
 }
 
+// Whether a set takes the symmetric kernels, where their slots fit.  The modes
+// of FP64-class accuracy do: the order of their sums moves results by 1e-14.
+static bool use_sym(int mode) { return mode == PM_FP64 || mode == PM_DD; }
+
+// Bodies per thread without a tuned entry, full decomposition.
+static int full_default_I(const ClusterSet &C, int mode)
+{
+    const int64_t mean = C.n / (C.K > 0 ? C.K : 1);
+    switch (mode) {
+    case PM_FP64: return 1;
+    case PM_DD: return 2;   // measured fastest at N = 262144
+    case PM_DS_FULL: return mean < 16384 ? 2 : 4;
+    default:
+        // float pairs (mixed and pure float): 8 bodies per thread measured
+        // fastest at N = 65536 and N = 262144 and on the 512-cluster
+        // ensemble (mean N 2519); small clusters keep 2 so the i-blocks
+        // stay narrow enough to give every resident block a unit
+        return mean < 2048 ? 2 : 8;
+    }
+}
+
+// The same for the symmetric one, by the work-weighted mean cluster size.
+static int sym_default_I(const ClusterSet &C, int mode)
+{
+    double n2 = 0;
+    for (int32_t k = 0; k < C.K; ++k) n2 += (double)C.nk[k] * (double)C.nk[k];
+    const double wn = n2 / (double)C.n;
+    if (mode == PM_FP64) return wn < 32768 ? 1 : 2;
+    return wn < 6144 ? 2 : 4;   // measured: pairsym_wide.cu
+}
+
 int plan_make(const Pool &P, ClusterSet &C, int precision, cudaStream_t st, Plan &out,
               const PairShape *force, bool use_table, int waves)
 {
     Plan pl;
     pl.precision = precision;
     pl.pl.mode = plan_mode(C, precision);
-    const int64_t mean = C.n / (C.K > 0 ? C.K : 1);
+    bool sym = use_sym(pl.pl.mode);
     int I, bps = 0, jt = 0;
     PairShape tuned;
     if (force) {
@@ -417,47 +471,55 @@ int plan_make(const Pool &P, ClusterSet &C, int precision, cudaStream_t st, Plan
         I = tuned.I;
         bps = tuned.blocks_per_sm;
         jt = tuned.jt;
-    } else if (pl.pl.mode == PM_FP64) {
-        I = 1;
-    } else if (pl.pl.mode == PM_DD) {
-        I = 2;   // measured fastest at N = 262144
-    } else if (pl.pl.mode == PM_DS_FULL) {
-        I = mean < 16384 ? 2 : 4;
     } else {
-        // float pairs (mixed and pure float): 8 bodies per thread measured
-        // fastest at N = 65536 and N = 262144 and on the 512-cluster
-        // ensemble (mean N 2519); small clusters keep 2 so the i-blocks
-        // stay narrow enough to give every resident block a unit
-        I = mean < 2048 ? 2 : 8;
+        I = sym ? sym_default_I(C, pl.pl.mode) : full_default_I(C, pl.pl.mode);
     }
     if (!pair_variant_exists(pl.pl.mode, I))
         return set_error(NB_EINVAL, "no pair kernel with %d bodies per thread for this precision",
                          I);
     pl.pl.I = I;
-    int occ = pair_occupancy(pl.pl.mode, I);
-    if (occ < 1) occ = 1;
-    if (waves > 0) bps = (waves < MAX_WAVES ? waves : MAX_WAVES) * occ;
-    pl.pl.blocks_per_sm = bps > 0 ? (bps < MAX_WAVES * occ ? bps : MAX_WAVES * occ)
-                                  : DEFAULT_WAVES * occ;
-    const int64_t want = (int64_t)P.num_sms * pl.pl.blocks_per_sm;
-    const int64_t resident = (int64_t)P.num_sms * occ;
-    if (jt == 0) {
-        // full-width j-tiles, halved while the units are too few to give
-        // every resident block one (small clusters)
-        int64_t w_full = 0;
-        for (int32_t k = 0; k < C.K; ++k)
-            w_full += ((C.nk[k] + TILE * I - 1) / (TILE * I)) * ((C.nk[k] + TILE - 1) / TILE);
-        jt = TILE;
-        while (jt > 32 && w_full * (TILE / jt) < resident) jt /= 2;
-    }
-    int rc = set_layout(C, TILE * I, st, jt);
-    if (rc) return rc;
     pl.pl.um = true;
     for (int32_t k = 0; k < C.K && pl.pl.um; ++k) pl.pl.um = C.mu[k] > 0;
-    const int64_t W = C.uoff[C.K];
-    int64_t G = want < W ? want : W;   // at least one unit per block
-    const int64_t slot_cap = part_slot_cap(P, C);
-    pl.pl.d = make_decomp(W, C.max_ntiles, TILE * I, G, slot_cap, jt);
+    int64_t rows = 0;   // partial sums needed
+    for (;;) {
+        int occ = sym ? sym_occupancy(pl.pl.mode, I) : pair_occupancy(pl.pl.mode, I);
+        if (occ < 1) occ = 1;
+        int b = bps;
+        if (waves > 0) b = (waves < MAX_WAVES ? waves : MAX_WAVES) * occ;
+        pl.pl.blocks_per_sm = b > 0 ? (b < MAX_WAVES * occ ? b : MAX_WAVES * occ)
+                                    : DEFAULT_WAVES * occ;
+        const int64_t want = (int64_t)P.num_sms * pl.pl.blocks_per_sm;
+        const int64_t resident = (int64_t)P.num_sms * occ;
+        int j = jt;
+        if (j == 0) {
+            // full-width j-tiles, halved while the units are too few to give
+            // every resident block one (small clusters)
+            j = TILE;
+            for (;;) {
+                int rc = set_units(C, TILE * I, j, sym);
+                if (rc) return rc;
+                if (j == 32 || C.uoff[C.K] >= resident) break;
+                j /= 2;
+            }
+        }
+        int rc = set_units(C, TILE * I, j, sym);
+        if (rc) return rc;
+        const int64_t W = C.uoff[C.K];
+        const int64_t G = want < W ? want : W;   // at least one unit per block
+        const int64_t full = part_elems_for(P.num_sms, C.n);
+        if (!sym) {
+            rc = set_reserve_part(C, full, st);
+            if (rc) return rc;
+            pl.pl.d = make_decomp(W, C.max_ntiles, TILE * I, G, part_slot_cap(C), j);
+            break;
+        }
+        const int64_t limit = C.part_limit / 24;
+        if (make_sym_decomp(C.nk.data(), C.K, C.uoff.data(), TILE * I, j, G, limit, true, pl.pl.d,
+                            C.poff.data(), &rows) &&
+            set_reserve_part(C, 3 * rows > full ? 3 * rows : full, st) == NB_OK)
+            break;
+        sym = false;   // the slots do not fit: the full kernels
+    }
     pl.pl.d.fpart = sp_family(pl.pl.mode) ? 1 : 0;
     // several clusters by value: launch the blocks largest-work first.  Not
     // with the near-pair pass beside the pair kernel: its kernels get SMs as
@@ -466,16 +528,21 @@ int plan_make(const Pool &P, ClusterSet &C, int precision, cudaStream_t st, Plan
     // slower); in the other modes it made the step 0.5-2.6% faster
     C.bperm_G = -1;
     if (pl.pl.mode != PM_FP64 && pl.pl.mode != PM_DS_NEAR && C.K > 1 && C.K <= PARAM_CLUSTERS &&
-        pl.pl.d.G <= PERM_CAP && !pl.pl.d.rows)
+        pl.pl.d.G <= PERM_CAP && !pl.pl.d.sym)
         block_order(C, pl.pl.d, I, sp_family(pl.pl.mode));
     for (int32_t k = 0; k < C.K; ++k)
         if (C.eps2d[k] == 0.0) pl.pl.d.mask_self = 1;
-    int occ_pot = pair_occupancy(PM_FP64, 1);
+    int occ_pot = potential_occupancy();
     if (occ_pot < 1) occ_pot = 1;
-    const int64_t Wp = C.uoff_pot[C.K];
-    int64_t Gp = (int64_t)P.num_sms * occ_pot;
-    if (Wp / 2 < Gp) Gp = Wp / 2 > 0 ? Wp / 2 : 1;
-    pl.pot = make_decomp(Wp, C.max_ntiles, TILE, Gp, slot_cap);
+    const int64_t Gp = (int64_t)P.num_sms * occ_pot;
+    // at most ceil(T G / W) + 1 <= T + 1 slots per body of a row of T units,
+    // (G / rows + 2) n in all: always within the full kernels' storage
+    int rc = NB_OK;
+    if (!make_sym_decomp(C.nk.data(), C.K, C.uoff_pot.data(), TILE * POT_I, POT_JT, Gp,
+                         C.part_elems / 3, false, pl.pot, C.poff_pot.data(), &rows))
+        rc = set_reserve_part(C, 3 * rows, st);
+    if (!rc) rc = set_layout(C, st);
+    if (rc) return rc;
     out = pl;
     return NB_OK;
 }
@@ -496,10 +563,9 @@ DevState view(const Pool &P, const ClusterSet &C, const Plan &pl)
     return s;
 }
 
-int64_t part_slot_cap(const Pool &P, const ClusterSet &C)
+int64_t part_slot_cap(const ClusterSet &C)
 {
-    const int64_t elems = C.part ? C.part_elems : P.s.part_elems;
-    const int64_t per = C.n > 0 ? elems / (3 * C.n) : MAX_PART_SLOTS;
+    const int64_t per = C.n > 0 ? C.part_elems / (3 * C.n) : MAX_PART_SLOTS;
     return per < MAX_PART_SLOTS ? per : MAX_PART_SLOTS;
 }
 
@@ -508,12 +574,10 @@ DevState view(const Pool &P, const ClusterSet &C, int precision)
     DevState s = P.s;
     s.cl = C.cl;
     s.n = C.n;
-    if (C.part) {
-        s.part = C.part;
-        s.part_elems = C.part_elems;
-    }
+    s.part = C.part;
+    s.part_elems = C.part_elems;
     s.pstride = C.n > 0 ? C.n : 1;
-    s.part_slots = part_slot_cap(P, C);
+    s.part_slots = part_slot_cap(C);
     s.diag = C.diag;
     s.red = C.red;
     s.red_len = C.scap * 16;
@@ -572,9 +636,10 @@ int enq_force(const Pool &P, const ClusterSet &C, const Plan &pl, const Phys &ph
     ht.ntiles = C.ntiles.data();
     ht.eps2f = C.eps2f.data();
     ht.mu = C.mu.data();
+    ht.poff = C.poff.data();
     const Decomp &d = pl.pl.d;
     if (C.bperm_G == d.G && C.bperm_W == d.W && C.bperm_jt == d.jt && C.bperm_ipb == d.ipb &&
-        !d.rows) {
+        !d.sym) {
         ht.perm = C.bperm.data();
         ht.nperm = (int32_t)C.bperm.size();
     }
@@ -620,7 +685,8 @@ int enq_step(const Pool &P, const ClusterSet &C, const Plan &pl, const Phys &ph,
     }
     // drift of the first leapfrog's half step (and the split it feeds, mass
     // words included: the later splits of the step rewrite coordinates only)
-    NB_TRY(launch_kick_drift(s, pl.pl.d, 0.0, 0.5 * wk[0] * h, 0, sp ? 2 : 0, ph.ext, st));
+    NB_TRY(launch_kick_drift(s, pl.pl.d, 0.0, 0.5 * wk[0] * h, 0, sp ? (pl.pl.d.sym ? 3 : 2) : 0, ph.ext,
+                             st));
     count(kernels, 1);
     for (int k = 0; k < K; ++k) {
         // adjacent half drifts of consecutive leapfrogs merge
@@ -629,7 +695,7 @@ int enq_step(const Pool &P, const ClusterSet &C, const Plan &pl, const Phys &ph,
         cudaEvent_t e0 = evs ? (*evs)[2 * k] : nullptr, e1 = evs ? (*evs)[2 * k + 1] : nullptr;
         int rc = enq_force(P, C, pl, ph, st, e0, e1, kernels);
         if (rc) return rc;
-        NB_TRY(launch_kick_drift(s, pl.pl.d, wk[k] * h, hd, 1, (sp && !last) ? 1 : 0, ph.ext,
+        NB_TRY(launch_kick_drift(s, pl.pl.d, wk[k] * h, hd, 1, (sp && !last) ? (pl.pl.d.sym ? 3 : 1) : 0, ph.ext,
                                  st));
         count(kernels, 1);
     }
@@ -650,7 +716,14 @@ int enq_energy(const Pool &P, const ClusterSet &C, const Plan &pl, const Phys &p
 {
     DevState s = view(P, C, pl);
     s.cl = C.cl_pot;
-    NB_TRY(launch_potential(s, pl.pot, st));
+    HostTab ht;
+    ht.K = C.K;
+    ht.uoff = C.uoff_pot.data();
+    ht.boff = C.boff.data();
+    ht.nk = C.nk.data();
+    ht.eps2f = C.eps2f.data();
+    ht.poff = C.poff_pot.data();
+    NB_TRY(launch_potential(s, pl.pot, ht, st));
     NB_TRY(launch_energy_reduce(s, pl.pot, ph.ext, ph.G, st));
     count(kernels, 3);
     return NB_OK;

@@ -36,14 +36,17 @@ struct Pool {
     DevState s;
     double *stage = nullptr;   // (7 cap) staging for interleaved host transfers
 };
-// own_part: allocate the partial-sum storage of a single cluster set (a
-// context); a pool shared by concurrent sets (the serving loop's groups)
-// leaves it out, and each set reserves its own (set_reserve_part).
-int pool_create(Pool &P, int device, int64_t cap, bool own_part = true);
-// Partial-sum doubles a set of n bodies may need: 3 min(giw + 2 n,
-// MAX_PART_SLOTS n), giw the widest grid's i-rows (SMs x MAX_WAVES x 3072).
-int64_t part_elems_for(const Pool &P, int64_t n);
+int pool_create(Pool &P, int device, int64_t cap);
+// Partial-sum doubles the full decomposition of a set of n bodies may need:
+// 3 min(giw + 2 n, MAX_PART_SLOTS n), giw the widest grid's i-rows (SMs x
+// MAX_WAVES x 3072).
+int64_t part_elems_for(int sms, int64_t n);
 void pool_destroy(Pool &P);
+
+// Bytes of partial sums a context's set may take for the symmetric kernels
+// (their slots grow as n^2 / i-block width: 0.9 GB at n = 262144 with
+// i-blocks of 1024 bodies); larger sets take the full kernels.
+constexpr int64_t SYM_PART_LIMIT = (int64_t)4 << 30;
 
 // Tables of one cluster set in a pool (host copy + device copy).
 struct ClusterSet {
@@ -52,7 +55,7 @@ struct ClusterSet {
     int64_t n = 0;             // bodies, noff[K]
     int64_t max_ntiles = 0;
     int ipb = 0;               // i-block width the pair units are counted with
-    std::vector<int64_t> boff, nk, noff, uoff, uoff_pot, seg_lo, seg_hi;
+    std::vector<int64_t> boff, nk, noff, uoff, uoff_pot, poff, poff_pot, seg_lo, seg_hi;
     std::vector<int32_t> ntiles, seg_k, seg_off;
     std::vector<float> eps2f;
     std::vector<double> eps, eps2d, dts;
@@ -75,10 +78,13 @@ struct ClusterSet {
     // pair kernel (it reads only the float planes, and writes only corr)
     cudaStream_t side = nullptr;
     cudaEvent_t fork = nullptr, join = nullptr;
-    // the set's own partial-sum storage (NULL: the pool's); sets that run
-    // concurrently in one pool must each have their own
+    // the set's partial-sum storage (sets that run concurrently in one pool
+    // must each have their own), reserved when a plan needs more than it has,
+    // and the bytes the symmetric decomposition's slots may take of it
     double *part = nullptr;
     int64_t part_elems = 0;
+    int64_t part_limit = SYM_PART_LIMIT;
+    bool part_ordered = false;   // stream-ordered allocation (sets beside running ones)
     // launch order of the pair kernel's blocks for the decomposition of the
     // last plan made (grid bperm_G over bperm_W units of width bperm_jt,
     // i-blocks of bperm_ipb bodies; bperm_G = -1: none)
@@ -94,9 +100,9 @@ int set_create(ClusterSet &C, int32_t kcap, int64_t body_cap, int priority = 0);
 // largest estimated work first.  I: bodies per thread; partial: the kernel
 // evaluates only the packed i-pairs that hold bodies.
 void block_order(ClusterSet &C, const Decomp &d, int I, bool partial);
-// Give the set its own partial-sum storage of at least elems doubles, grown
-// (stream-ordered allocation on st) when smaller; none of the set's work may
-// be in flight.
+// Give the set partial-sum storage of at least elems doubles, grown when
+// smaller (part_ordered: by stream-ordered allocation on st); none of the
+// set's work may be in flight.
 int set_reserve_part(ClusterSet &C, int64_t elems, cudaStream_t st);
 void set_destroy(ClusterSet &C);
 // Clusters k = 0..K-1 at pool slots [boff[k], boff[k] + nk[k]), softening
@@ -104,9 +110,10 @@ void set_destroy(ClusterSet &C);
 int set_define(ClusterSet &C, int32_t K, const int64_t *boff, const int64_t *nk,
                const double *eps, const double *dts);
 // Count pair units for i-blocks of ipb bodies and j-ranges of jt bodies (a
-// divisor of TILE), build reduction segments and upload every table
-// (stream-ordered).
-int set_layout(ClusterSet &C, int ipb, cudaStream_t st, int jt = TILE);
+// divisor of TILE) of the full or the symmetric decomposition (host only).
+int set_units(ClusterSet &C, int ipb, int jt, bool sym);
+// Build reduction segments and upload every table (stream-ordered).
+int set_layout(ClusterSet &C, cudaStream_t st);
 
 struct Plan {
     int precision = -1;
@@ -125,6 +132,7 @@ struct Plan {
 // stay fixed by its index (results stay bit-reproducible).
 constexpr int MAX_WAVES = 6;
 constexpr int DEFAULT_WAVES = 4;
+constexpr int POT_JT = TILE;   // j bodies per unit of the potential kernel
 struct PairShape {
     int I = 0;
     int blocks_per_sm = 0;
@@ -184,9 +192,8 @@ DevState view(const Pool &P, const ClusterSet &C, const Plan &pl);
 // of at most DS_FULL_MAX_PAIRS pairs forms the double-single difference on
 // every pair (no near-pair pass).
 int plan_mode(const ClusterSet &C, int precision);
-// Partial slots per body the set has in its storage (its own, else the
-// pool's) for its current bodies.
-int64_t part_slot_cap(const Pool &P, const ClusterSet &C);
+// Partial slots per body the set has in its storage for its current bodies.
+int64_t part_slot_cap(const ClusterSet &C);
 int mode_of(int precision);
 bool float_planes(int precision);
 

@@ -354,7 +354,8 @@ cudaError_t launch_frame(const DevState &s, double near_frac, bool near, cudaStr
 // MASS: also write the mass words of the j-stream copies (m and its float
 // rounding residue); the kick's per-substep splits leave them as the step's
 // first split wrote them (masses never change).
-template <bool MASS>
+// JS: write the j-stream copies (the symmetric kernels read the planes).
+template <bool MASS, bool JS = true>
 __device__ __forceinline__ void split_one(const DevState &s, const Frame &f, int64_t i,
                                           double x, double y, double z)
 {
@@ -368,6 +369,7 @@ __device__ __forceinline__ void split_one(const DevState &s, const Frame &f, int
     s.xl[i] = lx;
     s.yl[i] = ly;
     s.zl[i] = lz;
+    if (!JS) return;
     s.jd[2 * i] = make_float4(hx, hx, hy, hy);
     s.jl[2 * i] = make_float4(lx, lx, ly, ly);
     if (MASS) {
@@ -420,10 +422,11 @@ __device__ __forceinline__ void ff_add(float &h, float &l, float p, float e)
 // their bits (the conversion instruction runs on the FP64 pipe, 1/77 of the
 // FP32 rate here).
 template <int SB>
-__device__ __forceinline__ void sum_slots_ff(const DevState &s, int64_t count, int64_t t,
+__device__ __forceinline__ void sum_slots_ff(const DevState &s, const SlotRun &run,
                                              double &ax, double &ay, double &az)
 {
-    const float2 *part2 = reinterpret_cast<const float2 *>(s.part);
+    const int64_t count = run.count, ps = run.stride;
+    const float2 *part2 = reinterpret_cast<const float2 *>(s.part) + run.base;
     float hx = 0.f, lx = 0.f, hy = 0.f, ly = 0.f, hz = 0.f, lz = 0.f;
     for (int64_t k0 = 0; k0 < count; k0 += SB) {
         float2 bx[SB], by[SB], bz[SB];
@@ -431,10 +434,10 @@ __device__ __forceinline__ void sum_slots_ff(const DevState &s, int64_t count, i
         for (int q = 0; q < SB; ++q) {
             bx[q] = by[q] = bz[q] = make_float2(0.f, 0.f);
             if (k0 + q < count) {
-                const float2 *p = part2 + ((k0 + q) * 3) * s.pstride + t;
+                const float2 *p = part2 + ((k0 + q) * 3) * ps;
                 bx[q] = p[0];
-                by[q] = p[s.pstride];
-                bz[q] = p[2 * s.pstride];
+                by[q] = p[ps];
+                bz[q] = p[2 * ps];
             }
         }
 #pragma unroll
@@ -454,11 +457,10 @@ template <int SB, bool FP>
 __device__ __forceinline__ void sum_slots(const DevState &s, const Decomp &d, const BodyRef &r,
                                           int64_t t, double &ax, double &ay, double &az)
 {
-    int64_t first, count;
-    iblock_slots(d, s.cl, r.k, r.li, first, count);
-    (void)first;
+    const SlotRun run = slot_run(d, s.cl, r.k, r.li, t, s.pstride);
+    const int64_t count = run.count, ps = run.stride;
     if (FP) {
-        sum_slots_ff<SB>(s, count, t, ax, ay, az);
+        sum_slots_ff<SB>(s, run, ax, ay, az);
         if (s.corr) {
             ax += s.corr[r.gi];
             ay += s.corr[s.cap + r.gi];
@@ -474,10 +476,10 @@ __device__ __forceinline__ void sum_slots(const DevState &s, const Decomp &d, co
         for (int q = 0; q < SB; ++q) {
             bx[q] = by[q] = bz[q] = 0.0;
             if (k0 + q < count) {
-                const double *p = s.part + ((k0 + q) * 3) * s.pstride + t;
+                const double *p = s.part + run.base + ((k0 + q) * 3) * ps;
                 bx[q] = p[0];
-                by[q] = p[s.pstride];
-                bz[q] = p[2 * s.pstride];
+                by[q] = p[ps];
+                bz[q] = p[2 * ps];
             }
         }
 #pragma unroll
@@ -533,7 +535,9 @@ __global__ void kick_drift_kernel(DevState s, Decomp d, double wk, double wd, in
     s.x[i] = x;
     s.y[i] = y;
     s.z[i] = z;
-    if (do_split == 2)
+    if (do_split == 3)
+        split_one<false, false>(s, s.cl.frame[r.k], i, x, y, z);
+    else if (do_split == 2)
         split_one<true>(s, s.cl.frame[r.k], i, x, y, z);
     else if (do_split)
         split_one<false>(s, s.cl.frame[r.k], i, x, y, z);
@@ -618,7 +622,7 @@ cudaError_t launch_accel_out_range(const DevState &s, const Decomp &d, const Ext
 // ---- diagnostics -------------------------------------------------------------
 
 // Per segment: K, sum m_i phi_i, W_ext, P, L, non-finite count (10 values).
-// d is the potential kernel's decomposition (s.cl.uoff must be its units).
+// d is the potential kernel's decomposition (s.cl.uoff and poff must be its).
 __global__ void energy_partial_kernel(DevState s, Decomp d, ExtField ext)
 {
     __shared__ double sh[10 * RT];
@@ -633,14 +637,14 @@ __global__ void energy_partial_kernel(DevState s, Decomp d, ExtField ext)
         const int64_t i = r.gi;
         const double m = s.m[i], x = s.x[i], y = s.y[i], z = s.z[i];
         const double vx = s.vx[i], vy = s.vy[i], vz = s.vz[i];
-        int64_t first, count;
-        iblock_slots(d, s.cl, k, r.li, first, count);
+        const SlotRun run = slot_run(d, s.cl, k, r.li, t, s.pstride);
+        const int64_t count = run.count;
         double phi = 0.0;
         for (int64_t q0 = 0; q0 < count; q0 += 8) {
             double bp[8];
 #pragma unroll
             for (int q = 0; q < 8; ++q)
-                bp[q] = q0 + q < count ? s.part[((q0 + q) * 3) * s.pstride + t] : 0.0;
+                bp[q] = q0 + q < count ? s.part[run.base + ((q0 + q) * 3) * run.stride] : 0.0;
 #pragma unroll
             for (int q = 0; q < 8; ++q)
                 if (q0 + q < count) phi += bp[q];
@@ -670,7 +674,7 @@ __global__ void energy_final_kernel(DevState s, double G)
     cluster_sum<10>(s, v, sh);
     if (threadIdx.x == 0) {
         double *o = s.diag + (int64_t)blockIdx.x * DIAG_STRIDE;
-        const double W = -0.5 * G * v[1];
+        const double W = -G * v[1];   // each unordered pair once
         o[0] = v[0];
         o[1] = W;
         o[2] = v[2];

@@ -50,6 +50,8 @@ struct Clusters {
     const int32_t *cid = nullptr;    // [noff[K]] cluster of each linear body (K > 1)
     const double *mu = nullptr;      // [K]   the common mass of cluster k's bodies, 0 if
                                      //       they differ
+    const int64_t *poff = nullptr;   // [K]   first partial-sum row of cluster k (the
+                                     //       symmetric decomposition's slots)
 };
 
 // Cluster of linear body t: one load from the precomputed map (K = 1: 0).
@@ -115,6 +117,42 @@ struct DevState {
     int *flag = nullptr;        // non-finite flag
 };
 
+// Rows and tiles of the symmetric decomposition of one cluster of n bodies cut
+// into nb i-blocks of ipb bodies.  Each unordered pair of i-blocks is one
+// tile: row b holds the tiles (b, b + delta mod nb), delta = 0 (the block with
+// itself) up to nb / 2, the last only in the first half of the rows when nb is
+// even (both of its blocks would hold it otherwise).  So rows are equally
+// long within one tile, unlike the triangle's, and a run of units stays in
+// few rows.
+struct SymRows {
+    int32_t nb, half, D, split;   // rows [0, split) have D tiles, the others D - 1
+    __host__ __device__ SymRows(int64_t n, int32_t ipb)
+    {
+        nb = (int32_t)((n + ipb - 1) / ipb);
+        half = nb / 2;
+        D = half + 1;
+        split = (nb & 1) ? nb : half;
+    }
+    __host__ __device__ int32_t row_tiles(int32_t b) const { return b < split ? D : D - 1; }
+    // tiles before row b
+    __host__ __device__ int64_t row_first(int32_t b) const
+    {
+        return (int64_t)b * D - (b > split ? b - split : 0);
+    }
+    __host__ __device__ int64_t tiles() const { return row_first(nb); }
+    // row of tile q
+    __host__ __device__ int32_t row_of(int64_t q) const
+    {
+        const int64_t q1 = (int64_t)split * D;
+        return q < q1 ? (int32_t)(q / D) : split + (int32_t)((q - q1) / (D - 1));
+    }
+    // tiles whose j side is block c (one j slot per delta): 0, 1, ...
+    __host__ __device__ int32_t jslots(int32_t c) const
+    {
+        return (!(nb & 1) && c < half) ? half : half + 1;
+    }
+};
+
 // Stream-K-style decomposition of the pair work of a cluster set.  A unit is
 // (cluster k, i-block b, j-range t of jt bodies); units are numbered cluster
 // by cluster, u = uoff[k] + b * units_per_iblock(ntiles[k]) + t, W units in
@@ -146,6 +184,15 @@ struct Decomp {
     // in float-float arithmetic on the FP32 pipes; 0: doubles (FP64 and
     // float-float kernels, potential sums)
     int32_t fpart = 0;
+
+    // symmetric (each unordered pair once, its force added to both bodies): a
+    // unit is jt j bodies of one tile of SymRows; the sums of a unit's j bodies
+    // go to slot delta of those bodies (jsum = 1; the potential sums have
+    // none), the sums of a row's i bodies to the slots after their j slots, one
+    // per block of the row.  Cluster k's slots of n_k rows each start at row
+    // poff[k] of the storage, [slot][3][n_k].
+    int32_t sym = 0;
+    int32_t jsum = 0;
 
     // 1 when (W + 1) (G + 1) < 2^32: U and owner then divide in 32 bits (a
     // 64-bit division costs tens of instructions, on the kick's hot path)
@@ -179,6 +226,35 @@ __device__ __forceinline__ void iblock_slots(const Decomp &d, const Clusters &c,
     const int64_t u0 = c.uoff[k] + b * nt;
     first = d.owner(u0);
     count = d.owner(u0 + nt - 1) - first + 1;
+}
+
+// Partial sums of linear body t (local index li of cluster k): row of its
+// first slot, distance between slots, component stride and slot count.
+struct SlotRun {
+    int64_t base, stride, count;
+};
+__device__ __forceinline__ SlotRun slot_run(const Decomp &d, const Clusters &c, int32_t k,
+                                            int64_t li, int64_t t, int64_t pstride)
+{
+    SlotRun r;
+    if (!d.sym) {
+        int64_t first;
+        iblock_slots(d, c, k, li, first, r.count);
+        r.base = t;
+        r.stride = pstride;
+        return r;
+    }
+    const int64_t n = c.nk[k];
+    const SymRows sr(n, d.ipb);
+    const int32_t b = (int32_t)(li >> (__ffs(d.ipb) - 1));
+    const int32_t upt = d.ipb / d.jt;
+    const int64_t u0 = c.uoff[k] + sr.row_first(b) * upt;
+    const int64_t first = d.owner(u0);
+    r.count = d.owner(u0 + (int64_t)sr.row_tiles(b) * upt - 1) - first + 1;
+    if (d.jsum) r.count += sr.jslots(b);
+    r.base = 3 * c.poff[k] + li;
+    r.stride = n;
+    return r;
 }
 
 struct ExtField {
@@ -225,6 +301,7 @@ struct HostTab {
     const int32_t *ntiles = nullptr;
     const float *eps2f = nullptr;
     const double *mu = nullptr;
+    const int64_t *poff = nullptr;   // first partial-sum row of each cluster (symmetric)
     // launch order of the blocks (NULL: their index order): launch position
     // q runs block perm[q] of the decomposition, nperm = its grid
     const uint16_t *perm = nullptr;
@@ -242,15 +319,34 @@ constexpr int64_t MAX_PART_SLOTS = 128;
 // Resident blocks per SM of a pair-kernel variant (occupancy query).
 int pair_occupancy(int mode, int I);
 bool pair_variant_exists(int mode, int I);
+// The same of the symmetric kernels (pairsym.cu); 0: no such variant.
+int sym_occupancy(int mode, int I);
+int potential_occupancy();
+cudaError_t launch_pair_sym(const DevState &s, const PairLaunch &pl, const HostTab &ht, double G,
+                            cudaStream_t st);
+// Bodies per thread of the potential kernel (i-blocks of TILE * POT_I).
+constexpr int POT_I = 2;
+// Symmetric decomposition of clusters of nk bodies, whose units are counted in
+// uoff (sym_units), G blocks wanted, fewer when the partial sums would take
+// more than `limit` rows.  Fills poff (first row of each cluster) and *rows
+// (rows needed); false when the slots of the quarter of G take more.
+bool make_sym_decomp(const int64_t *nk, int32_t K, const int64_t *uoff, int ipb, int jt,
+                     int64_t G, int64_t limit, bool jsum, Decomp &d, int64_t *poff,
+                     int64_t *rows);
+// Units of each cluster, as prefix sums uoff[K + 1].
+void sym_units(const int64_t *nk, int32_t K, int ipb, int jt, int64_t *uoff);
 // Decomposition of the pair work of clusters with host-side sizes nk and
 // tiles, given units per cluster (host arrays), i-block width, target grid.
 Decomp make_decomp(int64_t W, int64_t max_ntiles, int ipb, int64_t G, int64_t slot_cap,
                    int jt = TILE, int rows = 0);
 cudaError_t launch_pair(const DevState &s, const PairLaunch &pl, const HostTab &ht, double G,
                         cudaStream_t st);
-// Potential sums phi_i = sum_{j != i} m_j / sqrt(r^2 + eps^2) (FP64) into
-// slot planes of s.part (component 0); decomposition with ipb = TILE.
-cudaError_t launch_potential(const DevState &s, const Decomp &d, cudaStream_t st);
+// Softened potential sums m_j / sqrt(r^2 + eps^2) (FP64), each unordered pair
+// once, on the side of one of its bodies (half on each inside a warp's row):
+// sum_i m_i phi_i is the sum over unordered pairs.  Into the slots of the
+// symmetric decomposition d with i-blocks of TILE * POT_I, component 0.
+cudaError_t launch_potential(const DevState &s, const Decomp &d, const HostTab &ht,
+                             cudaStream_t st);
 
 // ---- near-pair correction (near.cu) ----------------------------------------
 // Cell-table slots used for n bodies (four per body of every cluster).
@@ -280,7 +376,9 @@ cudaError_t launch_split(const DevState &s, cudaStream_t st);
 // One fused substep: optional kick v += wk dt_k (a_int + a_ext) from the
 // partial slots of decomposition d, then drift x += wd dt_k v, then refresh
 // the float planes: do_split 0 no, 1 coordinates only, 2 coordinates and the
-// j-stream mass words (needed once after any load; masses never change).
+// j-stream mass words (needed once after any load; masses never change),
+// 3 coordinates without the j-stream copies (the symmetric kernels, which
+// read the planes).
 cudaError_t launch_kick_drift(const DevState &s, const Decomp &d, double wk, double wd,
                               int do_kick, int do_split, const ExtField &ext, cudaStream_t st);
 // The same for linear bodies [t0, t1) only.

@@ -315,8 +315,8 @@ __global__ void __launch_bounds__(NC_T) near_correct_kernel(DevState s, double G
             if (ee[b] == (int)e0 || !(r2 < th2)) continue;
             const float4 Lj = s.ng_slo[ee[b]];
             const float ri = near_rsqrt(r2);
-            const float sf = UM ? __fmul_rn(ri, __fmul_rn(ri, ri))
-                                : __fmul_rn(__fmul_rn(mj, ri), __fmul_rn(ri, ri));
+            float sf = __fmul_rn(ri, __fmul_rn(ri, ri));
+            if (!UM) sf = __fmul_rn(mj, sf);
             // the same pair with the double-single coordinate difference
             const float ex = __fadd_rn(ddx, __fsub_rn(Lj.x, lxi));
             const float ey = __fadd_rn(ddy, __fsub_rn(Lj.y, lyi));
@@ -325,8 +325,8 @@ __global__ void __launch_bounds__(NC_T) near_correct_kernel(DevState s, double G
             e2 = __fmaf_rn(ey, ey, e2);
             e2 = __fmaf_rn(ez, ez, e2);
             const float re = near_rsqrt(e2);
-            const float se = UM ? __fmul_rn(re, __fmul_rn(re, re))
-                                : __fmul_rn(__fmul_rn(mj, re), __fmul_rn(re, re));
+            float se = __fmul_rn(re, __fmul_rn(re, re));
+            if (!UM) se = __fmul_rn(mj, se);
             ax += (double)__fmul_rn(ex, se) - (double)__fmul_rn(ddx, sf);
             ay += (double)__fmul_rn(ey, se) - (double)__fmul_rn(ddy, sf);
             az += (double)__fmul_rn(ez, se) - (double)__fmul_rn(ddz, sf);

@@ -33,6 +33,7 @@
 // loop's float contribution bit for bit.
 #include <cstring>
 
+#include "arith.cuh"
 #include "nb_internal.cuh"
 #include "split.cuh"
 
@@ -58,26 +59,6 @@ Decomp make_decomp(int64_t W, int64_t max_ntiles, int ipb, int64_t G, int64_t sl
     }
     d.narrow = (double)(d.W + 1) * (double)(d.G + 1) < 4294967296.0 ? 1 : 0;
     return d;
-}
-
-__device__ __forceinline__ float rsqrt_mufu(float x)
-{
-    float y;
-    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
-
-// Add float t to the double-single number (hi, lo): Knuth's two-sum of hi and
-// t, error folded into lo, then Dekker's fast two-sum to renormalise.
-__device__ __forceinline__ void ds_add(float &hi, float &lo, float t)
-{
-    const float s = __fadd_rn(hi, t);
-    const float bp = __fsub_rn(s, hi);
-    const float e = __fadd_rn(__fsub_rn(hi, __fsub_rn(s, bp)), __fsub_rn(t, bp));
-    const float l = __fadd_rn(lo, e);
-    const float h = __fadd_rn(s, l);
-    lo = __fsub_rn(l, __fsub_rn(h, s));
-    hi = h;
 }
 
 // One contiguous run of units of block g inside one cluster's i-block.
@@ -119,18 +100,6 @@ __device__ __forceinline__ int64_t block_of(const ParamTab<KC> &t)
 {
     if (KC >= PARAM_CLUSTERS && t.nperm > 0) return t.perm[blockIdx.x];
     return blockIdx.x;
-}
-
-// largest k in [0, K) with off[k] <= t
-template <typename T>
-__device__ __forceinline__ int32_t find_in(const T *off, int32_t K, int64_t t)
-{
-    int32_t lo = 0, hi = K;
-    while (hi - lo > 1) {
-        const int32_t mid = (lo + hi) >> 1;
-        if (off[mid] <= t) lo = mid; else hi = mid;
-    }
-    return lo;
 }
 
 // End of a unit's j range, clipped to the cluster's bodies rounded up to 32
@@ -251,8 +220,8 @@ __device__ __forceinline__ void chunk_pass(const float4 (*cb)[4], int j0, int ib
                 r2 = __ffma2_rn(dy, dy, r2);
                 r2 = __ffma2_rn(dz, dz, r2);
                 const float2 ri = make_float2(rsqrt_mufu(r2.x), rsqrt_mufu(r2.y));
-                float2 s = UM ? __fmul2_rn(ri, __fmul2_rn(ri, ri))
-                              : __fmul2_rn(__fmul2_rn(mm, ri), __fmul2_rn(ri, ri));
+                float2 s = __fmul2_rn(ri, __fmul2_rn(ri, ri));
+                if (!UM) s = __fmul2_rn(mm, s);
                 if (MASK) {
                     const int j = j0 + jj;
                     if (j == ibase + 2 * p * TILE) s.x = 0.f;
@@ -464,64 +433,6 @@ __global__ void __launch_bounds__(TILE, sp_min_blocks(P, MODE)) pair_sp_kernel(
 // costs more issue slots than it saves).  UM (all masses of the cluster
 // equal): 1 / r^3 without m, the caller scales by m.
 
-__device__ __forceinline__ float2 f2neg(float2 a) { return make_float2(-a.x, -a.y); }
-__device__ __forceinline__ float2 f2sub(float2 a, float2 b) { return __fadd2_rn(a, f2neg(b)); }
-
-// s + e = a + b exactly (Knuth).
-__device__ __forceinline__ void two_sum2(float2 a, float2 b, float2 &s, float2 &e)
-{
-    s = __fadd2_rn(a, b);
-    const float2 bb = f2sub(s, a);
-    e = __fadd2_rn(f2sub(a, f2sub(s, bb)), f2sub(b, bb));
-}
-
-// s + e = a + b exactly when |a| >= |b| (Dekker).
-__device__ __forceinline__ void fast_two_sum2(float2 a, float2 b, float2 &s, float2 &e)
-{
-    s = __fadd2_rn(a, b);
-    e = f2sub(b, f2sub(s, a));
-}
-
-// s + e = a + b exactly for a, b >= 0: the larger operand first (max / min
-// run on the ALU pipe, which this kernel leaves idle), then Dekker's fast
-// two-sum, three FMA-pipe operations instead of Knuth's six.
-__device__ __forceinline__ void pos_two_sum2(float2 a, float2 b, float2 &s, float2 &e)
-{
-    const float2 hi = make_float2(fmaxf(a.x, b.x), fmaxf(a.y, b.y));
-    const float2 lo = make_float2(fminf(a.x, b.x), fminf(a.y, b.y));
-    s = __fadd2_rn(a, b);
-    e = f2sub(lo, f2sub(s, hi));
-}
-
-// (ah + al) - (bh + bl), normalised.
-__device__ __forceinline__ void ff_diff(float2 ah, float2 al, float2 bh, float2 bl, float2 &dh,
-                                        float2 &dl)
-{
-    float2 s, e;
-    two_sum2(ah, f2neg(bh), s, e);
-    e = __fadd2_rn(e, f2sub(al, bl));
-    fast_two_sum2(s, e, dh, dl);
-}
-
-// h^2 + (2 h l) as an unnormalised pair (p, e): p = fl(h^2), e its error plus
-// the cross term.
-__device__ __forceinline__ void ff_sq(float2 h, float2 l, float2 &p, float2 &e)
-{
-    p = __fmul2_rn(h, h);
-    e = __ffma2_rn(h, h, f2neg(p));
-    e = __ffma2_rn(__fadd2_rn(h, h), l, e);
-}
-
-// (ah + al)(bh + bl) without the al bl term, unnormalised.
-__device__ __forceinline__ void ff_mul(float2 ah, float2 al, float2 bh, float2 bl, float2 &p,
-                                       float2 &e)
-{
-    p = __fmul2_rn(ah, bh);
-    e = __ffma2_rn(ah, bh, f2neg(p));
-    e = __ffma2_rn(ah, bl, e);
-    e = __ffma2_rn(al, bh, e);
-}
-
 template <int P>
 struct FFI {
     float2 xh[P], yh[P], zh[P], xl[P], yl[P], zl[P];         // i coordinates
@@ -714,11 +625,9 @@ __global__ void __launch_bounds__(TILE) pair_ff_kernel(
 // Double-precision pair kernel: the plain FP64 baseline (Sect. 4.2's DP mode
 // with structures of four doubles).  The block's j-range is staged through
 // shared memory up to TILE bodies at a time and broadcast to the threads'
-// i bodies.  With POT it sums the softened potential m_j / sqrt(r^2 + eps^2)
-// of eq. 4 instead (j = i always excluded), for the energy diagnostic.  UM
-// (all masses of the cluster equal): the pair term is d / r^3 without m_j,
+// i bodies.  UM (all masses of the cluster equal): the pair term is d / r^3 without m_j,
 // one multiply fewer on the FP64 pipe; the sums are scaled by G m.
-template <int I, bool POT, bool UM = false>
+template <int I, bool UM>
 __global__ void __launch_bounds__(TILE) pair_fp64_kernel(
     const double *__restrict__ x, const double *__restrict__ y, const double *__restrict__ z,
     const double *__restrict__ m, Clusters c, Decomp d, double G, double *__restrict__ part,
@@ -735,7 +644,7 @@ __global__ void __launch_bounds__(TILE) pair_fp64_kernel(
         const int n = sg.nk;
         const int64_t base = sg.base;
         const double eps2 = c.eps2d[sg.k];
-        const bool mask_self = POT || d.mask_self != 0;
+        const bool mask_self = d.mask_self != 0;
         const int ib0 = sg.b * d.ipb;
         int idx[I];
         double xi[I], yi[I], zi[I], ax[I], ay[I], az[I];
@@ -776,17 +685,11 @@ __global__ void __launch_bounds__(TILE) pair_fp64_kernel(
                     double r2 = fma(dx, dx, eps2);
                     r2 = fma(dy, dy, r2);
                     r2 = fma(dz, dz, r2);
-                    if (POT) {
-                        double wgt = mj * rsqrt_pow<true>(r2);
-                        if (diag && jglob + jj == idx[k]) wgt = 0.0;
-                        ax[k] += wgt;
-                    } else {
-                        double s = UM ? rsqrt_pow<false>(r2) : mj * rsqrt_pow<false>(r2);
-                        if (diag && jglob + jj == idx[k]) s = 0.0;
-                        ax[k] = fma(dx, s, ax[k]);
-                        ay[k] = fma(dy, s, ay[k]);
-                        az[k] = fma(dz, s, az[k]);
-                    }
+                    double s = UM ? rsqrt_pow<false>(r2) : mj * rsqrt_pow<false>(r2);
+                    if (diag && jglob + jj == idx[k]) s = 0.0;
+                    ax[k] = fma(dx, s, ax[k]);
+                    ay[k] = fma(dy, s, ay[k]);
+                    az[k] = fma(dz, s, az[k]);
                 }
             }
         }
@@ -796,13 +699,9 @@ __global__ void __launch_bounds__(TILE) pair_fp64_kernel(
             const int i = idx[k];
             if (i < n) {
                 double *p = part + (sg.slot * 3) * ps + sg.lbase + i;
-                if (POT) {
-                    p[0] = ax[k];
-                } else {
-                    p[0] = Gm * ax[k];
-                    p[ps] = Gm * ay[k];
-                    p[2 * ps] = Gm * az[k];
-                }
+                p[0] = Gm * ax[k];
+                p[ps] = Gm * ay[k];
+                p[2 * ps] = Gm * az[k];
             }
         }
         u += sg.t1 - sg.t0;
@@ -872,8 +771,8 @@ static cudaError_t launch_sp(const DevState &s, const PairLaunch &pl, const Host
 
 static dp_kernel_t dp_variant(int I, bool um = false)
 {
-    if (I == 1) return um ? pair_fp64_kernel<1, false, true> : pair_fp64_kernel<1, false>;
-    if (I == 2) return um ? pair_fp64_kernel<2, false, true> : pair_fp64_kernel<2, false>;
+    if (I == 1) return um ? pair_fp64_kernel<1, true> : pair_fp64_kernel<1, false>;
+    if (I == 2) return um ? pair_fp64_kernel<2, true> : pair_fp64_kernel<2, false>;
     return nullptr;
 }
 
@@ -908,6 +807,7 @@ int pair_occupancy(int mode, int I)
 cudaError_t launch_pair(const DevState &s, const PairLaunch &pl, const HostTab &ht, double G,
                         cudaStream_t st)
 {
+    if (pl.d.sym) return launch_pair_sym(s, pl, ht, G, st);
     if (pl.mode == PM_FP64) {
         dp_kernel_t k = dp_variant(pl.I, pl.um);
         if (!k) return cudaErrorInvalidValue;
@@ -920,13 +820,6 @@ cudaError_t launch_pair(const DevState &s, const PairLaunch &pl, const HostTab &
     case PARAM_CLUSTERS: return launch_sp<PARAM_CLUSTERS>(s, pl, ht, G, st);
     default: return launch_sp<0>(s, pl, ht, G, st);
     }
-}
-
-cudaError_t launch_potential(const DevState &s, const Decomp &d, cudaStream_t st)
-{
-    pair_fp64_kernel<1, true><<<(unsigned)d.G, TILE, 0, st>>>(s.x, s.y, s.z, s.m, s.cl, d, 1.0,
-                                                               s.part, s.pstride);
-    return cudaGetLastError();
 }
 
 }  // namespace nb

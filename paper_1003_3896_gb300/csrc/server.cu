@@ -90,6 +90,10 @@ constexpr size_t PAIR_IV_CAP = (size_t)1 << 20;
 constexpr int64_t SMALL_JOB = 16384;
 constexpr int NGROUPS = 12;               // (FP64, NB_DS, NB_DD) x (order 2, 6) x (small, large)
 
+// A group's partial sums for the symmetric kernels: a 32nd of the budget, or
+// this many bytes (the full kernels' fixed part) where that is more.
+constexpr double GROUP_PART_LEAST = 67.0e6;
+
 // Bytes of device memory the pool and the group scratch use per body slot:
 // state, float planes, j-stream, near-pair correction, staging, near-pair
 // scratch; plus the groups' partial sums, 2 x 24 bytes per body of a group
@@ -148,7 +152,8 @@ int upload(nb_server *s, Job &j)
     const int64_t nk = n;
     const double e = j.d.eps, one = 1.0;
     int rc = set_define(s->io, 1, &off, &nk, &e, &one);
-    if (!rc) rc = set_layout(s->io, TILE, s->io_stream);
+    if (!rc) rc = set_units(s->io, TILE, TILE, false);
+    if (!rc) rc = set_layout(s->io, s->io_stream);
     if (rc) return rc;
     double *sp = s->pool.stage + 7 * off, *sv = sp + 3 * n, *sm = sp + 6 * n;
     NB_TRY(cudaMemcpyAsync(sp, j.pos.data(), 3 * n * 8, cudaMemcpyHostToDevice, s->io_stream));
@@ -165,7 +170,8 @@ int download(nb_server *s, Job &j)
     const int64_t off = j.off, nk = n;
     const double e = j.d.eps, one = 1.0;
     int rc = set_define(s->io, 1, &off, &nk, &e, &one);
-    if (!rc) rc = set_layout(s->io, TILE, s->io_stream);
+    if (!rc) rc = set_units(s->io, TILE, TILE, false);
+    if (!rc) rc = set_layout(s->io, s->io_stream);
     if (rc) return rc;
     double *sp = s->pool.stage + 7 * off, *sv = sp + 3 * n;
     NB_TRY(launch_pack(view(s->pool, s->io, NB_FP64), sp, sv, s->io_stream));
@@ -315,7 +321,6 @@ int launch_step(nb_server *s, Group &g)
                             dts.data());
         g.set.mu = mu;
         // the group's own partial sums: groups step concurrently
-        if (!rc) rc = set_reserve_part(g.set, part_elems_for(s->pool, g.set.n), g.stream);
         // the large jobs' groups: the most waves, so their blocks are short
         // and free SM slots for the small jobs' kernels sooner
         const bool large = ((&g - s->groups) & 1) != 0;
@@ -454,7 +459,7 @@ int nb_server_create(const nb_server_params *p, nb_server **out)
         return set_error(NB_EINVAL, "HBM budget too small for one body");
     }
     s->cap = cap;
-    int rc = pool_create(s->pool, p->device, cap, /*own_part=*/false);
+    int rc = pool_create(s->pool, p->device, cap);
     int least = 0, greatest = 0;
     if (!rc && cudaDeviceGetStreamPriorityRange(&least, &greatest) != cudaSuccess)
         rc = set_error(NB_ECUDA, "stream priority query failed");
@@ -464,6 +469,8 @@ int nb_server_create(const nb_server_params *p, nb_server **out)
         gr.order = (g & 2) ? 6 : 2;
         const int prio = (g & 1) ? least : greatest;   // the small jobs' groups first
         rc = set_create(gr.set, p->max_jobs, cap, prio);
+        gr.set.part_ordered = true;
+        gr.set.part_limit = (int64_t)std::max(GROUP_PART_LEAST, p->hbm_budget_bytes / 32.0);
         if (!rc && cudaStreamCreateWithPriority(&gr.stream, cudaStreamNonBlocking, prio) != cudaSuccess)
             rc = set_error(NB_ECUDA, "stream creation failed");
         for (StepSlot &sl : gr.slot) {

@@ -210,11 +210,13 @@ int tune_pair(const Pool &P, ClusterSet &C, int precision, const Phys &ph, cudaS
         const int Is[] = {1, 2, 4, 8};
         for (int I : Is) {
             if (!pair_variant_exists(mode, I)) continue;
-            const int occ = pair_occupancy(mode, I);
+            const int occ = def.pl.d.sym ? sym_occupancy(mode, I) : pair_occupancy(mode, I);
             // finer j-ranges only pay when full-width units are scarce
             int64_t w_full = 0;
             for (int32_t k = 0; k < C.K; ++k)
-                w_full += ((C.nk[k] + TILE * I - 1) / (TILE * I)) * ((C.nk[k] + TILE - 1) / TILE);
+                w_full += def.pl.d.sym ? SymRows(C.nk[k], TILE * I).tiles() * I
+                                       : ((C.nk[k] + TILE * I - 1) / (TILE * I)) *
+                                             ((C.nk[k] + TILE - 1) / TILE);
             const bool scarce = w_full < 2 * (int64_t)P.num_sms * occ;
             // grids of 1 to MAX_WAVES resident waves, and single waves a
             // little below the occupancy limit.  With the near-pair pass
@@ -237,6 +239,8 @@ int tune_pair(const Pool &P, ClusterSet &C, int precision, const Phys &ph, cudaS
                 Plan pl;
                 rc = plan_make(P, C, precision, st, pl, &s, false);
                 if (rc) break;
+                // a shape whose symmetric slots do not fit the storage
+                if (pl.pl.d.sym != def.pl.d.sym) continue;
                 const int64_t tag = (pl.pl.d.G * 16 + I) * 256 + jt;
                 bool dup = false;
                 for (int64_t v : seen) dup = dup || v == tag;
