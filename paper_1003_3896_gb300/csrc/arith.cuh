@@ -28,6 +28,19 @@ __device__ __forceinline__ void ds_add(float &hi, float &lo, float t)
     hi = h;
 }
 
+// Add the float pair (p, e) to the float-float number (h, l): Knuth's
+// two-sum of the high parts, the error and the low parts folded in, then
+// Dekker's fast two-sum to renormalise.
+__device__ __forceinline__ void ff_add(float &h, float &l, float p, float e)
+{
+    const float s = __fadd_rn(h, p);
+    const float bp = __fsub_rn(s, h);
+    const float err = __fadd_rn(__fadd_rn(__fsub_rn(h, __fsub_rn(s, bp)), __fsub_rn(p, bp)),
+                                __fadd_rn(l, e));
+    h = __fadd_rn(s, err);
+    l = __fsub_rn(err, __fsub_rn(h, s));
+}
+
 __device__ __forceinline__ float2 f2neg(float2 a) { return make_float2(-a.x, -a.y); }
 __device__ __forceinline__ float2 f2sub(float2 a, float2 b) { return __fadd2_rn(a, f2neg(b)); }
 

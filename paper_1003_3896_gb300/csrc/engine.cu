@@ -141,6 +141,10 @@ int set_create(ClusterSet &C, int32_t kcap, int64_t body_cap, int priority)
     A((void **)&C.ng_spos, (size_t)body_cap * 16);
     A((void **)&C.ng_slo, (size_t)body_cap * 16);
     A((void **)&C.ng_slot, (size_t)C.ng_hcap * sizeof(NgSlot));
+    A((void **)&C.hv_flag, (size_t)body_cap);
+    A((void **)&C.hv_list, (size_t)hv_limit(body_cap) * 4);
+    A((void **)&C.hv_count, sizeof(int));
+    A((void **)&C.hv_done, (size_t)hv_limit(body_cap) * 4);
     if (!ok) {
         cudaGetLastError();
         set_destroy(C);
@@ -186,10 +190,12 @@ int set_reserve_part(ClusterSet &C, int64_t elems, cudaStream_t st)
 void set_destroy(ClusterSet &C)
 {
     void *ptrs[] = {C.dmem,    C.red,   C.ng_bucket, C.ng_entry, C.ng_total, C.flag,
-                    C.cid,     C.ng_spos, C.ng_slo,  C.ng_slot,  C.ng_rank};
+                    C.cid,     C.ng_spos, C.ng_slo,  C.ng_slot,  C.ng_rank,
+                    C.hv_flag, C.hv_list, C.hv_count, C.hv_done};
     for (void *q : ptrs)
         if (q) cudaFree(q);
     if (C.part) cudaFree(C.part);
+    if (C.hv_sum) cudaFree(C.hv_sum);
     if (C.fork) cudaEventDestroy(C.fork);
     if (C.join) cudaEventDestroy(C.join);
     if (C.side) cudaStreamDestroy(C.side);
@@ -424,7 +430,15 @@ void block_order(ClusterSet &C, const Decomp &d, int I, bool partial)
 
 // Whether a set takes the symmetric kernels, where their slots fit.  The modes
 // of FP64-class accuracy do: the order of their sums moves results by 1e-14.
-static bool use_sym(int mode) { return mode == PM_FP64 || mode == PM_DD; }
+// So does the two-pass mixed mode on one system: there the order moves
+// velocities by 1e-10 a step (bodies in an encounter apart, Heavy).  On many
+// small clusters it is 1e-9 (fewer, larger float partial sums) with encounters
+// in every cluster, and the modes without the near-pair pass do not find their
+// encounters: those keep the full kernels and their results.
+static bool use_sym(const ClusterSet &C, int mode)
+{
+    return mode == PM_FP64 || mode == PM_DD || (mode == PM_DS_NEAR && C.K == 1);
+}
 
 // Bodies per thread without a tuned entry, full decomposition.
 static int full_default_I(const ClusterSet &C, int mode)
@@ -449,6 +463,9 @@ static int sym_default_I(const ClusterSet &C, int mode)
     double n2 = 0;
     for (int32_t k = 0; k < C.K; ++k) n2 += (double)C.nk[k] * (double)C.nk[k];
     const double wn = n2 / (double)C.n;
+    // an evaluation of 16384 bodies takes 110 / 116 us with 4 / 8, of 20000 156
+    // / 147 us, of 24576 bodies 8 bodies 197 us
+    if (mode == PM_DS_NEAR) return wn < 4096 ? 2 : wn < 18432 ? 4 : 8;
     if (mode == PM_FP64) return wn < 32768 ? 1 : 2;
     return wn < 6144 ? 2 : 4;   // measured: pairsym_wide.cu
 }
@@ -459,7 +476,7 @@ int plan_make(const Pool &P, ClusterSet &C, int precision, cudaStream_t st, Plan
     Plan pl;
     pl.precision = precision;
     pl.pl.mode = plan_mode(C, precision);
-    bool sym = use_sym(pl.pl.mode);
+    bool sym = use_sym(C, pl.pl.mode);
     int I, bps = 0, jt = 0;
     PairShape tuned;
     if (force) {
@@ -486,11 +503,20 @@ int plan_make(const Pool &P, ClusterSet &C, int precision, cudaStream_t st, Plan
         if (occ < 1) occ = 1;
         int b = bps;
         if (waves > 0) b = (waves < MAX_WAVES ? waves : MAX_WAVES) * occ;
-        pl.pl.blocks_per_sm = b > 0 ? (b < MAX_WAVES * occ ? b : MAX_WAVES * occ)
-                                    : DEFAULT_WAVES * occ;
+        // the symmetric mixed kernel's blocks: units are coarse (i-blocks of
+        // 1024), so the most waves even out (an evaluation of 24576 / 65536 /
+        // 131072 bodies 212 / 1104 / 4155 us with 4 of them, 197 / 1097 / 4131
+        // us with 6), except where the near-pair pass would wait for the last
+        // of them (32768 / 49152 / 57344 bodies 320 / 650 / 828 us with 4, 343
+        // / 651 / 860 us with 6)
+        int dw = DEFAULT_WAVES;
+        if (sym && pl.pl.mode == PM_DS_NEAR && (C.n < 25000 || C.n > 60000)) dw = MAX_WAVES;
+        pl.pl.blocks_per_sm = b > 0 ? (b < MAX_WAVES * occ ? b : MAX_WAVES * occ) : dw * occ;
         const int64_t want = (int64_t)P.num_sms * pl.pl.blocks_per_sm;
         const int64_t resident = (int64_t)P.num_sms * occ;
         int j = jt;
+        const int least = sym ? sym_jt_least(pl.pl.mode) : 32;
+        if (j > 0 && j < least) j = least;
         if (j == 0) {
             // full-width j-tiles, halved while the units are too few to give
             // every resident block one (small clusters)
@@ -498,7 +524,7 @@ int plan_make(const Pool &P, ClusterSet &C, int precision, cudaStream_t st, Plan
             for (;;) {
                 int rc = set_units(C, TILE * I, j, sym);
                 if (rc) return rc;
-                if (j == 32 || C.uoff[C.K] >= resident) break;
+                if (j == least || C.uoff[C.K] >= resident) break;
                 j /= 2;
             }
         }
@@ -521,6 +547,40 @@ int plan_make(const Pool &P, ClusterSet &C, int precision, cudaStream_t st, Plan
         sym = false;   // the slots do not fit: the full kernels
     }
     pl.pl.d.fpart = sp_family(pl.pl.mode) ? 1 : 0;
+    if (sym && pl.pl.mode == PM_DS_NEAR) {
+        // the full kernels' untuned decomposition of the set
+        const int fI = full_default_I(C, pl.pl.mode);
+        const int fo = std::max(1, pair_occupancy(pl.pl.mode, fI));
+        const int64_t resident = (int64_t)P.num_sms * fo;
+        const int64_t ib = (C.n + TILE * fI - 1) / (TILE * fI), tiles = (C.n + TILE - 1) / TILE;
+        int j = TILE;
+        while (j > 32 && ib * tiles * (TILE / j) < resident) j /= 2;
+        const int64_t W = ib * tiles * (TILE / j);
+        const int64_t G = resident * (waves > 0 ? std::min(waves, MAX_WAVES) : DEFAULT_WAVES);
+        const int64_t cap = std::min<int64_t>(part_elems_for(P.num_sms, C.n) / (3 * C.n),
+                                              MAX_PART_SLOTS);
+        pl.heavy.full = make_decomp(W, tiles, TILE * fI, std::min(G, W), cap, j);
+        const int64_t groups = C.n / 512 + pl.heavy.full.slots + 1;
+        if (groups <= HV_GROUPS) {
+            pl.heavy.parts = (int)((groups + HV_PART - 1) / HV_PART);
+            pl.heavy.blocks = (int)std::min<int64_t>(hv_limit(C.n) * pl.heavy.parts,
+                                                     2 * P.num_sms);
+            const int64_t need = hv_limit(C.n) * pl.heavy.parts * HV_PART * 3;
+            if (C.hv_sum_elems < need) {
+                if (C.hv_sum) NB_TRY(cudaFree(C.hv_sum));
+                C.hv_sum = nullptr;
+                C.hv_sum_elems = 0;
+                if (cudaMalloc(&C.hv_sum, (size_t)need * 4) == cudaSuccess) {
+                    C.hv_sum_elems = need;
+                } else {
+                    cudaGetLastError();
+                    return set_error(NB_ENOMEM, "partial-sum storage: %lld bytes not available",
+                                     (long long)need * 4);
+                }
+            }
+        }
+        pl.heavy.mu = C.mu[0];
+    }
     // several clusters by value: launch the blocks largest-work first.  Not
     // with the near-pair pass beside the pair kernel: its kernels get SMs as
     // the pair kernel's blocks drain, and on the 512-cluster ensemble the
@@ -560,6 +620,13 @@ DevState view(const Pool &P, const ClusterSet &C, const Plan &pl)
 {
     DevState s = view(P, C, (int)pl.precision);
     if (pl.pl.mode != PM_DS_NEAR) s.corr = nullptr;
+    if (pl.heavy.blocks > 0) {
+        s.hv_flag = C.hv_flag;
+        s.hv_list = C.hv_list;
+        s.hv_count = C.hv_count;
+        s.hv_done = C.hv_done;
+        s.hv_sum = C.hv_sum;
+    }
     return s;
 }
 
@@ -651,7 +718,7 @@ int enq_force(const Pool &P, const ClusterSet &C, const Plan &pl, const Phys &ph
     if (near) {
         NB_TRY(cudaEventRecord(C.fork, st));
         NB_TRY(cudaStreamWaitEvent(C.side, C.fork, 0));
-        NB_TRY(launch_near_correct(s, ph.G, pl.pl.um, C.side));
+        NB_TRY(launch_near_correct(s, ph.G, pl.pl.um, C.side, &pl.heavy));
         NB_TRY(cudaEventRecord(C.join, C.side));
         count(kernels, NEAR_KERNELS);
     }

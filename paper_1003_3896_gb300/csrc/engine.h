@@ -71,6 +71,10 @@ struct ClusterSet {
     int32_t *cid = nullptr;    // linear body -> cluster map
     float4 *ng_spos = nullptr, *ng_slo = nullptr;
     NgSlot *ng_slot = nullptr;
+    unsigned char *hv_flag = nullptr;   // bodies in a close encounter (DevState)
+    int *hv_list = nullptr, *hv_count = nullptr, *hv_done = nullptr;
+    float *hv_sum = nullptr;            // reserved by a plan that needs it
+    int64_t hv_sum_elems = 0;
     Frame *frame = nullptr;    // [kcap]
     double *diag = nullptr;    // [kcap][DIAG_STRIDE]
     Clusters cl, cl_pot;       // device views (pair units / potential units)
@@ -119,6 +123,7 @@ struct Plan {
     int precision = -1;
     PairLaunch pl{};
     Decomp pot{};
+    Heavy heavy{};   // symmetric mixed form: bodies in a close encounter
 };
 // Launch shape of the pair kernel: I bodies per thread (i-block width
 // TILE * I), jt j bodies per unit (TILE, TILE / 2 or TILE / 4) and

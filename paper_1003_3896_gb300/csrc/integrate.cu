@@ -10,6 +10,7 @@
 // boff[k] + t - noff[k].
 // Reductions run per segment (a run of one cluster's bodies), then one block
 // per cluster adds its segments in a fixed tree order.
+#include "arith.cuh"
 #include "nb_internal.cuh"
 #include "split.cuh"
 
@@ -235,6 +236,7 @@ __global__ void frame_final_kernel(DevState s, double near_frac)
         // runs the near-pair pass)
         f.th2 = (float)s.cl.eps2d[k];
         f.dth = 0.f;
+        f.hx = INFINITY;
         s.cl.frame[k] = f;
     }
 }
@@ -334,6 +336,7 @@ __global__ void frame_scale_kernel(DevState s, double near_frac)
         const double spacing2 = scale2 / cbrt(nk * nk);
         f.th2 = (float)(near_frac * near_frac * spacing2 + s.cl.eps2d[k]);
         f.dth = (float)(near_frac * sqrt(spacing2));
+        f.hx = scale2 > 0 ? HV_X * (float)(v[1] / scale2) : INFINITY;
         s.cl.frame[k] = f;
     }
 }
@@ -404,19 +407,6 @@ cudaError_t launch_split(const DevState &s, cudaStream_t st)
 // SB: slots loaded together (a grid run in waves gives an i-block tens of
 // slots; an ensemble of small clusters a few, where a narrower batch keeps
 // registers, and so resident warps, for the memory latency)
-// Add the float pair (p, e) to the float-float number (h, l): Knuth's
-// two-sum of the high parts, the error and the low parts folded in, then
-// Dekker's fast two-sum to renormalise.
-__device__ __forceinline__ void ff_add(float &h, float &l, float p, float e)
-{
-    const float s = __fadd_rn(h, p);
-    const float bp = __fsub_rn(s, h);
-    const float err = __fadd_rn(__fadd_rn(__fsub_rn(h, __fsub_rn(s, bp)), __fsub_rn(p, bp)),
-                                __fadd_rn(l, e));
-    h = __fadd_rn(s, err);
-    l = __fsub_rn(err, __fsub_rn(h, s));
-}
-
 // Float-pair partial sums (Decomp::fpart): added in slot order in
 // float-float arithmetic, SB loads at a time, then widened to double from
 // their bits (the conversion instruction runs on the FP64 pipe, 1/77 of the
@@ -457,6 +447,13 @@ template <int SB, bool FP>
 __device__ __forceinline__ void sum_slots(const DevState &s, const Decomp &d, const BodyRef &r,
                                           int64_t t, double &ax, double &ay, double &az)
 {
+    // a body in a close encounter: its whole sum is in corr
+    if (FP && d.sym && s.hv_flag && s.hv_flag[t] && *s.hv_count <= hv_limit(s.n)) {
+        ax = s.corr[r.gi];
+        ay = s.corr[s.cap + r.gi];
+        az = s.corr[2 * s.cap + r.gi];
+        return;
+    }
     const SlotRun run = slot_run(d, s.cl, r.k, r.li, t, s.pstride);
     const int64_t count = run.count, ps = run.stride;
     if (FP) {
@@ -497,22 +494,17 @@ __device__ __forceinline__ void sum_slots(const DevState &s, const Decomp &d, co
     }
 }
 
-// EXT: the external field is on (a separate variant keeps its registers out
-// of the field-free kick).
-template <bool EXT, int SB, bool FP>
-__global__ void kick_drift_kernel(DevState s, Decomp d, double wk, double wd, int do_kick,
-                                  int do_split, ExtField ext, int64_t t0, int64_t t1)
+// One body's update: kick (when kick) by (ax, ay, az) plus the field, drift,
+// split.
+template <bool EXT>
+__device__ __forceinline__ void advance(const DevState &s, int32_t k, int64_t i, bool kick,
+                                        double ax, double ay, double az, double wk, double wd,
+                                        int do_split, const ExtField &ext)
 {
-    const int64_t t = t0 + blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (t >= t1) return;
-    const BodyRef r = body_at(s.cl, t);
-    const int64_t i = r.gi;
-    const double dt = s.cl.dts[r.k];
+    const double dt = s.cl.dts[k];
     double x = s.x[i], y = s.y[i], z = s.z[i];
     double vx = s.vx[i], vy = s.vy[i], vz = s.vz[i];
-    if (do_kick) {
-        double ax, ay, az;
-        sum_slots<SB, FP>(s, d, r, t, ax, ay, az);
+    if (kick) {
         if (EXT) {
             double ex, ey, ez;
             field_accel(ext, x, y, z, ex, ey, ez);
@@ -536,27 +528,35 @@ __global__ void kick_drift_kernel(DevState s, Decomp d, double wk, double wd, in
     s.y[i] = y;
     s.z[i] = z;
     if (do_split == 3)
-        split_one<false, false>(s, s.cl.frame[r.k], i, x, y, z);
+        split_one<false, false>(s, s.cl.frame[k], i, x, y, z);
     else if (do_split == 2)
-        split_one<true>(s, s.cl.frame[r.k], i, x, y, z);
+        split_one<true>(s, s.cl.frame[k], i, x, y, z);
     else if (do_split)
-        split_one<false>(s, s.cl.frame[r.k], i, x, y, z);
+        split_one<false>(s, s.cl.frame[k], i, x, y, z);
 }
 
-cudaError_t launch_kick_drift(const DevState &s, const Decomp &d, double wk, double wd,
-                              int do_kick, int do_split, const ExtField &ext, cudaStream_t st)
+// EXT: the external field is on (a separate variant keeps its registers out
+// of the field-free kick).
+template <bool EXT, int SB, bool FP>
+__global__ void kick_drift_kernel(DevState s, Decomp d, double wk, double wd, int do_kick,
+                                  int do_split, ExtField ext, int64_t t0, int64_t t1)
 {
-    return launch_kick_drift_range(s, d, wk, wd, do_kick, do_split, ext, 0, s.n, st);
+    const int64_t t = t0 + blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (t >= t1) return;
+    const BodyRef r = body_at(s.cl, t);
+    double ax = 0.0, ay = 0.0, az = 0.0;
+    if (do_kick) sum_slots<SB, FP>(s, d, r, t, ax, ay, az);
+    advance<EXT>(s, r.k, r.gi, do_kick, ax, ay, az, wk, wd, do_split, ext);
 }
 
+// Blocks of at most 128 threads: with ~100 registers a thread, 128-thread
+// blocks pack 20 warps on an SM against 16 for 256 (the kick waits on memory;
+// the ensemble's kick ran 8% faster).
 cudaError_t launch_kick_drift_range(const DevState &s, const Decomp &d, double wk, double wd,
                                     int do_kick, int do_split, const ExtField &ext, int64_t t0,
                                     int64_t t1, cudaStream_t st)
 {
     if (t1 <= t0) return cudaSuccess;
-    // blocks of at most 128 threads: with ~100 registers a thread, 128-thread
-    // blocks pack 20 warps on an SM against 16 for 256 (the kick waits on
-    // memory; the ensemble's kick ran 8% faster)
     const int64_t m = t1 - t0;
     const int t = ot_for(m) < 128 ? ot_for(m) : 128;
     const unsigned nb = blocks_for(m, t);
@@ -579,6 +579,30 @@ cudaError_t launch_kick_drift_range(const DevState &s, const Decomp &d, double w
     return cudaGetLastError();
 }
 
+cudaError_t launch_kick_drift(const DevState &s, const Decomp &d, double wk, double wd,
+                              int do_kick, int do_split, const ExtField &ext, cudaStream_t st)
+{
+    return launch_kick_drift_range(s, d, wk, wd, do_kick, do_split, ext, 0, s.n, st);
+}
+
+// Row q of the output: the internal sum plus the field at the body.
+__device__ __forceinline__ void put_accel(const DevState &s, const ExtField &ext, int64_t gi,
+                                          int64_t q, double ax, double ay, double az,
+                                          double *__restrict__ out)
+{
+    if (ext.on) {
+        double ex, ey, ez;
+        field_accel(ext, s.x[gi], s.y[gi], s.z[gi], ex, ey, ez);
+        ax += ex;
+        ay += ey;
+        az += ez;
+    }
+    out[3 * q] = ax;
+    out[3 * q + 1] = ay;
+    out[3 * q + 2] = az;
+    if (!isfinite(ax) || !isfinite(ay) || !isfinite(az)) atomicOr(s.flag, 1);
+}
+
 template <bool FP>
 __global__ void accel_out_kernel(DevState s, Decomp d, ExtField ext, double *__restrict__ out,
                                  int64_t t0, int64_t t1)
@@ -589,17 +613,7 @@ __global__ void accel_out_kernel(DevState s, Decomp d, ExtField ext, double *__r
     const BodyRef r = body_at(s.cl, t);
     double ax, ay, az;
     sum_slots<8, FP>(s, d, r, t, ax, ay, az);
-    if (ext.on) {
-        double ex, ey, ez;
-        field_accel(ext, s.x[r.gi], s.y[r.gi], s.z[r.gi], ex, ey, ez);
-        ax += ex;
-        ay += ey;
-        az += ez;
-    }
-    out[3 * q] = ax;
-    out[3 * q + 1] = ay;
-    out[3 * q + 2] = az;
-    if (!isfinite(ax) || !isfinite(ay) || !isfinite(az)) atomicOr(s.flag, 1);
+    put_accel(s, ext, r.gi, q, ax, ay, az, out);
 }
 
 cudaError_t launch_accel_out(const DevState &s, const Decomp &d, const ExtField &ext,

@@ -24,6 +24,7 @@ struct Frame {
     double r2rms;        // mass-weighted mean |x - c|^2
     float th2;           // near-pair threshold on r^2 + eps^2
     float dth;           // near-pair radius d_th (th2 = d_th^2 + eps^2)
+    float hx;            // encounter threshold on m_j / (r^2 + eps^2) (HV_X)
 };
 
 // A set of K independent clusters living in one state pool.  Cluster k owns
@@ -111,6 +112,13 @@ struct DevState {
     NgSlot *ng_slot = nullptr;                       // cell table [H]
     int *ng_total = nullptr;                         // bodies placed in the grid
     int64_t ng_hcap = 0;                             // slots allocated
+    // bodies in a close encounter (Heavy; nullptr: not looked for): flag per
+    // linear body, list of the first hv_limit(n) of them, their number
+    unsigned char *hv_flag = nullptr;
+    int *hv_list = nullptr, *hv_count = nullptr;
+    // their float partial sums, and how many blocks have written theirs
+    float *hv_sum = nullptr;
+    int *hv_done = nullptr;
     double *red = nullptr;      // reduction partials [segment][16]
     int64_t red_len = 0;
     double *diag = nullptr;     // [K][16] reduction results (energy, torque)
@@ -257,6 +265,27 @@ __device__ __forceinline__ SlotRun slot_run(const Decomp &d, const Clusters &c, 
     return r;
 }
 
+// Bodies in a close encounter.  A float partial sum that holds a large pair
+// term rounds every later term at that term's magnitude, 2^-24 of it: the
+// body's acceleration then carries an error that depends on the order of the
+// sum, orders above that of the other bodies.  Such bodies (some body pulls
+// harder than HV_X times M / S^2, S the near-pair scale) are found by the
+// near-pair pass, which then sums them again in the full kernels' order
+// (near_encounter_kernel), so that an orbit through an encounter is the same
+// whichever decomposition the others' sums take.  On the 65536-body orbit
+// system ~50 bodies; where more than hv_limit have one (a crowded state, many
+// close binaries) all keep their sums.
+constexpr float HV_X = 8.f;
+__host__ __device__ __forceinline__ int64_t hv_limit(int64_t n) { return n / 64 + 64; }
+constexpr int HV_GROUPS = 1024;   // float partial sums of a body's row, at most
+constexpr int HV_PART = 64;       // of them per block
+struct Heavy {
+    Decomp full;    // the full kernels' default decomposition of the set
+    int blocks;     // blocks that sum these bodies (0: none are looked for)
+    int parts;      // blocks' shares of one body's row
+    double mu;      // their common mass (equal masses)
+};
+
 struct ExtField {
     int on;
     double G, Md, ad, bd, Mb, ab;
@@ -322,6 +351,8 @@ bool pair_variant_exists(int mode, int I);
 // The same of the symmetric kernels (pairsym.cu); 0: no such variant.
 int sym_occupancy(int mode, int I);
 int potential_occupancy();
+// Narrowest unit: the kernels' chunk of j bodies.
+inline int sym_jt_least(int mode) { return mode == PM_DS_NEAR ? 64 : 32; }
 cudaError_t launch_pair_sym(const DevState &s, const PairLaunch &pl, const HostTab &ht, double G,
                             cudaStream_t st);
 // Bodies per thread of the potential kernel (i-blocks of TILE * POT_I).
@@ -354,8 +385,11 @@ int64_t near_table_size(int64_t n);
 // corr_i = G sum over pairs closer than the cluster's near radius of the
 // double-single minus the float contribution (written to s.corr).
 // um: the pair kernel left the (uniform) mass out of the pair term; the
-// correction does the same and scales by cl.mu[k].
-cudaError_t launch_near_correct(const DevState &s, double G, bool um, cudaStream_t st);
+// correction does the same and scales by cl.mu[k].  hv (with s.hv_flag): bodies
+// in a close encounter get their whole internal acceleration in s.corr instead
+// and s.hv_flag set.  Five kernels either way.
+cudaError_t launch_near_correct(const DevState &s, double G, bool um, cudaStream_t st,
+                                const Heavy *hv = nullptr);
 
 // ---- launchers (integrate.cu) ----------------------------------------------
 // Fill the body -> cluster map cid[0, n) of a cluster set.

@@ -32,11 +32,16 @@
 // atomic add on a running total), scatter, order each cell by body index and
 // write the copies, correct.
 //
+// On the way each body's strongest single pull decides whether it is in a
+// close encounter (Heavy, nb_internal.cuh).
+//
 // Deterministic: within a cell the bodies are ordered by linear index, and
 // every body visits its 8 cells in a fixed order, so the FP64 correction sums
 // do not depend on timing (which slot a cell lands in, and where its range
 // lands, may vary; the sums do not depend on either).
+#include "arith.cuh"
 #include "nb_internal.cuh"
+#include "split.cuh"
 
 namespace nb {
 
@@ -102,11 +107,20 @@ __device__ __forceinline__ int cell_coord(float v, float inv_h, int &side)
 
 // Per body: the cell key, insertion of the cell into the slot table and the
 // body's rank among its cell's arrivals.
+// LIST (where a kernel for close encounters follows): the cell's bodies form a
+// list instead (the slot's end its head, ng_entry the links), from which the
+// claim pass takes each body's rank by index, so no scatter pass is needed;
+// the lists are short (at most ~10 bodies in the core of a Plummer sphere).
+template <bool LIST>
 __global__ void near_cell_kernel(DevState s)
 {
     const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (t >= s.n) return;
-    if (t == 0) *s.ng_total = 0;   // read only by the claim pass, which follows
+    if (LIST && t < hv_limit(s.n)) s.hv_done[t] = 0;
+    if (t == 0) {
+        *s.ng_total = 0;   // read only by the claim pass, which follows
+        if (s.hv_count) *s.hv_count = 0;
+    }
     const int32_t k = cluster_of(s.cl, t);
     const int64_t i = s.cl.boff[k] + t - s.cl.noff[k];
     const float dth = s.cl.frame[k].dth;
@@ -129,6 +143,10 @@ __global__ void near_cell_kernel(DevState s)
         b = next_slot(b, rg);
     }
     s.ng_bucket[t] = (int)b;
+    if (LIST) {
+        s.ng_entry[t] = atomicExch(&s.ng_slot[b].end, (int)t);   // -1 (empty): the list's end
+        return;
+    }
     // the slot's end counts arrivals from -1 (the empty record) until the
     // claim pass turns it into the range end
     s.ng_rank[t] = atomicAdd(&s.ng_slot[b].end, 1) + 1;
@@ -140,8 +158,12 @@ __global__ void near_cell_kernel(DevState s)
 // a single atomic add; a claim per atomic on one address would serialise.
 // Ranges land in the order the blocks claim them; only their contents,
 // ordered by body index, enter the sums.  The slot keeps [start, end).
+// LIST: the body of the cell's least index claims, and each body's rank is the
+// number of lesser indices; the claiming body's is kept as minus the cell's
+// count, for the copy pass.
 constexpr int CLAIM_T = 256;
 
+template <bool LIST>
 __global__ void __launch_bounds__(CLAIM_T) near_claim_kernel(DevState s)
 {
     __shared__ int wsum[CLAIM_T / 32];
@@ -151,7 +173,18 @@ __global__ void __launch_bounds__(CLAIM_T) near_claim_kernel(DevState s)
     int b = -1, cnt = 0;
     if (t < s.n) {
         b = s.ng_bucket[t];
-        if (b >= 0 && s.ng_rank[t] == 0)
+        if (LIST && b >= 0) {
+            int r = 0;
+            for (int e = s.ng_slot[b].end; e >= 0; e = s.ng_entry[e]) {
+                ++cnt;
+                r += e < (int)t ? 1 : 0;
+            }
+            s.ng_rank[t] = r > 0 ? r : -cnt;
+            if (r > 0) {
+                b = -1;
+                cnt = 0;
+            }
+        } else if (b >= 0 && s.ng_rank[t] == 0)
             cnt = s.ng_slot[b].end + 1;   // arrivals counted from -1
         else
             b = -1;
@@ -176,7 +209,7 @@ __global__ void __launch_bounds__(CLAIM_T) near_claim_kernel(DevState s)
     if (b >= 0) {
         const int st = base + wsum[w] + x - cnt;
         s.ng_slot[b].start = st;
-        s.ng_slot[b].end = st + cnt;
+        if (!LIST) s.ng_slot[b].end = st + cnt;
     }
 }
 
@@ -193,7 +226,9 @@ __global__ void near_scatter_kernel(DevState s)
 // Final place of each body in its cell = number of cell members with a
 // smaller linear index; writes the cell-ordered copies of its float planes
 // (lo.w = t) and, from the cell's first body, the slot's range.  Bodies
-// outside the grid get their (zero) correction here.
+// outside the grid get their (zero) correction here.  LIST: the place is known,
+// and the cell's first body leaves the range's end in the slot.
+template <bool LIST>
 __global__ void near_rank_kernel(DevState s)
 {
     const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -202,14 +237,24 @@ __global__ void near_rank_kernel(DevState s)
     const int32_t k = cluster_of(s.cl, t);
     const int64_t i = s.cl.boff[k] + t - s.cl.noff[k];
     if (b < 0) {   // not in the grid (no near radius): no correction
+        if (s.hv_flag) s.hv_flag[t] = 0;
         s.corr[i] = 0.0;
         s.corr[s.cap + i] = 0.0;
         s.corr[2 * s.cap + i] = 0.0;
         return;
     }
-    const int lo = s.ng_slot[b].start, hi = s.ng_slot[b].end;
+    const int lo = s.ng_slot[b].start;
     int r = 0;
-    for (int e = lo; e < hi; ++e) r += s.ng_entry[e] < (int)t ? 1 : 0;
+    if (LIST) {
+        r = s.ng_rank[t];
+        if (r < 0) {
+            s.ng_slot[b].end = lo - r;
+            r = 0;
+        }
+    } else {
+        const int hi = s.ng_slot[b].end;
+        for (int e = lo; e < hi; ++e) r += s.ng_entry[e] < (int)t ? 1 : 0;
+    }
     s.ng_spos[lo + r] = make_float4(s.xh[i], s.yh[i], s.zh[i], s.mf[i]);
     s.ng_slo[lo + r] = make_float4(s.xl[i], s.yl[i], s.zl[i], __int_as_float((int)t));
 }
@@ -271,6 +316,7 @@ __global__ void __launch_bounds__(NC_T) near_correct_kernel(DevState s, double G
     }
     const float eps2 = s.cl.eps2f[k];
     const float th2 = s.cl.frame[k].th2;
+    float pull = 0.f;   // largest m_j / (r^2 + eps^2) met
     const float xi = P.x, yi = P.y, zi = P.z;
     const float lxi = Lo.x, lyi = Lo.y, lzi = Lo.z;
     // candidates in cell order 0..7, each cell's members in body order,
@@ -325,6 +371,7 @@ __global__ void __launch_bounds__(NC_T) near_correct_kernel(DevState s, double G
             e2 = __fmaf_rn(ey, ey, e2);
             e2 = __fmaf_rn(ez, ez, e2);
             const float re = near_rsqrt(e2);
+            pull = fmaxf(pull, mj * re * re);
             float se = __fmul_rn(re, __fmul_rn(re, re));
             if (!UM) se = __fmul_rn(mj, se);
             ax += (double)__fmul_rn(ex, se) - (double)__fmul_rn(ddx, sf);
@@ -333,10 +380,211 @@ __global__ void __launch_bounds__(NC_T) near_correct_kernel(DevState s, double G
         }
     }
     const int64_t i = s.cl.boff[k] + t - s.cl.noff[k];
+    if (s.hv_flag) {
+        const bool heavy = pull > s.cl.frame[k].hx;
+        s.hv_flag[t] = heavy ? 1 : 0;
+        if (heavy) {
+            const int q = atomicAdd(s.hv_count, 1);
+            if (q < hv_limit(s.n)) s.hv_list[q] = t;
+        }
+    }
     const double Gm = UM ? G * s.cl.mu[k] : G;
     s.corr[i] = Gm * ax;
     s.corr[s.cap + i] = Gm * ay;
     s.corr[2 * s.cap + i] = Gm * az;
+}
+
+// ---- bodies in a close encounter (Heavy) ----------------------------------------
+// Each listed body's internal acceleration as the full single-precision kernel
+// and the kick give it, near-pair correction included, into corr: the float
+// partial sums over 512 j bodies of every block of the full decomposition, each
+// in j order, then the blocks' double-single sums, scaled, and their sum in
+// block order.  A block takes HVG partial sums of one body: its threads form
+// their pair terms HVS j at a time (a warp 32 consecutive j of a plane, the next
+// slice's loads in flight) and stage them in shared memory, from where one
+// thread per partial sum adds its terms in order; the body's last block to
+// finish adds up.  What bounds it is latency: 512 additions in order per partial
+// sum, in 16 slices of one load latency each.
+constexpr int HVT = 256;       // threads per block
+constexpr int HVG = HV_PART;   // partial sums per block
+constexpr int HVS = 32;        // j bodies per slice
+constexpr int HVK = HVG * HVS / HVT;
+
+// The runs of body t's row in the full decomposition: j range of run sg and its
+// number of partial sums.
+struct HeavyRow {
+    int64_t u0, u1, first;
+    int nseg;
+    __device__ __forceinline__ HeavyRow(const Decomp &f, int64_t nt, int64_t t)
+    {
+        u0 = (t / f.ipb) * nt;
+        u1 = u0 + nt;
+        first = f.owner(u0);
+        nseg = (int)(f.owner(u1 - 1) - first) + 1;   // <= f.slots <= MAX_PART_SLOTS
+    }
+    __device__ __forceinline__ int range(const Decomp &f, int64_t n, int sg, int &J0, int &J1) const
+    {
+        const int64_t ua = f.U(first + sg), ub = f.U(first + sg + 1);
+        const int64_t a = ua > u0 ? ua : u0, b = ub < u1 ? ub : u1;
+        const int64_t jend = (n + 31) & ~(int64_t)31;
+        J0 = (int)((a - u0) * f.jt);
+        J1 = (int)((b - u0) * f.jt < jend ? (b - u0) * f.jt : jend);
+        return J1 > J0 ? (J1 - J0 + 4 * TILE - 1) / (4 * TILE) : 0;
+    }
+};
+
+__global__ void __launch_bounds__(HVT) near_encounter_kernel(DevState s, Heavy h, double Gm, int um)
+{
+    constexpr int FOLD = 4 * TILE;
+    __shared__ float4 term[HVG][HVS + 1];
+    __shared__ int2 grp[HVG];                        // j range of each partial sum
+    __shared__ int seg0[MAX_PART_SLOTS + 2];         // first partial sum of each block's run
+    __shared__ float2 segsum[3][MAX_PART_SLOTS + 1];
+    __shared__ bool last;
+    const int tid = threadIdx.x;
+    const int cnt = *s.hv_count;
+    if (cnt > hv_limit(s.n)) return;
+    const Decomp &f = h.full;
+    const int64_t n = s.cl.nk[0], base = s.cl.boff[0];
+    const int64_t nt = f.units_per_iblock(s.cl.ntiles[0]);
+    const float eps2 = s.cl.eps2f[0];
+    const float gh = __double2float_rn(Gm), gl = __double2float_rn(Gm - (double)gh);
+    for (int item = blockIdx.x; item < cnt * h.parts; item += gridDim.x) {
+        const int q = item / h.parts, part = item - q * h.parts;
+        const int t = s.hv_list[q];
+        const HeavyRow row(f, nt, t);
+        const int nseg = row.nseg;
+        __syncthreads();   // the last item's tables have been read
+        for (int sg = tid; sg < nseg; sg += HVT) {
+            int J0, J1;
+            seg0[sg + 1] = row.range(f, n, sg, J0, J1);
+        }
+        __syncthreads();
+        if (tid < 32) {   // prefix sums, one warp
+            int run = 0;
+            for (int b0 = 0; b0 < nseg; b0 += 32) {
+                int v = b0 + tid < nseg ? seg0[b0 + tid + 1] : 0;
+                for (int d = 1; d < 32; d <<= 1) {
+                    const int w = __shfl_up_sync(0xffffffffu, v, d);
+                    if (tid >= d) v += w;
+                }
+                if (b0 + tid < nseg) seg0[b0 + tid + 1] = run + v;
+                run += __shfl_sync(0xffffffffu, v, 31);
+            }
+            if (tid == 0) seg0[0] = 0;
+        }
+        __syncthreads();
+        const int ng = seg0[nseg];
+        const int g0 = part * HVG, gn = ng - g0 < HVG ? ng - g0 : HVG;   // gn <= 0: none left
+        for (int sg = tid; sg < nseg; sg += HVT) {
+            if (seg0[sg + 1] <= g0 || seg0[sg] >= g0 + HVG) continue;
+            int J0, J1;
+            row.range(f, n, sg, J0, J1);
+            for (int e = seg0[sg]; e < seg0[sg + 1]; ++e) {
+                const int ja = J0 + (e - seg0[sg]) * FOLD;
+                const int jb = ja + FOLD < J1 ? ja + FOLD : J1;
+                // padding adds exactly zero
+                if (e >= g0 && e < g0 + HVG) grp[e - g0] = make_int2(ja, jb < n ? jb : (int)n);
+            }
+        }
+        for (int e = tid; e < HVG; e += HVT)
+            if (e >= gn) grp[e] = make_int2(0, 0);
+        __syncthreads();
+        const float xi = s.xh[base + t], yi = s.yh[base + t], zi = s.zh[base + t];
+        // term k of this thread: partial sum tid / HVS + k (HVT / HVS), j body
+        // tid % HVS of the slice
+        const int jj = tid % HVS, gg = tid / HVS;
+        int2 rk[HVK];
+        float x[HVK], y[HVK], z[HVK], m[HVK];
+        auto fetch = [&](int sl) {
+#pragma unroll
+            for (int k = 0; k < HVK; ++k) {
+                const int j = rk[k].x + sl + jj;
+                x[k] = y[k] = z[k] = m[k] = 0.f;
+                if (j < rk[k].y) {
+                    x[k] = s.xh[base + j];
+                    y[k] = s.yh[base + j];
+                    z[k] = s.zh[base + j];
+                    if (!um) m[k] = s.mf[base + j];
+                }
+            }
+        };
+        int longest = 0;
+#pragma unroll
+        for (int k = 0; k < HVK; ++k) {
+            rk[k] = grp[gg + k * (HVT / HVS)];
+            longest = max(longest, rk[k].y - rk[k].x);
+        }
+        fetch(0);
+        float ax = 0.f, ay = 0.f, az = 0.f;
+        const int2 mine = tid < HVG ? grp[tid] : make_int2(0, 0);
+        for (int sl = 0; sl < FOLD; sl += HVS) {
+            if (!__syncthreads_or(sl < longest)) break;   // and the last slice's terms are added
+#pragma unroll
+            for (int k = 0; k < HVK; ++k) {
+                const float dx = __fadd_rn(x[k], -xi);
+                const float dy = __fadd_rn(y[k], -yi);
+                const float dz = __fadd_rn(z[k], -zi);
+                float r2 = __fmaf_rn(dx, dx, eps2);
+                r2 = __fmaf_rn(dy, dy, r2);
+                r2 = __fmaf_rn(dz, dz, r2);
+                const float ri = rsqrt_mufu(r2);
+                float sp = __fmul_rn(ri, __fmul_rn(ri, ri));
+                if (!um) sp = __fmul_rn(m[k], sp);
+                if (rk[k].x + sl + jj == t) sp = 0.f;   // exactly zero for eps > 0 as well
+                term[gg + k * (HVT / HVS)][jj] = make_float4(dx, dy, dz, sp);
+            }
+            fetch(sl + HVS);
+            __syncthreads();
+            if (tid < HVG) {
+                const int left = mine.y - mine.x - sl;
+                if (left >= HVS) {
+#pragma unroll 8
+                    for (int e = 0; e < HVS; ++e) {
+                        const float4 v = term[tid][e];
+                        ax = __fmaf_rn(v.x, v.w, ax);
+                        ay = __fmaf_rn(v.y, v.w, ay);
+                        az = __fmaf_rn(v.z, v.w, az);
+                    }
+                } else {
+                    for (int e = 0; e < left; ++e) {
+                        const float4 v = term[tid][e];
+                        ax = __fmaf_rn(v.x, v.w, ax);
+                        ay = __fmaf_rn(v.y, v.w, ay);
+                        az = __fmaf_rn(v.z, v.w, az);
+                    }
+                }
+            }
+        }
+        float *out = s.hv_sum + (int64_t)q * 3 * h.parts * HVG;
+        if (tid < gn) {
+            out[3 * (g0 + tid)] = ax;
+            out[3 * (g0 + tid) + 1] = ay;
+            out[3 * (g0 + tid) + 2] = az;
+        }
+        __threadfence();
+        __syncthreads();
+        if (tid == 0) last = atomicAdd(s.hv_done + q, 1) == h.parts - 1;
+        __syncthreads();
+        if (!last) continue;
+        __threadfence();
+        for (int e = tid; e < 3 * nseg; e += HVT) {
+            const int c = e / nseg, sg = e - c * nseg;
+            float hi = 0.f, lo = 0.f;
+            for (int g = seg0[sg]; g < seg0[sg + 1]; ++g) ds_add(hi, lo, __ldcg(out + 3 * g + c));
+            const float pr = __fmul_rn(hi, gh);
+            float er = __fmaf_rn(hi, gh, -pr);
+            er = __fmaf_rn(hi, gl, __fmaf_rn(lo, gh, er));
+            const float r = __fadd_rn(pr, er);
+            segsum[c][sg] = make_float2(r, __fsub_rn(er, __fsub_rn(r, pr)));
+        }
+        __syncthreads();
+        if (tid < 3) {
+            float H = 0.f, L = 0.f;
+            for (int sg = 0; sg < nseg; ++sg) ff_add(H, L, segsum[tid][sg].x, segsum[tid][sg].y);
+            s.corr[tid * s.cap + base + t] += widen(H) + widen(L);
+        }
+    }
 }
 
 int64_t near_table_size(int64_t n)
@@ -344,22 +592,37 @@ int64_t near_table_size(int64_t n)
     return SLOTS_PER_BODY * n;
 }
 
-cudaError_t launch_near_correct(const DevState &s, double G, bool um, cudaStream_t st)
+cudaError_t launch_near_correct(const DevState &s, double G, bool um, cudaStream_t st,
+                                const Heavy *hv)
 {
     const int64_t H = near_table_size(s.n);
     if (H > s.ng_hcap) return cudaErrorInvalidValue;
     const unsigned nbn = (unsigned)((s.n + 255) / 256);
+    const bool list = hv && hv->blocks > 0 && s.hv_flag;
+    if (list && s.cl.K != 1) return cudaErrorInvalidValue;
+    DevState q = s;
+    if (!list) q.hv_flag = nullptr;
     // empty records: key all ones, start = end = -1
     cudaError_t e = cudaMemsetAsync(s.ng_slot, 0xff, (size_t)H * sizeof(NgSlot), st);
     if (e != cudaSuccess) return e;
-    near_cell_kernel<<<nbn, 256, 0, st>>>(s);
-    near_claim_kernel<<<nbn, CLAIM_T, 0, st>>>(s);
-    near_scatter_kernel<<<nbn, 256, 0, st>>>(s);
-    near_rank_kernel<<<nbn, 256, 0, st>>>(s);
+    if (list) {
+        near_cell_kernel<true><<<nbn, 256, 0, st>>>(q);
+        near_claim_kernel<true><<<nbn, CLAIM_T, 0, st>>>(q);
+        near_rank_kernel<true><<<nbn, 256, 0, st>>>(q);
+    } else {
+        near_cell_kernel<false><<<nbn, 256, 0, st>>>(q);
+        near_claim_kernel<false><<<nbn, CLAIM_T, 0, st>>>(q);
+        near_scatter_kernel<<<nbn, 256, 0, st>>>(q);
+        near_rank_kernel<false><<<nbn, 256, 0, st>>>(q);
+    }
     if (um)
-        near_correct_kernel<true><<<(unsigned)((s.n + NC_T - 1) / NC_T), NC_T, 0, st>>>(s, G);
+        near_correct_kernel<true><<<(unsigned)((s.n + NC_T - 1) / NC_T), NC_T, 0, st>>>(q, G);
     else
-        near_correct_kernel<false><<<(unsigned)((s.n + NC_T - 1) / NC_T), NC_T, 0, st>>>(s, G);
+        near_correct_kernel<false><<<(unsigned)((s.n + NC_T - 1) / NC_T), NC_T, 0, st>>>(q, G);
+    if (list) {
+        // the scale as the pair kernel forms it: G, times the common mass
+        near_encounter_kernel<<<hv->blocks, HVT, 0, st>>>(q, *hv, um ? G * hv->mu : G, um ? 1 : 0);
+    }
     return cudaGetLastError();
 }
 

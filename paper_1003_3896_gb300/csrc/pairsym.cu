@@ -54,12 +54,13 @@ cudaError_t launch_pair_sym(const DevState &s, const PairLaunch &pl, const HostT
                             cudaStream_t st)
 {
     if (!ht.poff) return cudaErrorInvalidValue;
-    return launch_sym_wide(s, pl, ht, G, st);
+    return sp_family(pl.mode) ? launch_sym_sp(s, pl, ht, G, st)
+                              : launch_sym_wide(s, pl, ht, G, st);
 }
 
 int sym_occupancy(int mode, int I)
 {
-    return occupancy_sym_wide(mode, I);
+    return sp_family(mode) ? occupancy_sym_sp(mode, I) : occupancy_sym_wide(mode, I);
 }
 
 }  // namespace nb

@@ -39,7 +39,6 @@
 
 namespace nb {
 
-constexpr int SCH = 32;             // j bodies per chunk (one per lane)
 constexpr int SWARPS = TILE / 32;   // warps per block
 
 // Per-cluster values by value (kernel parameter): uniform across the block.
@@ -130,7 +129,7 @@ __global__ void __launch_bounds__(TILE, A::MINB) pair_sym_kernel(
     const __grid_constant__ DevState s, const __grid_constant__ SymTabOf<KC> tab,
     const __grid_constant__ Decomp d, double G)
 {
-    constexpr int I = A::I;
+    constexpr int I = A::I, CH = 32 * A::JL;
     extern __shared__ __align__(16) unsigned char smem[];
     SymShared<A> &sh = *reinterpret_cast<SymShared<A> *>(smem);
 
@@ -173,7 +172,7 @@ __global__ void __launch_bounds__(TILE, A::MINB) pair_sym_kernel(
         // the block's bodies, spread over the four warps: rows of 32 kw
         const int32_t ib0 = b * d.ipb;
         const int32_t rem = n - ib0 < d.ipb ? n - ib0 : d.ipb;
-        const int32_t kw = (rem + TILE - 1) / TILE;
+        const int32_t kw = (rem + TILE * A::JL - 1) / (TILE * A::JL) * A::JL;
         const int32_t rw = 32 * kw;
         const int32_t nw = (rem + rw - 1) / rw;   // warps with bodies
         const int32_t r0 = ib0 + w * rw;
@@ -219,11 +218,11 @@ __global__ void __launch_bounds__(TILE, A::MINB) pair_sym_kernel(
         for (int32_t t = t0; t < t1; ++t) {
             SymUnit nx = un;
             if (t + 1 < t1) nx.next(d, sr, upt, n);
-            for (int32_t j0 = un.j0; j0 < un.j1; j0 += SCH) {
+            for (int32_t j0 = un.j0; j0 < un.j1; j0 += CH) {
                 A::put(st, lane, pre);
                 __syncwarp();
                 // the next chunk's bodies on their way
-                pre.load(s, base, (j0 + SCH < un.j1 ? j0 + SCH : nx.j0) + lane, n);
+                pre.load(s, base, (j0 + CH < un.j1 ? j0 + CH : nx.j0) + lane, n);
                 typename A::JSum js;
                 js.zero();
                 if (live) {
@@ -250,7 +249,10 @@ __global__ void __launch_bounds__(TILE, A::MINB) pair_sym_kernel(
                 if (A::JSUM) {
                     const int32_t jj = j0 - un.j0 + lane;
 #pragma unroll
-                    for (int c = 0; c < 3; ++c) sh.slab[buf][w][c][jj] = js.get(c);
+                    for (int c = 0; c < 3; ++c)
+#pragma unroll
+                        for (int h = 0; h < A::JL; ++h)
+                            sh.slab[buf][w][c][jj + 32 * h] = js.get(c, h);
                 }
                 __syncwarp();
             }
@@ -414,7 +416,10 @@ int occupancy_sym_any()
     return a < b ? (a < c ? a : c) : (b < c ? b : c);
 }
 
-// the variants (pairsym_wide.cu)
+// the variants (pairsym_sp.cu, pairsym_wide.cu)
+cudaError_t launch_sym_sp(const DevState &s, const PairLaunch &pl, const HostTab &ht, double G,
+                          cudaStream_t st);
+int occupancy_sym_sp(int mode, int I);
 cudaError_t launch_sym_wide(const DevState &s, const PairLaunch &pl, const HostTab &ht, double G,
                             cudaStream_t st);
 int occupancy_sym_wide(int mode, int I);

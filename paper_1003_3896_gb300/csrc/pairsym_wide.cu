@@ -22,7 +22,7 @@ namespace {
 // bodies, where few units per block are left (N = 3000: 35 against 43 us).
 template <int P, bool UM_>
 struct Dd {
-    static constexpr int I = 2 * P;
+    static constexpr int I = 2 * P, JL = 1;
     static constexpr bool UM = UM_, JSUM = true, SELF = false;
     static constexpr int ACC = 0, FOLD_CHUNKS = 1;
     static constexpr int MINB = P == 1 ? 3 : 2;
@@ -40,7 +40,7 @@ struct Dd {
     };
 
     struct Stage {
-        float4 xy[2 * SCH], zm[2 * SCH], lxy[2 * SCH], lzm[2 * SCH];
+        float4 xy[64], zm[64], lxy[64], lzm[64];
     };
     struct Pre {
         float x, y, z, m, lx, ly, lz, lm;
@@ -67,7 +67,7 @@ struct Dd {
     {
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
-            const int e = lane + h * SCH;
+            const int e = lane + h * 32;
             st.xy[e] = make_float4(p.x, p.x, p.y, p.y);
             st.zm[e] = make_float4(p.z, p.z, p.m, p.m);
             st.lxy[e] = make_float4(p.lx, p.lx, p.ly, p.ly);
@@ -157,7 +157,7 @@ struct Dd {
         {
             return ((double)h.x + (double)h.y) + ((double)l.x + (double)l.y);
         }
-        __device__ __forceinline__ double get(int c) const
+        __device__ __forceinline__ double get(int c, int) const
         {
             return c == 0 ? both(xh, xl) : c == 1 ? both(yh, yl) : both(zh, zl);
         }
@@ -182,7 +182,7 @@ struct Dd {
         const float2 c32 = make_float2(1.5f, 1.5f), c158 = make_float2(1.875f, 1.875f);
         const int next = (lane + 1) & 31;
 #pragma unroll 4
-        for (int t = 0; t < SCH; ++t) {
+        for (int t = 0; t < 32; ++t) {
             const int e = lane + t;
             const float4 A = st.xy[e], B = st.zm[e], C = st.lxy[e], D = st.lzm[e];
             const float2 xjh = make_float2(A.x, A.y), yjh = make_float2(A.z, A.w);
@@ -288,7 +288,7 @@ struct Dd {
 // half the full sum's pairs, the energy of N = 32768 in 11.8 instead of 25.4 ms.
 template <int I_, bool UM_, bool POT>
 struct F64 {
-    static constexpr int I = I_;
+    static constexpr int I = I_, JL = 1;
     static constexpr bool UM = UM_, JSUM = !POT, SELF = POT;
     static constexpr int ACC = 0, FOLD_CHUNKS = 1 << 30;
     static constexpr int MINB = 4;
@@ -300,7 +300,7 @@ struct F64 {
         __device__ __forceinline__ Eps(float, const double *p) : e2(*p) {}
     };
     struct Stage {
-        double x[2 * SCH], y[2 * SCH], z[2 * SCH], m[UM ? 1 : 2 * SCH];
+        double x[64], y[64], z[64], m[UM ? 1 : 64];
     };
     struct Pre {
         double x, y, z, m;
@@ -321,7 +321,7 @@ struct F64 {
     {
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
-            const int e = lane + h * SCH;
+            const int e = lane + h * 32;
             st.x[e] = p.x;
             st.y[e] = p.y;
             st.z[e] = p.z;
@@ -359,7 +359,7 @@ struct F64 {
     struct JSum {
         double x, y, z;
         __device__ __forceinline__ void zero() { x = y = z = 0.0; }
-        __device__ __forceinline__ double get(int c) const { return c == 0 ? x : c == 1 ? y : z; }
+        __device__ __forceinline__ double get(int c, int) const { return c == 0 ? x : c == 1 ? y : z; }
     };
 
     static __device__ __forceinline__ int32_t groups(int32_t kw) { return kw; }
@@ -370,7 +370,7 @@ struct F64 {
     {
         const int next = (lane + 1) & 31;
 #pragma unroll 2
-        for (int t = 0; t < SCH; ++t) {
+        for (int t = 0; t < 32; ++t) {
             const int e = lane + t;
             const double xj = st.x[e], yj = st.y[e], zj = st.z[e];
             const double mj = UM ? 1.0 : st.m[e];

@@ -232,7 +232,8 @@ int tune_pair(const Pool &P, ClusterSet &C, int precision, const Phys &ph, cudaS
             for (int w : {MAX_WAVES, DEFAULT_WAVES, 2})
                 if (!beside || w >= DEFAULT_WAVES) bs[nb++] = w * occ;
             for (int b = occ; !beside && b >= 1 && b > occ - 4; --b) bs[nb++] = b;
-            for (int jt = TILE; rc == NB_OK && jt >= (scarce ? 32 : TILE); jt /= 2)
+            const int least = !scarce ? TILE : def.pl.d.sym ? sym_jt_least(mode) : 32;
+            for (int jt = TILE; rc == NB_OK && jt >= least; jt /= 2)
             for (int q = 0; q < nb; ++q) {
                 const int b = bs[q];
                 const PairShape s{I, b, jt};
