@@ -275,17 +275,18 @@ struct Dd {
 };
 
 // ---- double precision and potential -------------------------------------------
-// The pair term of pair_fp64_kernel: 3 differences, 3 FMAs, 6 operations for
-// (r^2 + eps^2)^(-3/2), 3 FMAs per side: 18 FP64-pipe operations for two
-// interactions (equal masses), 9 each instead of 15.  The FP64 pipe bounds it:
-// 61 Gpair/s at N = 16384 (59 at 4096) where the full kernel runs 38, one
-// evaluation 7.45 -> 4.67 ms.  One and two bodies per thread run alike at N =
-// 16384; one keeps i-blocks narrow for small systems (N = 1024: 27 against 49
-// us), two halves the j slots of large ones.  POT: the potential
+// The pair term of pair_fp64_kernel: 3 differences, 3 FMAs, 3 operations for
+// (r^2 + eps^2)^(-3/2) (split.cuh), 3 FMAs per side: 15 FP64-pipe operations for
+// two interactions (equal masses) instead of 24.  The FP64 pipe bounds it: 75
+// Gpair/s at N = 16384 (72 at 4096) where the full kernel ran 38 with six
+// operations for the power, one evaluation 7.45 -> 3.83 ms.  One and two bodies
+// per thread run alike at N = 16384; one keeps i-blocks narrow for small systems
+// (N = 1024: 25 against 43 us), two halves the j slots of large ones.  POT: the potential
 // m_j / sqrt(r^2 + eps^2) of eq. 4 summed on the i side alone, each unordered
 // pair once: a pair inside a warp's own row, which both of its bodies
 // evaluate, counts half, so sum_i m_i phi_i is the sum over unordered pairs:
-// half the full sum's pairs, the energy of N = 32768 in 11.8 instead of 25.4 ms.
+// half the full sum's pairs at 10 operations, the energy of N = 32768 in 9.7
+// instead of 25.4 ms.
 template <int I_, bool UM_, bool POT>
 struct F64 {
     static constexpr int I = I_, JL = 1;
@@ -381,9 +382,9 @@ struct F64 {
                 r2 = fma(dy, dy, r2);
                 r2 = fma(dz, dz, r2);
                 if (POT) {
-                    double v = mj * rsqrt_pow<true>(r2);
-                    if (MASK) v = t == 0 && kd == kk ? 0.0 : 0.5 * v;
-                    is.ax[kk] += v;
+                    double ri = rsqrt_pow<true>(r2);
+                    if (MASK && t == 0 && kd == kk) ri = 0.0;
+                    is.ax[kk] = fma(MASK ? 0.5 * mj : mj, ri, is.ax[kk]);
                 } else {
                     double sp = rsqrt_pow<false>(r2);
                     if (MASK && t == 0 && kd == kk) sp = 0.0;

@@ -62,16 +62,21 @@ __device__ __forceinline__ double widen(float f)
 }
 
 // R^(-1/2) (POT) or R^(-3/2) in double for R >= 0, refined from the float
-// estimate y0 = rsqrt.approx(R_f): R_f is R truncated to float and y0 is
-// widened to double, both from their bits (the conversion instructions would
-// run on the FP64 pipe, which bounds the FP64 pair kernel and the kick's
-// field).  With R y0^2 = 1 - v, |v| < 2^-20 (the estimate's error and the
-// truncation's),
-//     R^(-1/2) = y0 (1 + v/2 + 3 v^2 / 8 + O(v^3)),
-//     R^(-3/2) = y0^3 (1 + 3 v / 2 + 15 v^2 / 8 + O(v^3)),
-// the dropped terms below 2^-58 relative; y0^2 is exact (y0 has 24 bits) and
-// v is one fused multiply-add, so 5 or 6 FP64 operations replace the double
-// rsqrt and the cube.  R outside the float range (the padding's 1e300, R = 0,
+// estimate rsqrt.approx(R_f), R_f being R truncated to float from its bits.
+// The FP64 pipe bounds the kernels that call this (2 lanes per SM clock), so it
+// does three operations there and the rest goes to the integer and float pipes:
+//   y0   the estimate rounded to 17 bits, y0 = M 2^k; then M^2 and M^3 are
+//        integers of at most 34 and 51 bits, and y0^2 and y0^3 doubles built
+//        from them exactly;
+//   v    1 - R y0^2, one fused multiply-add: |v| < 2^-15.9, exact to 2^-69;
+//   m    R^(-1/2) = y0 (1 + m), m = v / 2 + v^2 (3/8 + 5/16 v + O(v^2)), or
+//        R^(-3/2) = y0^3 (1 + m), m = 3 v / 2 + v^2 (15/8 + 35/16 v + O(v^2)): the
+//        dropped terms are below 2^-62, and the v^2 term, below 2^-30.8, needs
+//        only float precision.
+// Within 1.1 and 1.4 units of 2^-53 of the exact powers (emulated); before, with y0 to 24 bits, y0^2
+// and y0^3 and the whole series in double, five and six operations and 1.5 and
+// 3.3 units.  N = 16384 FP64 evaluation 4.65 -> 3.83 ms, energy of N = 32768
+// 11.8 -> 9.7 ms.  R outside the float range (the padding's 1e300, R = 0,
 // non-finite R) takes the library rsqrt.
 template <bool POT>
 __device__ __forceinline__ double rsqrt_pow(double R)
@@ -85,12 +90,38 @@ __device__ __forceinline__ double rsqrt_pow(double R)
     const float rf = __int_as_float(((E - 1023 + 127) << 23) | (int)((b >> 29) & 0x7FFFFFu));
     float yf;
     asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(yf) : "f"(rf));
-    const double y0 = widen(yf);
-    const double q = __dmul_rn(y0, y0);
-    const double v = __fma_rn(-R, q, 1.0);
-    if (POT) return __fma_rn(y0, __dmul_rn(v, __fma_rn(v, 0.375, 0.5)), y0);
-    const double y3 = __dmul_rn(q, y0);
-    return __fma_rn(y3, __dmul_rn(v, __fma_rn(v, 1.875, 1.5)), y3);
+    const unsigned int yr = (__float_as_uint(yf) + 0x40u) & ~0x7Fu;   // 17 bits, to nearest
+    const unsigned int M = ((yr >> 7) & 0xFFFFu) | 0x10000u;          // y0 = M 2^(ey - 143)
+    const int ey = (int)(yr >> 23);
+    // y0^2: the leading bit of M^2 is 32 or 33
+    const unsigned long long P = (unsigned long long)M * M;
+    const int s2 = (int)(P >> 33);
+    const unsigned long long qb =
+        (P << (20 - s2)) + ((unsigned long long)(2 * ey + 768 + s2) << 52);
+    const double v = __fma_rn(-R, __longlong_as_double((long long)qb), 1.0);
+    // v to float from its bits: v = 0 or 2^-90 < |v| < 2^-15 (its exponent field
+    // is 0x380 to 0x3FF, whose low seven bits are the float's)
+    const unsigned int vh = (unsigned int)((unsigned long long)__double_as_longlong(v) >> 32);
+    const unsigned int vl = (unsigned int)__double_as_longlong(v);
+    const unsigned int vt = __funnelshift_l(vl, vh, 3);
+    const float vf = __uint_as_float((vt & 0x3FFFFFFFu) | (vh & ~0x3FFFFFFFu));
+    const float w = __fmul_rn(__fmul_rn(vf, vf), POT ? __fmaf_rn(vf, 0.3125f, 0.375f)
+                                                     : __fmaf_rn(vf, 2.1875f, 1.875f));
+    // w >= 0 to double from its bits (0 gives 2^-127, of no effect)
+    const unsigned long long wb =
+        ((unsigned long long)__float_as_uint(w) << 29) + ((unsigned long long)896 << 52);
+    const double m = __fma_rn(POT ? 0.5 : 1.5, v, __longlong_as_double((long long)wb));
+    unsigned long long yb;
+    if (POT) {
+        yb = ((unsigned long long)yr << 29) + ((unsigned long long)896 << 52);
+    } else {
+        // y0^3: the leading bit of M^3 is 48, 49 or 50
+        const unsigned long long Q = P * M;
+        const int lz = __clz((int)(Q >> 32));   // 15, 14 or 13
+        yb = (Q << (lz - 11)) + ((unsigned long long)(3 * ey + 656 - lz) << 52);
+    }
+    const double y = __longlong_as_double((long long)yb);
+    return __fma_rn(y, m, y);
 }
 
 }  // namespace nb
