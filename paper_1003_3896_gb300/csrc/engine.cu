@@ -729,8 +729,11 @@ int enq_force(const Pool &P, const ClusterSet &C, const Plan &pl, const Phys &ph
     return NB_OK;
 }
 
+bool ahead_ok(const Plan &pl) { return !float_planes(pl.precision); }
+
 int enq_step(const Pool &P, const ClusterSet &C, const Plan &pl, const Phys &ph, int order,
-             double h, cudaStream_t st, const std::vector<cudaEvent_t> *evs, int64_t *kernels)
+             double h, cudaStream_t st, const std::vector<cudaEvent_t> *evs, int64_t *kernels,
+             bool ahead, bool next)
 {
     const bool sp = float_planes(pl.precision);
     const DevState s = view(P, C, pl);
@@ -752,9 +755,12 @@ int enq_step(const Pool &P, const ClusterSet &C, const Plan &pl, const Phys &ph,
     }
     // drift of the first leapfrog's half step (and the split it feeds, mass
     // words included: the later splits of the step rewrite coordinates only)
-    NB_TRY(launch_kick_drift(s, pl.pl.d, 0.0, 0.5 * wk[0] * h, 0, sp ? (pl.pl.d.sym ? 3 : 2) : 0, ph.ext,
-                             st));
-    count(kernels, 1);
+    const int first_split = pl.pl.d.sym ? 3 : 2, split = pl.pl.d.sym ? 3 : 1;
+    const double hd0 = 0.5 * wk[0] * h;
+    if (!ahead) {
+        NB_TRY(launch_kick_drift(s, pl.pl.d, 0.0, hd0, 0, sp ? first_split : 0, ph.ext, st));
+        count(kernels, 1);
+    }
     for (int k = 0; k < K; ++k) {
         // adjacent half drifts of consecutive leapfrogs merge
         const double hd = 0.5 * (wk[k] + (k + 1 < K ? wk[k + 1] : 0.0)) * h;
@@ -762,8 +768,8 @@ int enq_step(const Pool &P, const ClusterSet &C, const Plan &pl, const Phys &ph,
         cudaEvent_t e0 = evs ? (*evs)[2 * k] : nullptr, e1 = evs ? (*evs)[2 * k + 1] : nullptr;
         int rc = enq_force(P, C, pl, ph, st, e0, e1, kernels);
         if (rc) return rc;
-        NB_TRY(launch_kick_drift(s, pl.pl.d, wk[k] * h, hd, 1, (sp && !last) ? (pl.pl.d.sym ? 3 : 1) : 0, ph.ext,
-                                 st));
+        NB_TRY(launch_kick_drift(s, pl.pl.d, wk[k] * h, hd, 1, sp && !last ? split : 0, ph.ext, st,
+                                 last && next ? hd0 : 0.0));
         count(kernels, 1);
     }
     return NB_OK;

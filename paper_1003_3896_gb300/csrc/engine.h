@@ -211,9 +211,13 @@ int enq_split(const Pool &P, const ClusterSet &C, const Plan &pl, const Phys &ph
 int enq_force(const Pool &P, const ClusterSet &C, const Plan &pl, const Phys &ph,
               cudaStream_t st, cudaEvent_t ev0, cudaEvent_t ev1, int64_t *kernels);
 // One step of length dt (times each cluster's scale) of order 2 or 6.
-// evs (optional) has 2 events per force evaluation for the pair kernels.
+// evs (optional) has 2 events per force evaluation for the pair kernels.  ahead
+// (only where no split frame is taken between steps, ahead_ok): the step before
+// has made this one's first half drift; next: this one makes the next one's.
 int enq_step(const Pool &P, const ClusterSet &C, const Plan &pl, const Phys &ph, int order,
-             double dt, cudaStream_t st, const std::vector<cudaEvent_t> *evs, int64_t *kernels);
+             double dt, cudaStream_t st, const std::vector<cudaEvent_t> *evs, int64_t *kernels,
+             bool ahead = false, bool next = false);
+bool ahead_ok(const Plan &pl);
 int enq_accel_out(const Pool &P, const ClusterSet &C, const Plan &pl, const Phys &ph,
                   double *out, cudaStream_t st, int64_t *kernels);
 // Energy / momentum per cluster into C.diag.

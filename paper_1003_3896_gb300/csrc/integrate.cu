@@ -499,7 +499,7 @@ __device__ __forceinline__ void sum_slots(const DevState &s, const Decomp &d, co
 template <bool EXT>
 __device__ __forceinline__ void advance(const DevState &s, int32_t k, int64_t i, bool kick,
                                         double ax, double ay, double az, double wk, double wd,
-                                        int do_split, const ExtField &ext)
+                                        double wd2, int do_split, const ExtField &ext)
 {
     const double dt = s.cl.dts[k];
     double x = s.x[i], y = s.y[i], z = s.z[i];
@@ -524,6 +524,12 @@ __device__ __forceinline__ void advance(const DevState &s, int32_t k, int64_t i,
     x += hd * vx;
     y += hd * vy;
     z += hd * vz;
+    if (wd2 != 0.0) {
+        const double h2 = wd2 * dt;
+        x += h2 * vx;
+        y += h2 * vy;
+        z += h2 * vz;
+    }
     s.x[i] = x;
     s.y[i] = y;
     s.z[i] = z;
@@ -538,30 +544,30 @@ __device__ __forceinline__ void advance(const DevState &s, int32_t k, int64_t i,
 // EXT: the external field is on (a separate variant keeps its registers out
 // of the field-free kick).
 template <bool EXT, int SB, bool FP>
-__global__ void kick_drift_kernel(DevState s, Decomp d, double wk, double wd, int do_kick,
-                                  int do_split, ExtField ext, int64_t t0, int64_t t1)
+__global__ void kick_drift_kernel(DevState s, Decomp d, double wk, double wd, double wd2,
+                                  int do_kick, int do_split, ExtField ext, int64_t t0, int64_t t1)
 {
     const int64_t t = t0 + blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (t >= t1) return;
     const BodyRef r = body_at(s.cl, t);
     double ax = 0.0, ay = 0.0, az = 0.0;
     if (do_kick) sum_slots<SB, FP>(s, d, r, t, ax, ay, az);
-    advance<EXT>(s, r.k, r.gi, do_kick, ax, ay, az, wk, wd, do_split, ext);
+    advance<EXT>(s, r.k, r.gi, do_kick, ax, ay, az, wk, wd, wd2, do_split, ext);
 }
 
 // Blocks of at most 128 threads: with ~100 registers a thread, 128-thread
 // blocks pack 20 warps on an SM against 16 for 256 (the kick waits on memory;
 // the ensemble's kick ran 8% faster).
-cudaError_t launch_kick_drift_range(const DevState &s, const Decomp &d, double wk, double wd,
-                                    int do_kick, int do_split, const ExtField &ext, int64_t t0,
-                                    int64_t t1, cudaStream_t st)
+static cudaError_t kick_drift(const DevState &s, const Decomp &d, double wk, double wd, double wd2,
+                              int do_kick, int do_split, const ExtField &ext, int64_t t0,
+                              int64_t t1, cudaStream_t st)
 {
     if (t1 <= t0) return cudaSuccess;
     const int64_t m = t1 - t0;
     const int t = ot_for(m) < 128 ? ot_for(m) : 128;
     const unsigned nb = blocks_for(m, t);
     const bool narrow = d.slots <= 4;   // every i-block has at most 4 slots
-#define NB_KD(E, B, F) kick_drift_kernel<E, B, F><<<nb, t, 0, st>>>(s, d, wk, wd, do_kick, do_split, ext, t0, t1)
+#define NB_KD(E, B, F) kick_drift_kernel<E, B, F><<<nb, t, 0, st>>>(s, d, wk, wd, wd2, do_kick, do_split, ext, t0, t1)
     if (d.fpart) {
         if (ext.on) {
             if (narrow) NB_KD(true, 4, true); else NB_KD(true, 8, true);
@@ -580,9 +586,17 @@ cudaError_t launch_kick_drift_range(const DevState &s, const Decomp &d, double w
 }
 
 cudaError_t launch_kick_drift(const DevState &s, const Decomp &d, double wk, double wd,
-                              int do_kick, int do_split, const ExtField &ext, cudaStream_t st)
+                              int do_kick, int do_split, const ExtField &ext, cudaStream_t st,
+                              double wd2)
 {
-    return launch_kick_drift_range(s, d, wk, wd, do_kick, do_split, ext, 0, s.n, st);
+    return kick_drift(s, d, wk, wd, wd2, do_kick, do_split, ext, 0, s.n, st);
+}
+
+cudaError_t launch_kick_drift_range(const DevState &s, const Decomp &d, double wk, double wd,
+                                    int do_kick, int do_split, const ExtField &ext, int64_t t0,
+                                    int64_t t1, cudaStream_t st)
+{
+    return kick_drift(s, d, wk, wd, 0.0, do_kick, do_split, ext, t0, t1, st);
 }
 
 // Row q of the output: the internal sum plus the field at the body.

@@ -412,9 +412,11 @@ cudaError_t launch_split(const DevState &s, cudaStream_t st);
 // the float planes: do_split 0 no, 1 coordinates only, 2 coordinates and the
 // j-stream mass words (needed once after any load; masses never change),
 // 3 coordinates without the j-stream copies (the symmetric kernels, which
-// read the planes).
+// read the planes).  wd2: a second drift after it, rounded apart (the first half
+// drift of the next step).
 cudaError_t launch_kick_drift(const DevState &s, const Decomp &d, double wk, double wd,
-                              int do_kick, int do_split, const ExtField &ext, cudaStream_t st);
+                              int do_kick, int do_split, const ExtField &ext, cudaStream_t st,
+                              double wd2 = 0.0);
 // The same for linear bodies [t0, t1) only.
 cudaError_t launch_kick_drift_range(const DevState &s, const Decomp &d, double wk, double wd,
                                     int do_kick, int do_split, const ExtField &ext, int64_t t0,

@@ -482,6 +482,16 @@ int nb_server_create(const nb_server_params *p, nb_server **out)
                     rc = set_error(NB_ECUDA, "event creation failed");
         }
     }
+    // load the groups' pair kernels now: a kernel's first use loads its code,
+    // and the scheduler would hold up admissions for it
+    for (int mode : {(int)PM_DS_NEAR, (int)PM_DS_FULL, (int)PM_DD, (int)PM_FP64})
+        for (int I : {1, 2, 4, 8}) {
+            if (!rc && pair_variant_exists(mode, I)) {
+                pair_occupancy(mode, I);
+                if (mode != PM_DS_FULL) sym_occupancy(mode, I);
+            }
+        }
+    if (!rc) potential_occupancy();
     if (!rc) rc = set_create(s->io, 1, cap);
     // uploads and downloads are synchronised by the scheduler thread, which
     // feeds no group while it waits: their pack / unpack kernels go first
