@@ -385,7 +385,28 @@ void block_order(ClusterSet &C, const Decomp &d, int I, bool partial)
     const int64_t G = d.G;
     const double full = (TILE / 32) * (I / 2 + 0.5);
     std::vector<double> cost((size_t)G, 0.0);
-    for (int64_t g = 0; g < G; ++g) {
+    for (int64_t g = 0; g < G && d.sym; ++g)
+        for (int64_t u = d.U(g); u < d.U(g + 1);) {
+            const int32_t k = (int32_t)(std::upper_bound(C.uoff.begin(),
+                                                         C.uoff.begin() + C.K + 1, u) -
+                                        C.uoff.begin()) - 1;
+            const SymRows sr(C.nk[k], d.ipb);
+            const int32_t upt = d.ipb / d.jt;
+            const int32_t b = sr.row_of((u - C.uoff[k]) / upt);
+            const int64_t rf = C.uoff[k] + sr.row_first(b) * upt;
+            const int64_t n = C.nk[k], rem = std::min<int64_t>(d.ipb, n - (int64_t)b * d.ipb);
+            const double rows = (double)rem / TILE;   // of full width, per warp
+            for (; u < d.U(g + 1) && u < rf + (int64_t)sr.row_tiles(b) * upt; ++u) {
+                const int32_t t = (int32_t)(u - rf), delta = t / upt;
+                const int32_t c = b + delta < sr.nb ? b + delta : b + delta - sr.nb;
+                const int64_t j0 = (int64_t)c * d.ipb + (t % upt) * d.jt;
+                const int64_t js = std::max<int64_t>(0, std::min<int64_t>(d.jt, n - j0));
+                // the tile of a block with itself: 10 of 16 rows' worth
+                cost[(size_t)g] += (delta ? 1.0 : 0.625) * rows * (double)((js + 31) / 32 * 32);
+            }
+            cost[(size_t)g] += 16.0 * I;
+        }
+    for (int64_t g = 0; g < G && !d.sym; ++g) {
         int64_t u = d.U(g);
         const int64_t uend = d.U(g + 1);
         double c = 0.0;
@@ -588,7 +609,7 @@ int plan_make(const Pool &P, ClusterSet &C, int precision, cudaStream_t st, Plan
     // slower); in the other modes it made the step 0.5-2.6% faster
     C.bperm_G = -1;
     if (pl.pl.mode != PM_FP64 && pl.pl.mode != PM_DS_NEAR && C.K > 1 && C.K <= PARAM_CLUSTERS &&
-        pl.pl.d.G <= PERM_CAP && !pl.pl.d.sym)
+        pl.pl.d.G <= PERM_CAP && (!pl.pl.d.sym || pl.pl.d.W <= 4 * PERM_CAP))
         block_order(C, pl.pl.d, I, sp_family(pl.pl.mode));
     for (int32_t k = 0; k < C.K; ++k)
         if (C.eps2d[k] == 0.0) pl.pl.d.mask_self = 1;
@@ -705,8 +726,7 @@ int enq_force(const Pool &P, const ClusterSet &C, const Plan &pl, const Phys &ph
     ht.mu = C.mu.data();
     ht.poff = C.poff.data();
     const Decomp &d = pl.pl.d;
-    if (C.bperm_G == d.G && C.bperm_W == d.W && C.bperm_jt == d.jt && C.bperm_ipb == d.ipb &&
-        !d.sym) {
+    if (C.bperm_G == d.G && C.bperm_W == d.W && C.bperm_jt == d.jt && C.bperm_ipb == d.ipb) {
         ht.perm = C.bperm.data();
         ht.nperm = (int32_t)C.bperm.size();
     }

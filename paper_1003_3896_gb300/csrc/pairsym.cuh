@@ -42,9 +42,13 @@ namespace nb {
 constexpr int SWARPS = TILE / 32;   // warps per block
 
 // Per-cluster values by value (kernel parameter): uniform across the block.
+// The widest table also carries the blocks' launch order (nperm = 0: index
+// order).
 template <int KC>
 struct SymTab {
     int32_t K;
+    int32_t nperm;
+    uint16_t perm[KC >= PARAM_CLUSTERS ? PERM_CAP : 1];
     int64_t uoff[KC + 1];
     int64_t boff[KC];
     int64_t poff[KC];
@@ -108,6 +112,19 @@ __device__ __forceinline__ void phase_wait(uint32_t bar, uint32_t parity, int *f
     atomicOr(flag, 2);
 }
 
+// Block of the decomposition that launch position q runs: sets of clusters carry
+// an order by estimated work, largest first (block_order), so that the cheap
+// blocks (ragged rows, tiles of blocks with themselves) set the kernel's tail;
+// units and slots stay with the block's index.  Float-float kernel of 200 clusters
+// of 100 to 1500 bodies 277 -> 266 us, of 48 79 -> 77 us.  For one system such an
+// order changed nothing (16384 bodies 109 -> 112 us).
+template <int KC>
+__device__ __forceinline__ int64_t sym_block(const SymTabOf<KC> &t)
+{
+    if (KC >= PARAM_CLUSTERS && t.nperm > 0) return t.perm[blockIdx.x];
+    return blockIdx.x;
+}
+
 // A: the arithmetic.  It gives
 //   I          bodies per thread; groups(kw): how many groups of them hold bodies
 //   JSUM       whether the j side is summed (not for the potential)
@@ -143,7 +160,7 @@ __global__ void __launch_bounds__(TILE, A::MINB) pair_sym_kernel(
             asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(SWARPS) : "memory");
         __syncthreads();
     }
-    const int64_t g = blockIdx.x;
+    const int64_t g = sym_block<KC>(tab);
     int64_t u = d.U(g);
     const int64_t uend = d.U(g + 1);
     const int32_t upt = d.ipb / d.jt;
@@ -371,6 +388,10 @@ cudaError_t launch_sym(const DevState &s, const PairLaunch &pl, const HostTab &h
     if (KC > 0) {
         if (ht.K > KC) return cudaErrorInvalidValue;
         t.K = ht.K;
+        if (KC >= PARAM_CLUSTERS && ht.perm && ht.nperm == pl.d.G && ht.nperm <= PERM_CAP) {
+            t.nperm = ht.nperm;
+            for (int32_t q = 0; q < ht.nperm; ++q) t.perm[q] = ht.perm[q];
+        }
         for (int32_t q = 0; q < ht.K; ++q) {
             t.uoff[q] = ht.uoff[q];
             t.boff[q] = ht.boff[q];

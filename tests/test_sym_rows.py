@@ -9,7 +9,8 @@ What must hold for every launch the planner can make:
   those bodies' j slots are all written, and by one tile each;
 * no body has more partial sums (j slots plus the blocks of its row) than the
   rows reserved for its cluster, clusters do not overlap, and the rows needed
-  stay within the limit (a violation would write past the storage).
+  stay within the limit (a violation would write past the storage);
+* the launch order of several clusters' blocks is a permutation of the grid.
 """
 import os
 import shutil
@@ -22,7 +23,7 @@ SRC = r"""
 #include <cstdio>
 #include <cstdint>
 #include <vector>
-#include "nb_internal.cuh"
+#include "engine.h"
 
 using namespace nb;
 
@@ -79,6 +80,16 @@ int main()
         if (d.G < (G < d.W ? G : d.W)) ++shrunk;
         for (int64_t g = 0; g < d.G; ++g) bad += d.U(g + 1) <= d.U(g);
         const int64_t upt = ipb / jt;
+        if (K > 1 && d.G <= PERM_CAP) {
+            ClusterSet C;
+            C.K = K;
+            C.nk = nk;
+            C.uoff = uoff;
+            block_order(C, d, I, false);
+            std::vector<char> seen((size_t)d.G, 0);
+            bad += (int64_t)C.bperm.size() != d.G;
+            for (uint16_t g : C.bperm) bad += g >= d.G || seen[g]++;
+        }
         for (int k = 0; k < K; ++k) {
             const SymRows sr(nk[k], ipb);
             const int64_t end = k + 1 < K ? poff[k + 1] : rows;
@@ -106,7 +117,7 @@ def test_symmetric_rows_cover_pairs_and_bound_slots(tmp_path):
     src.write_text(SRC)
     exe = tmp_path / "sym_rows"
     subprocess.run([nvcc, *build.ARCH, "-O2", "-std=c++17", "-I", os.path.join(PKG, "csrc"),
-                    str(src), "-o", str(exe), "-L", os.path.dirname(lib), "-lnbsym",
+                    "-I", os.path.join(ROOT, "include"), str(src), "-o", str(exe), "-L", os.path.dirname(lib), "-lnbsym",
                     "-Xlinker", "-rpath=" + os.path.dirname(lib)], check=True)
     r = subprocess.run([str(exe)], capture_output=True, text=True, timeout=300)
     assert r.returncode == 0, r.stdout + r.stderr
