@@ -129,7 +129,9 @@ typedef struct {
     double L[3];
 } nb_energy_t;
 
-/* Timing of the pair-force kernel while profiling is on (nb_prof_enable). */
+/* Timing of the pair-force kernel while profiling is on (nb_prof_enable).  The
+ * steps of a small system, otherwise one kernel per call, then run as separate
+ * kernels, with the same results. */
 typedef struct {
     int64_t pair_launches;    /* pair-force kernel launches timed */
     double pair_ms;           /* their summed device time, CUDA events */

@@ -749,6 +749,18 @@ int enq_force(const Pool &P, const ClusterSet &C, const Plan &pl, const Phys &ph
     return NB_OK;
 }
 
+int stage_weights(int order, double *w)
+{
+    if (order == 2) {
+        w[0] = 1.0;
+        return 1;
+    }
+    const double w0 = 1.0 - 2.0 * (SI6_W1 + SI6_W2 + SI6_W3);
+    const double seq[7] = {SI6_W3, SI6_W2, SI6_W1, w0, SI6_W1, SI6_W2, SI6_W3};
+    for (int k = 0; k < 7; ++k) w[k] = seq[k];
+    return 7;
+}
+
 bool ahead_ok(const Plan &pl) { return !float_planes(pl.precision); }
 
 int enq_step(const Pool &P, const ClusterSet &C, const Plan &pl, const Phys &ph, int order,
@@ -758,16 +770,7 @@ int enq_step(const Pool &P, const ClusterSet &C, const Plan &pl, const Phys &ph,
     const bool sp = float_planes(pl.precision);
     const DevState s = view(P, C, pl);
     double wk[7];
-    int K;
-    if (order == 2) {
-        K = 1;
-        wk[0] = 1.0;
-    } else {
-        K = 7;
-        const double w0 = 1.0 - 2.0 * (SI6_W1 + SI6_W2 + SI6_W3);
-        const double seq[7] = {SI6_W3, SI6_W2, SI6_W1, w0, SI6_W1, SI6_W2, SI6_W3};
-        for (int k = 0; k < 7; ++k) wk[k] = seq[k];
-    }
+    const int K = stage_weights(order, wk);
     if (sp) {
         const bool near = pl.pl.mode == PM_DS_NEAR;
         NB_TRY(launch_frame(s, ph.near_frac, near, st));

@@ -218,6 +218,17 @@ int enq_step(const Pool &P, const ClusterSet &C, const Plan &pl, const Phys &ph,
              double dt, cudaStream_t st, const std::vector<cudaEvent_t> *evs, int64_t *kernels,
              bool ahead = false, bool next = false);
 bool ahead_ok(const Plan &pl);
+// Kick weights of a step of the given order (2 or 6); their number.
+int stage_weights(int order, double *w);
+// Whole steps of a small system in one kernel (small.cu): whether the set and
+// its plan qualify (one system of at most SMALL_MAX bodies in pure float, or
+// SMALL_MAX_DS in every-pair double-single: small.cu has the reason), and the
+// steps (the bits of enq_step).
+constexpr int SMALL_MAX = 1024, SMALL_MAX_DS = 768;
+constexpr int SMALL_SLOTS = 40;
+bool small_ok(const ClusterSet &C, const Plan &pl);
+int small_steps(const Pool &P, const ClusterSet &C, const Plan &pl, const Phys &ph, int order,
+                double h, int64_t steps, cudaStream_t st);
 int enq_accel_out(const Pool &P, const ClusterSet &C, const Plan &pl, const Phys &ph,
                   double *out, cudaStream_t st, int64_t *kernels);
 // Energy / momentum per cluster into C.diag.

@@ -13,6 +13,7 @@
 #include "arith.cuh"
 #include "nb_internal.cuh"
 #include "split.cuh"
+#include "step.cuh"
 
 namespace nb {
 
@@ -45,30 +46,6 @@ __device__ __forceinline__ BodyRef body_at(const Clusters &c, int64_t t)
     r.li = t - c.noff[r.k];
     r.gi = c.boff[r.k] + r.li;
     return r;
-}
-
-// Acceleration of the smooth field of eq. 3, a = -grad Phi, for the
-// Miyamoto-Nagai disk plus Plummer bulge potential
-//   Phi = -G Md / sqrt(R^2 + (ad + sqrt(z^2 + bd^2))^2) - G Mb / sqrt(r^2 + ab^2).
-// Written with three reciprocal square roots and no division: the FP64 pipe
-// of this part runs at a small fraction of the FP32 rate, and a double
-// division or square root costs several times an rsqrt.
-__device__ __forceinline__ void field_accel(const ExtField &e, double x, double y, double z,
-                                            double &ax, double &ay, double &az)
-{
-    // the inverse square-root powers refined in double from float estimates
-    // (split.cuh: the FP64 pipe carries the kick here)
-    const double R2 = x * x + y * y;
-    const double s2 = z * z + e.bd * e.bd;
-    const double rs = rsqrt_pow<true>(s2);       // 1 / sqrt(z^2 + bd^2)
-    const double q = e.ad + s2 * rs;             // ad + sqrt(z^2 + bd^2)
-    const double kd = e.G * e.Md * rsqrt_pow<false>(R2 + q * q);
-    const double kb = e.G * e.Mb * rsqrt_pow<false>(R2 + z * z + e.ab * e.ab);
-    double kh = 0.0;   // softened central point mass
-    if (e.Mbh > 0) kh = e.G * e.Mbh * rsqrt_pow<false>(R2 + z * z + e.eps2bh);
-    ax = -(kd + kb + kh) * x;
-    ay = -(kd + kb + kh) * y;
-    az = -(kd * q * rs + kb + kh) * z;
 }
 
 __device__ __forceinline__ double field_phi(const ExtField &e, double x, double y, double z)
@@ -205,12 +182,7 @@ __global__ void frame_partial_kernel(DevState s)
     double v[5] = {0, 0, 0, 0, 0};
     for (int64_t t = s.cl.seg_lo[sg] + threadIdx.x; t < s.cl.seg_hi[sg]; t += RT) {
         const int64_t i = base + t;
-        const double m = s.m[i], x = s.x[i], y = s.y[i], z = s.z[i];
-        v[0] += m;
-        v[1] += m * x;
-        v[2] += m * y;
-        v[3] += m * z;
-        v[4] += m * (x * x + y * y + z * z);
+        moment_add(v, s.m[i], s.x[i], s.y[i], s.z[i]);
     }
     block_sum<5>(v, sh);
     if (threadIdx.x == 0)
@@ -224,19 +196,7 @@ __global__ void frame_final_kernel(DevState s, double near_frac)
     cluster_sum<5>(s, v, sh);
     if (threadIdx.x == 0) {
         const int k = blockIdx.x;
-        Frame f;
-        const double M = v[0];
-        const double iM = M > 0 ? 1.0 / M : 0.0;   // one division, four products
-        f.cx = v[1] * iM;
-        f.cy = v[2] * iM;
-        f.cz = v[3] * iM;
-        const double r2 = M > 0 ? v[4] * iM - (f.cx * f.cx + f.cy * f.cy + f.cz * f.cz) : 0.0;
-        f.r2rms = r2 > 0 ? r2 : 0.0;
-        // no near-pair radius yet (set by frame_scale_kernel when the plan
-        // runs the near-pair pass)
-        f.th2 = (float)s.cl.eps2d[k];
-        f.dth = 0.f;
-        f.hx = INFINITY;
+        const Frame f = frame_of(v, s.cl.eps2d[k]);
         s.cl.frame[k] = f;
     }
 }
@@ -505,30 +465,24 @@ __device__ __forceinline__ void advance(const DevState &s, int32_t k, int64_t i,
     double x = s.x[i], y = s.y[i], z = s.z[i];
     double vx = s.vx[i], vy = s.vy[i], vz = s.vz[i];
     if (kick) {
-        if (EXT) {
-            double ex, ey, ez;
-            field_accel(ext, x, y, z, ex, ey, ez);
-            ax += ex;
-            ay += ey;
-            az += ez;
-        }
+        if (EXT) field_accel(ext, x, y, z, ax, ay, az);
         const double hk = wk * dt;
-        vx += hk * ax;
-        vy += hk * ay;
-        vz += hk * az;
+        vx = moved(hk, ax, vx);
+        vy = moved(hk, ay, vy);
+        vz = moved(hk, az, vz);
         s.vx[i] = vx;
         s.vy[i] = vy;
         s.vz[i] = vz;
     }
     const double hd = wd * dt;
-    x += hd * vx;
-    y += hd * vy;
-    z += hd * vz;
+    x = moved(hd, vx, x);
+    y = moved(hd, vy, y);
+    z = moved(hd, vz, z);
     if (wd2 != 0.0) {
         const double h2 = wd2 * dt;
-        x += h2 * vx;
-        y += h2 * vy;
-        z += h2 * vz;
+        x = moved(h2, vx, x);
+        y = moved(h2, vy, y);
+        z = moved(h2, vz, z);
     }
     s.x[i] = x;
     s.y[i] = y;
@@ -604,13 +558,7 @@ __device__ __forceinline__ void put_accel(const DevState &s, const ExtField &ext
                                           int64_t q, double ax, double ay, double az,
                                           double *__restrict__ out)
 {
-    if (ext.on) {
-        double ex, ey, ez;
-        field_accel(ext, s.x[gi], s.y[gi], s.z[gi], ex, ey, ez);
-        ax += ex;
-        ay += ey;
-        az += ez;
-    }
+    if (ext.on) field_accel(ext, s.x[gi], s.y[gi], s.z[gi], ax, ay, az);
     out[3 * q] = ax;
     out[3 * q + 1] = ay;
     out[3 * q + 2] = az;
@@ -731,7 +679,7 @@ __global__ void torque_partial_kernel(DevState s, ExtField ext)
     for (int64_t t = s.cl.seg_lo[sg] + threadIdx.x; t < s.cl.seg_hi[sg]; t += RT) {
         const int64_t i = base + t;
         const double m = s.m[i], x = s.x[i], y = s.y[i], z = s.z[i];
-        double ax, ay, az;
+        double ax = 0.0, ay = 0.0, az = 0.0;
         field_accel(ext, x, y, z, ax, ay, az);
         v[0] += m * (y * az - z * ay);
         v[1] += m * (z * ax - x * az);

@@ -61,6 +61,7 @@ struct nb_ctx {
     std::vector<double> mu_k;      // common mass per cluster (0: masses differ)
     int64_t n = 0;                 // bodies loaded (0: none)
     bool planned = false;
+    bool small = false;            // its steps run in one kernel (small.cu)
     bool split_stale = true;
     std::vector<StepGraph> graphs;
     bool prof_on = false;
@@ -155,6 +156,7 @@ int replan(nb_ctx *c, int64_t n)
         c->set.mu.assign(nk.size(), 0.0);
     rc = plan_make(c->pool, c->set, c->p.precision, c->stream, c->plan);
     if (rc) return rc;
+    c->small = small_ok(c->set, c->plan);
     free_graphs(c);
     c->planned = true;
     c->split_stale = true;
@@ -303,15 +305,8 @@ int nb_abi_version(void) { return NB_ABI_VERSION; }
 int nb_stage_weights(int order, double *w)
 {
     if (!w) return set_error(NB_EINVAL, "w is NULL");
-    if (order == 2) {
-        w[0] = 1.0;
-        return 1;
-    }
-    if (order != 6) return set_error(NB_EINVAL, "order must be 2 or 6");
-    const double w0 = 1.0 - 2.0 * (SI6_W1 + SI6_W2 + SI6_W3);
-    const double seq[7] = {SI6_W3, SI6_W2, SI6_W1, w0, SI6_W1, SI6_W2, SI6_W3};
-    for (int k = 0; k < 7; ++k) w[k] = seq[k];
-    return 7;
+    if (order != 2 && order != 6) return set_error(NB_EINVAL, "order must be 2 or 6");
+    return stage_weights(order, w);
 }
 
 const char *nb_last_error(void) { return last_error(); }
@@ -620,6 +615,13 @@ int nb_step(nb_ctx *c, int order, double dt, int64_t nsteps)
     if (c->n == 0) return set_error(NB_ESTATE, "nb_step before nb_load");
     if (nsteps == 0) return NB_OK;
     DeviceGuard dg(c->p.device);
+    if (c->small && !c->prof_on) {
+        const int rc = small_steps(c->pool, c->set, c->plan, c->phys, order, dt, nsteps, c->stream);
+        if (rc) return rc;
+        NB_TRY(cudaStreamSynchronize(c->stream));
+        c->split_stale = true;
+        return NB_OK;
+    }
     int64_t pairs = 0;
     for (int64_t q = 0; q < c->set.K; ++q) pairs += c->set.nk[q] * c->set.nk[q];
     // consecutive steps of a call share a half drift where no frame is taken
@@ -856,6 +858,7 @@ int nb_tune(nb_ctx *c, int reps, nb_tune_t *out)
         return set_error(rc, "%s", why.c_str());
     }
     c->plan = pl;
+    c->small = small_ok(c->set, c->plan);
     if (out) {
         out->precision = rep.precision;
         out->bodies_per_thread = rep.shape.I;
