@@ -221,12 +221,13 @@ bool ahead_ok(const Plan &pl);
 // Kick weights of a step of the given order (2 or 6); their number.
 int stage_weights(int order, double *w);
 // Whole steps of a small system in one kernel (small.cu): whether the set and
-// its plan qualify (one system of at most SMALL_MAX bodies in pure float, or
-// SMALL_MAX_DS in every-pair double-single: small.cu has the reason), and the
-// steps (the bits of enq_step).
-constexpr int SMALL_MAX = 1024, SMALL_MAX_DS = 768;
+// its plan qualify (one system of at most SMALL_MAX bodies in pure float or
+// every-pair double-single), whether steps of an order gain by it, and the steps
+// (the bits of enq_step).
+constexpr int SMALL_MAX = 1024;
 constexpr int SMALL_SLOTS = 40;
 bool small_ok(const ClusterSet &C, const Plan &pl);
+bool small_order(const ClusterSet &C, const Plan &pl, int order);
 int small_steps(const Pool &P, const ClusterSet &C, const Plan &pl, const Phys &ph, int order,
                 double h, int64_t steps, cudaStream_t st);
 int enq_accel_out(const Pool &P, const ClusterSet &C, const Plan &pl, const Phys &ph,

@@ -364,13 +364,95 @@ cudaError_t launch_split(const DevState &s, cudaStream_t st)
 
 // ---- substep -----------------------------------------------------------------
 
-// SB: slots loaded together (a grid run in waves gives an i-block tens of
+// Sum of a run of slots.  Float-pair partial sums (Decomp::fpart) are added in
+// float-float arithmetic on the FP32 pipes and widened to double from their bits
+// at the end (the conversion instruction runs on the FP64 pipe, 1/77 of the
+// FP32 rate here); others in double.
+template <bool FP>
+struct SlotSum;
+template <>
+struct SlotSum<true> {
+    float hx = 0.f, lx = 0.f, hy = 0.f, ly = 0.f, hz = 0.f, lz = 0.f;
+    __device__ __forceinline__ void add(const SlotSum &o)
+    {
+        ff_add(hx, lx, o.hx, o.lx);
+        ff_add(hy, ly, o.hy, o.ly);
+        ff_add(hz, lz, o.hz, o.lz);
+    }
+    __device__ __forceinline__ void get(double &ax, double &ay, double &az) const
+    {
+        ax = widen(hx) + widen(lx);
+        ay = widen(hy) + widen(ly);
+        az = widen(hz) + widen(lz);
+    }
+};
+template <>
+struct SlotSum<false> {
+    double x = 0.0, y = 0.0, z = 0.0;
+    __device__ __forceinline__ void add(const SlotSum &o)
+    {
+        x += o.x;
+        y += o.y;
+        z += o.z;
+    }
+    __device__ __forceinline__ void get(double &ax, double &ay, double &az) const
+    {
+        ax = x;
+        ay = y;
+        az = z;
+    }
+};
+
+// Slots [k0, k1) in order, four of them loaded together (more would cost resident
+// warps, which hide the memory latency better).
+template <bool FP>
+__device__ __forceinline__ SlotSum<FP> sum_run(const DevState &s, const SlotRun &run, int64_t k0,
+                                               int64_t k1)
+{
+    constexpr int SB = 4;
+    const int64_t ps = run.stride;
+    int64_t at = run.base + 3 * k0 * ps;
+    SlotSum<FP> a;
+    for (; k0 < k1; k0 += SB) {
+        SlotSum<FP> b[SB];
+#pragma unroll
+        for (int q = 0; q < SB; ++q) {
+            if (k0 + q >= k1) continue;
+            if constexpr (FP) {
+                const float2 *p = reinterpret_cast<const float2 *>(s.part) + at;
+                const float2 x = p[0], y = p[ps], z = p[2 * ps];
+                b[q].hx = x.x;
+                b[q].lx = x.y;
+                b[q].hy = y.x;
+                b[q].ly = y.y;
+                b[q].hz = z.x;
+                b[q].lz = z.y;
+            } else {
+                const double *p = s.part + at;
+                b[q].x = p[0];
+                b[q].y = p[ps];
+                b[q].z = p[2 * ps];
+            }
+            at += 3 * ps;
+        }
+#pragma unroll
+        for (int q = 0; q < SB; ++q)
+            if (k0 + q < k1) a.add(b[q]);
+    }
+    return a;
+}
+
+// A body in a close encounter: its whole sum is in corr.
+template <bool FP>
+__device__ __forceinline__ bool is_heavy(const DevState &s, const Decomp &d, int64_t t)
+{
+    return FP && d.sym && s.hv_flag && s.hv_flag[t] && *s.hv_count <= hv_limit(s.n);
+}
+
+// One thread per body (slot_parts = 1).  SB: slots loaded together (a grid run in waves gives an i-block tens of
 // slots; an ensemble of small clusters a few, where a narrower batch keeps
 // registers, and so resident warps, for the memory latency)
-// Float-pair partial sums (Decomp::fpart): added in slot order in
-// float-float arithmetic, SB loads at a time, then widened to double from
-// their bits (the conversion instruction runs on the FP64 pipe, 1/77 of the
-// FP32 rate here).
+// Float-pair partial sums in slot order.
 template <int SB>
 __device__ __forceinline__ void sum_slots_ff(const DevState &s, const SlotRun &run,
                                              double &ax, double &ay, double &az)
@@ -407,8 +489,7 @@ template <int SB, bool FP>
 __device__ __forceinline__ void sum_slots(const DevState &s, const Decomp &d, const BodyRef &r,
                                           int64_t t, double &ax, double &ay, double &az)
 {
-    // a body in a close encounter: its whole sum is in corr
-    if (FP && d.sym && s.hv_flag && s.hv_flag[t] && *s.hv_count <= hv_limit(s.n)) {
+    if (is_heavy<FP>(s, d, t)) {
         ax = s.corr[r.gi];
         ay = s.corr[s.cap + r.gi];
         az = s.corr[2 * s.cap + r.gi];
@@ -454,17 +535,40 @@ __device__ __forceinline__ void sum_slots(const DevState &s, const Decomp &d, co
     }
 }
 
-// One body's update: kick (when kick) by (ax, ay, az) plus the field, drift,
-// split.
-template <bool EXT>
-__device__ __forceinline__ void advance(const DevState &s, int32_t k, int64_t i, bool kick,
+// A body's state and what its update reads besides the sums: a kernel that waits
+// at a barrier for the sums loads them ahead (the others gain nothing by it: at
+// a million bodies the registers it holds cost 2 us of 86).
+struct BodyState {
+    double x, y, z, vx, vy, vz, dt;
+    Frame f;
+};
+__device__ __forceinline__ BodyState load_body(const DevState &s, int32_t k, int64_t i)
+{
+    BodyState b;
+    b.x = s.x[i];
+    b.y = s.y[i];
+    b.z = s.z[i];
+    b.vx = s.vx[i];
+    b.vy = s.vy[i];
+    b.vz = s.vz[i];
+    b.dt = s.cl.dts[k];
+    return b;
+}
+
+// One body's update: kick (KICK) by (ax, ay, az) plus the field, drift, split
+// (AHEAD: in the frame loaded with the state).  TWO: the first half drift of the
+// next step may follow (wd2 not zero; FP64 only, the others take a frame between
+// steps).  What a launch does is fixed at compile time where it can be: every
+// double-precision operation, comparisons included, costs a set of a million
+// bodies 2 us.
+template <bool EXT, bool KICK, bool TWO, bool AHEAD, bool SYM>
+__device__ __forceinline__ void advance(const DevState &s, const BodyState &b, int32_t k, int64_t i,
                                         double ax, double ay, double az, double wk, double wd,
                                         double wd2, int do_split, const ExtField &ext)
 {
-    const double dt = s.cl.dts[k];
-    double x = s.x[i], y = s.y[i], z = s.z[i];
-    double vx = s.vx[i], vy = s.vy[i], vz = s.vz[i];
-    if (kick) {
+    const double dt = b.dt;
+    double x = b.x, y = b.y, z = b.z, vx = b.vx, vy = b.vy, vz = b.vz;
+    if (KICK) {
         if (EXT) field_accel(ext, x, y, z, ax, ay, az);
         const double hk = wk * dt;
         vx = moved(hk, ax, vx);
@@ -478,7 +582,7 @@ __device__ __forceinline__ void advance(const DevState &s, int32_t k, int64_t i,
     x = moved(hd, vx, x);
     y = moved(hd, vy, y);
     z = moved(hd, vz, z);
-    if (wd2 != 0.0) {
+    if (TWO && wd2 != 0.0) {
         const double h2 = wd2 * dt;
         x = moved(h2, vx, x);
         y = moved(h2, vy, y);
@@ -487,26 +591,109 @@ __device__ __forceinline__ void advance(const DevState &s, int32_t k, int64_t i,
     s.x[i] = x;
     s.y[i] = y;
     s.z[i] = z;
-    if (do_split == 3)
-        split_one<false, false>(s, s.cl.frame[k], i, x, y, z);
-    else if (do_split == 2)
-        split_one<true>(s, s.cl.frame[k], i, x, y, z);
-    else if (do_split)
-        split_one<false>(s, s.cl.frame[k], i, x, y, z);
+    const Frame &f = AHEAD ? b.f : s.cl.frame[k];
+    // 1: coordinates, 2: and masses, 3: planes only (the symmetric kernels read no
+    // more).  A branch of its own for each decomposition: with all three in one
+    // kernel the stores of a million bodies took 78 us instead of 57
+    if (SYM) {
+        if (do_split) split_one<false, false>(s, f, i, x, y, z);
+    } else if (do_split == 2) {
+        split_one<true>(s, f, i, x, y, z);
+    } else if (do_split) {
+        split_one<false>(s, f, i, x, y, z);
+    }
 }
 
-// EXT: the external field is on (a separate variant keeps its registers out
-// of the field-free kick).
-template <bool EXT, int SB, bool FP>
-__global__ void kick_drift_kernel(DevState s, Decomp d, double wk, double wd, double wd2,
-                                  int do_kick, int do_split, ExtField ext, int64_t t0, int64_t t1)
+// A drift alone.
+template <bool SYM>
+__global__ void drift_kernel(DevState s, double wd, int do_split, int64_t t0, int64_t t1)
 {
     const int64_t t = t0 + blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (t >= t1) return;
     const BodyRef r = body_at(s.cl, t);
-    double ax = 0.0, ay = 0.0, az = 0.0;
-    if (do_kick) sum_slots<SB, FP>(s, d, r, t, ax, ay, az);
-    advance<EXT>(s, r.k, r.gi, do_kick, ax, ay, az, wk, wd, wd2, do_split, ext);
+    advance<false, false, false, false, SYM>(s, load_body(s, r.k, r.gi), r.k, r.gi, 0.0, 0.0, 0.0,
+                                             0.0, wd, 0.0, do_split, ExtField());
+}
+
+// EXT: the external field is on (a separate variant keeps its registers out
+// of the field-free kick).
+template <bool EXT, int SB, bool FP, bool SYM>
+__global__ void kick_drift_kernel(DevState s, Decomp dd, double wk, double wd, double wd2,
+                                  int do_split, ExtField ext, int64_t t0, int64_t t1)
+{
+    const int64_t t = t0 + blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (t >= t1) return;
+    Decomp d = dd;
+    d.sym = SYM ? 1 : 0;   // the other decomposition's indexing costs registers
+    const BodyRef r = body_at(s.cl, t);
+    double ax, ay, az;
+    sum_slots<SB, FP>(s, d, r, t, ax, ay, az);
+    advance<EXT, true, !FP, false, SYM>(s, load_body(s, r.k, r.gi), r.k, r.gi, ax, ay, az, wk, wd,
+                                        wd2, do_split, ext);
+}
+
+// The sums with a warp per run of slots, 32 bodies per block: true, and the
+// sums, in the first warp.
+template <int NP, bool FP, typename Ahead>
+__device__ __forceinline__ bool split_sum(const DevState &s, const Decomp &d, int64_t t,
+                                          int64_t t1, BodyRef &r, Ahead ahead, double &ax,
+                                          double &ay, double &az)
+{
+    __shared__ SlotSum<FP> part[NP - 1][32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    SlotSum<FP> a;
+    double cx = 0.0, cy = 0.0, cz = 0.0;
+    bool heavy = false;
+    if (t < t1) {
+        r = body_at(s.cl, t);
+        if (w == 0) {
+            ahead(r);
+            heavy = is_heavy<FP>(s, d, t);
+            if (s.corr) {
+                cx = s.corr[r.gi];
+                cy = s.corr[s.cap + r.gi];
+                cz = s.corr[2 * s.cap + r.gi];
+            }
+        }
+        const SlotRun run = slot_run(d, s.cl, r.k, r.li, t, s.pstride);
+        const int64_t c = (run.count + NP - 1) / NP;
+        const int64_t k0 = w * c, k1 = k0 + c < run.count ? k0 + c : run.count;
+        a = sum_run<FP>(s, run, k0, k1);
+        if (w > 0) part[w - 1][lane] = a;
+    }
+    __syncthreads();
+    if (w > 0 || t >= t1) return false;
+    for (int q = 0; q < NP - 1; ++q) a.add(part[q][lane]);
+    ax = ay = az = 0.0;
+    if (!heavy) a.get(ax, ay, az);
+    if (s.corr) {
+        ax += cx;
+        ay += cy;
+        az += cz;
+    }
+    return true;
+}
+
+// Blocks per SM that hold SUM_WARPS warps.
+template <bool EXT, int NP, bool FP, bool SYM>
+__global__ void __launch_bounds__(32 * NP, SUM_WARPS / NP) kick_split_kernel(
+    DevState s, Decomp dd, double wk, double wd, double wd2, int do_split, ExtField ext, int64_t t0,
+    int64_t t1)
+{
+    const int64_t t = t0 + blockIdx.x * (int64_t)32 + (threadIdx.x & 31);
+    Decomp d = dd;
+    d.sym = SYM ? 1 : 0;
+    BodyRef r{};
+    BodyState b{};
+    double ax, ay, az;
+    if (split_sum<NP, FP>(
+            s, d, t, t1, r,
+            [&](const BodyRef &q) {
+                b = load_body(s, q.k, q.gi);
+                if (do_split) b.f = s.cl.frame[q.k];
+            },
+            ax, ay, az))
+        advance<EXT, true, !FP, true, SYM>(s, b, r.k, r.gi, ax, ay, az, wk, wd, wd2, do_split, ext);
 }
 
 // Blocks of at most 128 threads: with ~100 registers a thread, 128-thread
@@ -520,21 +707,49 @@ static cudaError_t kick_drift(const DevState &s, const Decomp &d, double wk, dou
     const int64_t m = t1 - t0;
     const int t = ot_for(m) < 128 ? ot_for(m) : 128;
     const unsigned nb = blocks_for(m, t);
-    const bool narrow = d.slots <= 4;   // every i-block has at most 4 slots
-#define NB_KD(E, B, F) kick_drift_kernel<E, B, F><<<nb, t, 0, st>>>(s, d, wk, wd, wd2, do_kick, do_split, ext, t0, t1)
-    if (d.fpart) {
-        if (ext.on) {
-            if (narrow) NB_KD(true, 4, true); else NB_KD(true, 8, true);
-        } else {
-            if (narrow) NB_KD(false, 4, true); else NB_KD(false, 8, true);
-        }
-    } else {
-        if (ext.on) {
-            if (narrow) NB_KD(true, 4, false); else NB_KD(true, 8, false);
-        } else {
-            if (narrow) NB_KD(false, 4, false); else NB_KD(false, 8, false);
-        }
+    if (!do_kick) {
+        if (d.sym)
+            drift_kernel<true><<<nb, t, 0, st>>>(s, wd, do_split, t0, t1);
+        else
+            drift_kernel<false><<<nb, t, 0, st>>>(s, wd, do_split, t0, t1);
+        return cudaGetLastError();
     }
+    const int parts = slot_parts(d, s.n);
+    if (parts > 1) {
+        const unsigned ns = blocks_for(m, 32);
+#define NB_KS(E, P, F, S) kick_split_kernel<E, P, F, S><<<ns, 32 * P, 0, st>>>(s, d, wk, wd, wd2, do_split, ext, t0, t1)
+#define NB_KP(E, F, S) \
+    if (parts == 8) NB_KS(E, 8, F, S); else if (parts == 4) NB_KS(E, 4, F, S); else NB_KS(E, 2, F, S)
+#define NB_KE(F, S) \
+    if (ext.on) { NB_KP(true, F, S); } else { NB_KP(false, F, S); }
+        if (d.fpart && d.sym) {
+            NB_KE(true, true)
+        } else if (d.fpart) {
+            NB_KE(true, false)
+        } else if (d.sym) {
+            NB_KE(false, true)
+        } else {
+            NB_KE(false, false)
+        }
+#undef NB_KE
+#undef NB_KP
+#undef NB_KS
+        return cudaGetLastError();
+    }
+    const bool narrow = d.slots <= 4;   // every i-block has at most 4 slots
+#define NB_KD(E, B, F, S) kick_drift_kernel<E, B, F, S><<<nb, t, 0, st>>>(s, d, wk, wd, wd2, do_split, ext, t0, t1)
+#define NB_KB(E, F, S) \
+    if (narrow) NB_KD(E, 4, F, S); else NB_KD(E, 8, F, S)
+    if (d.fpart && d.sym) {
+        if (ext.on) { NB_KB(true, true, true); } else { NB_KB(false, true, true); }
+    } else if (d.fpart) {
+        if (ext.on) { NB_KB(true, true, false); } else { NB_KB(false, true, false); }
+    } else if (d.sym) {
+        if (ext.on) { NB_KB(true, false, true); } else { NB_KB(false, false, true); }
+    } else {
+        if (ext.on) { NB_KB(true, false, false); } else { NB_KB(false, false, false); }
+    }
+#undef NB_KB
 #undef NB_KD
     return cudaGetLastError();
 }
@@ -551,6 +766,32 @@ cudaError_t launch_kick_drift_range(const DevState &s, const Decomp &d, double w
                                     int64_t t1, cudaStream_t st)
 {
     return kick_drift(s, d, wk, wd, 0.0, do_kick, do_split, ext, t0, t1, st);
+}
+
+// Loads the code of the kernels of a field-free step (a kernel's first launch
+// otherwise does, and waits for it).
+cudaError_t load_step_kernels()
+{
+    const void *all[] = {
+        (const void *)frame_partial_kernel, (const void *)frame_final_kernel,
+        (const void *)frame_harmonic_kernel, (const void *)frame_scale_kernel,
+        (const void *)drift_kernel<true>, (const void *)drift_kernel<false>,
+        (const void *)unpack_kernel, (const void *)pack_kernel, (const void *)cluster_map_kernel,
+#define NB_LD(F, S)                                                                              \
+    (const void *)kick_drift_kernel<false, 4, F, S>,                                             \
+        (const void *)kick_drift_kernel<false, 8, F, S>,                                         \
+        (const void *)kick_split_kernel<false, 2, F, S>,                                         \
+        (const void *)kick_split_kernel<false, 4, F, S>,                                         \
+        (const void *)kick_split_kernel<false, 8, F, S>
+        NB_LD(true, true), NB_LD(true, false), NB_LD(false, true), NB_LD(false, false)
+#undef NB_LD
+    };
+    for (const void *f : all) {
+        cudaFuncAttributes at;
+        const cudaError_t e = cudaFuncGetAttributes(&at, f);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
 }
 
 // Row q of the output: the internal sum plus the field at the body.
@@ -578,6 +819,17 @@ __global__ void accel_out_kernel(DevState s, Decomp d, ExtField ext, double *__r
     put_accel(s, ext, r.gi, q, ax, ay, az, out);
 }
 
+template <int NP, bool FP>
+__global__ void __launch_bounds__(32 * NP, SUM_WARPS / NP) accel_split_kernel(
+    DevState s, Decomp d, ExtField ext, double *__restrict__ out, int64_t t0, int64_t t1)
+{
+    const int64_t q = blockIdx.x * (int64_t)32 + (threadIdx.x & 31);
+    BodyRef r{};
+    double ax, ay, az;
+    if (split_sum<NP, FP>(s, d, t0 + q, t1, r, [](const BodyRef &) {}, ax, ay, az))
+        put_accel(s, ext, r.gi, q, ax, ay, az, out);
+}
+
 cudaError_t launch_accel_out(const DevState &s, const Decomp &d, const ExtField &ext,
                              double *out_aos, cudaStream_t st)
 {
@@ -587,6 +839,18 @@ cudaError_t launch_accel_out(const DevState &s, const Decomp &d, const ExtField 
 cudaError_t launch_accel_out_range(const DevState &s, const Decomp &d, const ExtField &ext,
                                    double *out_aos, int64_t t0, int64_t t1, cudaStream_t st)
 {
+    const int parts = slot_parts(d, s.n);
+    if (parts > 1) {
+        const unsigned ns = blocks_for(t1 - t0, 32);
+#define NB_AS(P, F) accel_split_kernel<P, F><<<ns, 32 * P, 0, st>>>(s, d, ext, out_aos, t0, t1)
+        if (d.fpart) {
+            if (parts == 8) NB_AS(8, true); else if (parts == 4) NB_AS(4, true); else NB_AS(2, true);
+        } else {
+            if (parts == 8) NB_AS(8, false); else if (parts == 4) NB_AS(4, false); else NB_AS(2, false);
+        }
+#undef NB_AS
+        return cudaGetLastError();
+    }
     const int t = ot_for(t1 - t0);
     if (d.fpart)
         accel_out_kernel<true><<<blocks_for(t1 - t0, t), t, 0, st>>>(s, d, ext, out_aos, t0, t1);

@@ -265,6 +265,26 @@ __device__ __forceinline__ SlotRun slot_run(const Decomp &d, const Clusters &c, 
     return r;
 }
 
+// Adding up a body's slots is a chain of loads, tens of slots deep where a grid
+// runs in waves: 14 us of a 100 us evaluation of 15360 bodies, 18 of 45 at 2587
+// in float-float.  Rows of more than 4 slots are therefore added in slot_parts
+// runs of equal length, each in slot order, and the runs' sums in order, a warp
+// per run.
+// As many runs (8, 4, 2) as keep every warp resident at once, SUM_WARPS of them
+// on each of 152 SMs.  Per evaluation (us; one run, 2, 4, 8 runs): mixed mode
+//   N =  2587    24.4   21.9   19.3   17.9
+//   N = 15360   100.2   97.9   95.4  100.5
+//   N = 30720   291.8  286.9  291.2  294.6
+//   N = 65536  1099.8 1106.0 1104.8 1115.0
+// float-float, N = 2587: 45.4, 40.8, 38.2, 37.0.
+constexpr int SUM_WARPS = 24;
+__host__ __device__ __forceinline__ int slot_parts(const Decomp &d, int64_t n)
+{
+    if (d.slots <= 4) return 1;
+    const int64_t w = (n + 31) / 32, most = SUM_WARPS * 152;
+    return 8 * w <= most ? 8 : 4 * w <= most ? 4 : 2 * w <= most ? 2 : 1;
+}
+
 // Bodies in a close encounter.  A float partial sum that holds a large pair
 // term rounds every later term at that term's magnitude, 2^-24 of it: the
 // body's acceleration then carries an error that depends on the order of the
@@ -414,6 +434,8 @@ cudaError_t launch_split(const DevState &s, cudaStream_t st);
 // 3 coordinates without the j-stream copies (the symmetric kernels, which
 // read the planes).  wd2: a second drift after it, rounded apart (the first half
 // drift of the next step).
+cudaError_t load_step_kernels();
+cudaError_t load_near_kernels();
 cudaError_t launch_kick_drift(const DevState &s, const Decomp &d, double wk, double wd,
                               int do_kick, int do_split, const ExtField &ext, cudaStream_t st,
                               double wd2 = 0.0);

@@ -615,7 +615,7 @@ int nb_step(nb_ctx *c, int order, double dt, int64_t nsteps)
     if (c->n == 0) return set_error(NB_ESTATE, "nb_step before nb_load");
     if (nsteps == 0) return NB_OK;
     DeviceGuard dg(c->p.device);
-    if (c->small && !c->prof_on) {
+    if (c->small && small_order(c->set, c->plan, order) && !c->prof_on) {
         const int rc = small_steps(c->pool, c->set, c->plan, c->phys, order, dt, nsteps, c->stream);
         if (rc) return rc;
         NB_TRY(cudaStreamSynchronize(c->stream));

@@ -269,7 +269,8 @@ __global__ void near_rank_kernel(DevState s)
 // correction repeats exactly that and scales by the cluster's mass.
 constexpr int NC_T = 256;   // threads per block of the correction
 
-template <bool UM>
+// HEAVY: bodies in a close encounter are listed.
+template <bool UM, bool HEAVY>
 __global__ void __launch_bounds__(NC_T) near_correct_kernel(DevState s, double G)
 {
     // per thread: the ranges of its 8 probed cells (empty: start = end), so
@@ -371,7 +372,7 @@ __global__ void __launch_bounds__(NC_T) near_correct_kernel(DevState s, double G
             e2 = __fmaf_rn(ey, ey, e2);
             e2 = __fmaf_rn(ez, ez, e2);
             const float re = near_rsqrt(e2);
-            pull = fmaxf(pull, mj * re * re);
+            if (HEAVY) pull = fmaxf(pull, mj * re * re);
             float se = __fmul_rn(re, __fmul_rn(re, re));
             if (!UM) se = __fmul_rn(mj, se);
             ax += (double)__fmul_rn(ex, se) - (double)__fmul_rn(ddx, sf);
@@ -380,7 +381,7 @@ __global__ void __launch_bounds__(NC_T) near_correct_kernel(DevState s, double G
         }
     }
     const int64_t i = s.cl.boff[k] + t - s.cl.noff[k];
-    if (s.hv_flag) {
+    if (HEAVY) {
         const bool heavy = pull > s.cl.frame[k].hx;
         s.hv_flag[t] = heavy ? 1 : 0;
         if (heavy) {
@@ -587,9 +588,41 @@ __global__ void __launch_bounds__(HVT) near_encounter_kernel(DevState s, Heavy h
     }
 }
 
+cudaError_t load_near_kernels()
+{
+    const void *all[] = {(const void *)near_cell_kernel<true>,
+                         (const void *)near_cell_kernel<false>,
+                         (const void *)near_claim_kernel<true>,
+                         (const void *)near_claim_kernel<false>,
+                         (const void *)near_scatter_kernel,
+                         (const void *)near_rank_kernel<true>,
+                         (const void *)near_rank_kernel<false>,
+                         (const void *)near_correct_kernel<true, true>,
+                         (const void *)near_correct_kernel<true, false>,
+                         (const void *)near_correct_kernel<false, true>,
+                         (const void *)near_correct_kernel<false, false>,
+                         (const void *)near_encounter_kernel};
+    for (const void *f : all) {
+        cudaFuncAttributes at;
+        const cudaError_t e = cudaFuncGetAttributes(&at, f);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}
+
 int64_t near_table_size(int64_t n)
 {
     return SLOTS_PER_BODY * n;
+}
+
+template <bool UM>
+static void correct(const DevState &s, double G, bool heavy, cudaStream_t st)
+{
+    const unsigned nb = (unsigned)((s.n + NC_T - 1) / NC_T);
+    if (heavy)
+        near_correct_kernel<UM, true><<<nb, NC_T, 0, st>>>(s, G);
+    else
+        near_correct_kernel<UM, false><<<nb, NC_T, 0, st>>>(s, G);
 }
 
 cudaError_t launch_near_correct(const DevState &s, double G, bool um, cudaStream_t st,
@@ -616,9 +649,9 @@ cudaError_t launch_near_correct(const DevState &s, double G, bool um, cudaStream
         near_rank_kernel<false><<<nbn, 256, 0, st>>>(q);
     }
     if (um)
-        near_correct_kernel<true><<<(unsigned)((s.n + NC_T - 1) / NC_T), NC_T, 0, st>>>(q, G);
+        correct<true>(q, G, list, st);
     else
-        near_correct_kernel<false><<<(unsigned)((s.n + NC_T - 1) / NC_T), NC_T, 0, st>>>(q, G);
+        correct<false>(q, G, list, st);
     if (list) {
         // the scale as the pair kernel forms it: G, times the common mass
         near_encounter_kernel<<<hv->blocks, HVT, 0, st>>>(q, *hv, um ? G * hv->mu : G, um ? 1 : 0);

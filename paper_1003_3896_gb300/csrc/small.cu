@@ -14,17 +14,21 @@
 // packed, and run), folded, scaled, added in run order, the frame's moments by
 // the same tree.  So results do not depend on which path ran a step.
 //
-// What bounds it: up to about 400 bodies the barriers, exchanges and the chain of
-// double-precision operations between them (3.6 to 4.2 us per force evaluation);
-// above, the FP32 pipes of 16 SMs.  Mixed mode, 480 bodies, no field: a call of
-// one leapfrog step 28.3 -> 22.5 us (13 us of it the launch and the return to the
-// host), 64 steps 22.6 -> 9.2 us each, a sixth-order step 78.8 -> 55.5 us.
+// What bounds it: up to about 500 bodies the barriers, exchanges and the chain of
+// double-precision operations between them (4 to 5 us per force evaluation);
+// above, the FP32 pipes of 16 SMs.
 //
-// The lines: with the pair sums on 16 SMs a sixth-order step of the mixed mode
-// takes 78 us against 99 at 640 bodies, 96 against 105 at 777 and 110 against 107
-// at 900 (with the field; 68, 90 and 100 against 83, 95 and 93 without), so
-// SMALL_MAX_DS = 768; pure float, with half the arithmetic, still gains at 1024
-// (92 against 103 us), where the shared memory ends.
+// The lines, measured (us; separate kernels -> here, mixed mode without a field):
+//   bodies   one leapfrog call   64 leapfrogs, each   sixth-order call
+//     384       27.5 -> 22.2        18.2 ->  8.6        71.0 -> 53.0
+//     512       28.0 -> 22.2        18.9 ->  8.9        71.7 -> 54.1
+//     704       29.1 -> 25.5        19.6 -> 11.5        75.9 -> 71.4
+//     768       28.5 -> 26.3        19.6 -> 12.7        74.8 -> 79.3
+//    1024       29.4 -> 29.3        20.0 -> 15.5        76.1 -> 99.4
+// pure float: 1024 leapfrogs 19.5 -> 12.6, sixth order 768 70.5 -> 67.8, 896 73.0
+// -> 75.7.  So leapfrogs up to SMALL_MAX = 1024, where the shared memory ends, and
+// sixth-order steps, which spread the launch and the frame over seven
+// evaluations, up to SMALL_SI6_DS and SMALL_SI6_FP32.
 #include <cooperative_groups.h>
 
 #include "arith.cuh"
@@ -32,6 +36,8 @@
 #include "step.cuh"
 
 namespace nb {
+constexpr int SMALL_SI6_DS = 704, SMALL_SI6_FP32 = 832;
+
 namespace {
 
 namespace cg = cooperative_groups;
@@ -49,7 +55,7 @@ struct SmallShared {
     double tree[5][SRT];
     double mom[SEGS][5];                         // every segment's moments
     int J0[2][SMALL_SLOTS], J1[2][SMALL_SLOTS];  // runs of the (at most two) rows
-    int nrun[2];
+    int nrun[2], c8[2];                          // their number, slots per part
 };
 
 struct SmallArgs {
@@ -67,6 +73,11 @@ struct SmallArgs {
     double Gm;
 };
 
+// q / n for 0 <= q < 4096 and n <= OWN (a multiplication: the quotients are taken
+// in every force evaluation).
+__device__ __forceinline__ unsigned reciprocal(int n) { return n ? ((1u << 20) + n - 1) / n : 0u; }
+__device__ __forceinline__ int over(int q, unsigned r) { return (int)((unsigned)q * r >> 20); }
+
 template <bool FULL, bool UM, bool EXT>
 __global__ void __launch_bounds__(SMT, 1) small_step_kernel(const __grid_constant__ SmallArgs a)
 {
@@ -82,6 +93,7 @@ __global__ void __launch_bounds__(SMT, 1) small_step_kernel(const __grid_constan
     const int i0 = rank * own < n ? rank * own : n, i1 = i0 + own < n ? i0 + own : n;
     const int nown = i1 - i0;
     const float eps2 = a.eps2f;
+    const int np8 = slot_parts(d, n);
     const double dt = a.dt, hstep = a.h;
     const float gh = __double2float_rn(a.Gm), gl = __double2float_rn(a.Gm - (double)gh);
 
@@ -122,7 +134,10 @@ __global__ void __launch_bounds__(SMT, 1) small_step_kernel(const __grid_constan
         }
         const int64_t first = d.owner(u0);
         const int nr = (int)(d.owner(u1 - 1) - first) + 1;   // <= d.slots <= SMALL_SLOTS
-        if (tid == 0) sh.nrun[r] = nr;
+        if (tid == 0) {
+            sh.nrun[r] = nr;
+            sh.c8[r] = (nr + np8 - 1) / np8;
+        }
         if (tid < nr) {
             const int64_t ua = d.U(first + tid), ub = d.U(first + tid + 1);
             sh.J0[r][tid] = (int)(((ua > u0 ? ua : u0) - u0) * d.jt);
@@ -135,6 +150,9 @@ __global__ void __launch_bounds__(SMT, 1) small_step_kernel(const __grid_constan
         cluster.map_shared_rank(&sh, mine ? (i0 + tid) / SEG_BODIES : 0);
     int buf = 0;
     cluster.sync();   // every block of the cluster runs
+    const int np = (nown + 1) / 2, row1 = (row0 + 1) * d.ipb;
+    const unsigned by_np = reciprocal(np), by_nown = reciprocal(nown);
+    const int most = sh.nrun[0] > sh.nrun[1] ? sh.nrun[0] : sh.nrun[1];
 
     for (int64_t step = 0; step < a.steps; ++step) {
         // the frame's moments, a segment per block: 256 threads' sums, then the
@@ -175,11 +193,9 @@ __global__ void __launch_bounds__(SMT, 1) small_step_kernel(const __grid_constan
         for (int k = -1; k < a.stages; ++k) {
             if (k >= 0) {
                 // pair sums: own bodies 2p, 2p + 1 (packed) against one run
-                const int np = (nown + 1) / 2;
-                const int most = sh.nrun[0] > sh.nrun[1] ? sh.nrun[0] : sh.nrun[1];
                 for (int q = tid; q < np * most; q += SMT) {
-                    const int g = q / np, il = 2 * (q - g * np), i = i0 + il;
-                    const int r = i / d.ipb - row0;
+                    const int g = over(q, by_np), il = 2 * (q - g * np), i = i0 + il;
+                    const int r = i >= row1;
                     if (g >= sh.nrun[r]) continue;
                     const int J0 = sh.J0[r][g], J1 = sh.J1[r][g];
                     const bool two = il + 1 < nown;
@@ -252,13 +268,29 @@ __global__ void __launch_bounds__(SMT, 1) small_step_kernel(const __grid_constan
                     }
                 }
                 __syncthreads();
+                // the runs' sums, a thread per body and part (slot_parts)
+                for (int q = tid; q < nown * np8; q += SMT) {
+                    const int p = over(q, by_nown), il = q - p * nown;
+                    const int r = i0 + il >= row1, nr = sh.nrun[r], c8 = sh.c8[r], g0 = p * c8;
+                    if (g0 >= nr) continue;
+                    float h[3] = {0.f, 0.f, 0.f}, l[3] = {0.f, 0.f, 0.f};
+                    for (int g = g0; g < nr && g < g0 + c8; ++g)
+#pragma unroll
+                        for (int c = 0; c < 3; ++c) {
+                            const float2 t = sh.run[c][g][il];
+                            ff_add(h[c], l[c], t.x, t.y);
+                        }
+#pragma unroll
+                    for (int c = 0; c < 3; ++c) sh.run[c][g0][il] = make_float2(h[c], l[c]);
+                }
+                __syncthreads();
             }
             const bool last = k + 1 == a.stages;
             if (mine) {
                 if (k >= 0) {
-                    const int nr = sh.nrun[(i0 + tid) / d.ipb - row0];
+                    const int r = i0 + tid >= row1, nr = sh.nrun[r], c8 = sh.c8[r];
                     float H[3] = {0.f, 0.f, 0.f}, L[3] = {0.f, 0.f, 0.f};
-                    for (int g = 0; g < nr; ++g)
+                    for (int g = 0; g < nr; g += c8)
 #pragma unroll
                         for (int c = 0; c < 3; ++c) {
                             const float2 p = sh.run[c][g][tid];
@@ -305,7 +337,7 @@ __global__ void __launch_bounds__(SMT, 1) small_step_kernel(const __grid_constan
                 }
                 __syncthreads();
                 for (int q = tid; q < nown * SB; q += SMT) {
-                    const int r = q / nown, i = i0 + q - r * nown;
+                    const int r = over(q, by_nown), i = i0 + q - r * nown;
                     if (r == rank) continue;
                     SmallShared *o = cluster.map_shared_rank(&sh, r);
                     o->hi[to][i] = sh.hi[to][i];
@@ -368,14 +400,18 @@ bool fits(Kernel kernel)
 bool small_ok(const ClusterSet &C, const Plan &pl)
 {
     const Decomp &d = pl.pl.d;
-    const int64_t most = pl.pl.mode == PM_FP32 ? SMALL_MAX : SMALL_MAX_DS;
-    if (C.K != 1 || C.n > most || d.sym || d.rows || d.b0 || d.slots > SMALL_SLOTS)
+    if (C.K != 1 || C.n > SMALL_MAX || d.sym || d.rows || d.b0 || d.slots > SMALL_SLOTS)
         return false;
     // a block's bodies lie in at most two rows
     if (d.ipb < OWN || !d.fpart) return false;
     if (pl.pl.mode != PM_DS_FULL && pl.pl.mode != PM_FP32) return false;
     return fits(kernel_of(pl.pl.mode == PM_DS_FULL, pl.pl.um, false)) &&
            fits(kernel_of(pl.pl.mode == PM_DS_FULL, pl.pl.um, true));
+}
+
+bool small_order(const ClusterSet &C, const Plan &pl, int order)
+{
+    return order == 2 || C.n <= (pl.pl.mode == PM_FP32 ? SMALL_SI6_FP32 : SMALL_SI6_DS);
 }
 
 int small_steps(const Pool &P, const ClusterSet &C, const Plan &pl, const Phys &ph, int order,
