@@ -456,9 +456,26 @@ void block_order(ClusterSet &C, const Decomp &d, int I, bool partial)
 // small clusters it is 1e-9 (fewer, larger float partial sums) with encounters
 // in every cluster, and the modes without the near-pair pass do not find their
 // encounters: those keep the full kernels and their results.
+//
+// A small system in double precision and many small clusters in float-float keep
+// the full kernels too: their units (a j range against every body of one row)
+// spread over the GPU where the symmetric ones leave SMs without a unit or run
+// mostly diagonal tiles.  Double precision, one leapfrog (us, full / symmetric):
+// 512 bodies 23.6 / 28.2, 720 25.0 / 36.4, 768 23.6 / 28.3, 800 33.4 / 28.3, 1300
+// 61.9 / 50.1.  Float-float: 100 clusters of 100 to 300 bodies 52.5 / 66.9, 40 and
+// 200 of 100 to 600 53.5 / 56.1 and 134 / 139, 400 of them 230 / 213, 48 of 100 to
+// 800 68 / 68.  (One system of up to 1600 bodies in float-float would gain 4 us of
+// 37 too, but the two kernels' sums differ by 1.2e-14 there, more than a system
+// may differ from itself in a batch.)
 static bool use_sym(const ClusterSet &C, int mode)
 {
-    return mode == PM_FP64 || mode == PM_DD || (mode == PM_DS_NEAR && C.K == 1);
+    if (mode == PM_DS_NEAR) return C.K == 1;
+    if (mode != PM_FP64 && mode != PM_DD) return false;
+    double n2 = 0;
+    for (int32_t k = 0; k < C.K; ++k) n2 += (double)C.nk[k] * (double)C.nk[k];
+    if (mode == PM_FP64) return n2 > 784.0 * 784.0;
+    const double wn = n2 / (double)C.n;
+    return C.K == 1 || (wn > 250 && (wn > 380 || n2 > 5000.0 * 5000.0));
 }
 
 // Bodies per thread without a tuned entry, full decomposition.
