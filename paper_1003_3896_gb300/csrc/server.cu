@@ -93,6 +93,7 @@ constexpr int NGROUPS = 12;               // (FP64, NB_DS, NB_DD) x (order 2, 6)
 // A group's partial sums for the symmetric kernels: a 32nd of the budget, or
 // this many bytes (the full kernels' fixed part) where that is more.
 constexpr double GROUP_PART_LEAST = 67.0e6;
+constexpr int64_t GROUP_PART_WARM = 1 << 24;   // of it at creation
 
 // Bytes of device memory the pool and the group scratch use per body slot:
 // state, float planes, j-stream, near-pair correction, staging, near-pair
@@ -344,6 +345,38 @@ int launch_step(nb_server *s, Group &g)
     return NB_OK;
 }
 
+// A step of one body of no mass in every group, and its upload and download,
+// before the scheduler starts: what a first use costs (partial sums of jobs of a
+// few thousand bodies, allocator, launch paths; 2.3 ms for the first of them in a
+// process) otherwise holds up the first admissions.
+int warm(nb_server *s)
+{
+    Job j;
+    j.d.n = 1;
+    j.d.eps = 1.0;
+    j.off = 0;
+    j.pos.assign(3, 0.0);
+    j.vel.assign(3, 0.0);
+    j.mass.assign(1, 0.0);
+    int rc = upload(s, j);
+    const int64_t off = 0, n = 1;
+    const double one = 1.0;
+    for (Group &g : s->groups) {
+        if (!rc) rc = set_reserve_part(g.set, GROUP_PART_WARM / 8, g.stream);
+        if (!rc) rc = set_define(g.set, 1, &off, &n, &one, &one);
+        g.set.mu.assign(1, 0.0);
+        Plan pl;
+        if (!rc) rc = plan_make(s->pool, g.set, g.precision, g.stream, pl);
+        int64_t k = 0;
+        StepSlot &sl = g.slot[0];
+        if (!rc) rc = enq_step(s->pool, g.set, pl, s->phys, g.order, 1.0, g.stream, &sl.ev, &k);
+        if (!rc) NB_TRY(cudaEventRecord(sl.done, g.stream));
+        if (!rc) NB_TRY(cudaStreamSynchronize(g.stream));
+    }
+    if (!rc) rc = download(s, j);
+    return rc;
+}
+
 void fail_all(nb_server *s, const char *why)
 {
     for (auto &g : s->groups) {
@@ -482,8 +515,10 @@ int nb_server_create(const nb_server_params *p, nb_server **out)
                     rc = set_error(NB_ECUDA, "event creation failed");
         }
     }
-    // load the groups' pair kernels now: a kernel's first use loads its code,
-    // and the scheduler would hold up admissions for it
+    // load the groups' kernels now: a kernel's first use loads its code, and the
+    // scheduler would hold up admissions for it
+    if (!rc && (load_step_kernels() != cudaSuccess || load_near_kernels() != cudaSuccess))
+        rc = set_error(NB_ECUDA, "loading kernels failed");
     for (int mode : {(int)PM_DS_NEAR, (int)PM_DS_FULL, (int)PM_DD, (int)PM_FP64})
         for (int I : {1, 2, 4, 8}) {
             if (!rc && pair_variant_exists(mode, I)) {
@@ -501,6 +536,11 @@ int nb_server_create(const nb_server_params *p, nb_server **out)
                 cudaEventRecord(s->ref, s->io_stream) != cudaSuccess ||
                 cudaEventSynchronize(s->ref) != cudaSuccess))
         rc = set_error(NB_ECUDA, "reference event failed");
+    if (rc) {
+        nb_server_destroy(s);
+        return rc;
+    }
+    rc = warm(s);
     if (rc) {
         nb_server_destroy(s);
         return rc;
