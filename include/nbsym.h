@@ -450,7 +450,8 @@ typedef struct {
                                  about 436 bytes per body slot, plus the
                                  groups' partial sums beyond that share (at
                                  most ~67 MB or a 32nd of the budget,
-                                 whichever is more, per group of the twelve) */
+                                 whichever is more, per group of the twelve;
+                                 17 MB each from the start) */
     int max_jobs;             /* resident jobs at most, 1..65536 */
     double G;                 /* as nb_params */
     int ext_on;

@@ -6,8 +6,9 @@
 // so every block gets the same amount of work whatever the cluster sizes are
 // (one cluster, or an ensemble of uneven clusters in one launch).  Each thread
 // owns I i-bodies and keeps their sums in registers; every pair of each
-// cluster's N x N array is evaluated, as in the paper (Sect. 4.2), not
-// N(N-1)/2.  Clusters of equal masses leave m out of the pair term (scaled in
+// cluster's N x N array is evaluated, as in the paper (Sect. 4.2); pairsym.cuh
+// has the kernels that evaluate each unordered pair once, and use_sym
+// (engine.cu) says which sets take which.  Clusters of equal masses leave m out of the pair term (scaled in
 // afterwards), and in partly filled i-blocks a warp evaluates only the packed
 // i-pairs that hold bodies.
 //
