@@ -8,9 +8,9 @@
 // owns I i-bodies and keeps their sums in registers; every pair of each
 // cluster's N x N array is evaluated, as in the paper (Sect. 4.2); pairsym.cuh
 // has the kernels that evaluate each unordered pair once, and use_sym
-// (engine.cu) says which sets take which.  Clusters of equal masses leave m out of the pair term (scaled in
-// afterwards), and in partly filled i-blocks a warp evaluates only the packed
-// i-pairs that hold bodies.
+// (engine.cu) says which sets take which.  Clusters of equal masses leave m out
+// of the pair term (scaled in afterwards), and in partly filled i-blocks a warp
+// evaluates only the packed i-pairs that hold bodies.
 //
 // Single-precision family (one template, three modes):
 //   PM_DS_NEAR  float pair arithmetic on coordinates relative to the cluster's
