@@ -362,8 +362,8 @@ __global__ void __launch_bounds__(NC_T) near_correct_kernel(DevState s, double G
             if (ee[b] == (int)e0 || !(r2 < th2)) continue;
             const float4 Lj = s.ng_slo[ee[b]];
             const float ri = near_rsqrt(r2);
-            float sf = __fmul_rn(ri, __fmul_rn(ri, ri));
-            if (!UM) sf = __fmul_rn(mj, sf);
+            const float sf = UM ? __fmul_rn(ri, __fmul_rn(ri, ri))
+                                : __fmul_rn(__fmul_rn(mj, ri), __fmul_rn(ri, ri));
             // the same pair with the double-single coordinate difference
             const float ex = __fadd_rn(ddx, __fsub_rn(Lj.x, lxi));
             const float ey = __fadd_rn(ddy, __fsub_rn(Lj.y, lyi));
@@ -373,8 +373,8 @@ __global__ void __launch_bounds__(NC_T) near_correct_kernel(DevState s, double G
             e2 = __fmaf_rn(ez, ez, e2);
             const float re = near_rsqrt(e2);
             if (HEAVY) pull = fmaxf(pull, mj * re * re);
-            float se = __fmul_rn(re, __fmul_rn(re, re));
-            if (!UM) se = __fmul_rn(mj, se);
+            const float se = UM ? __fmul_rn(re, __fmul_rn(re, re))
+                                : __fmul_rn(__fmul_rn(mj, re), __fmul_rn(re, re));
             ax += (double)__fmul_rn(ex, se) - (double)__fmul_rn(ddx, sf);
             ay += (double)__fmul_rn(ey, se) - (double)__fmul_rn(ddy, sf);
             az += (double)__fmul_rn(ez, se) - (double)__fmul_rn(ddz, sf);
@@ -530,8 +530,7 @@ __global__ void __launch_bounds__(HVT) near_encounter_kernel(DevState s, Heavy h
                 r2 = __fmaf_rn(dy, dy, r2);
                 r2 = __fmaf_rn(dz, dz, r2);
                 const float ri = rsqrt_mufu(r2);
-                float sp = __fmul_rn(ri, __fmul_rn(ri, ri));
-                if (!um) sp = __fmul_rn(m[k], sp);
+                float sp = __fmul_rn(um ? ri : __fmul_rn(m[k], ri), __fmul_rn(ri, ri));
                 if (rk[k].x + sl + jj == t) sp = 0.f;   // exactly zero for eps > 0 as well
                 term[gg + k * (HVT / HVS)][jj] = make_float4(dx, dy, dz, sp);
             }

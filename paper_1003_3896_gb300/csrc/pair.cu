@@ -221,8 +221,10 @@ __device__ __forceinline__ void chunk_pass(const float4 (*cb)[4], int j0, int ib
                 r2 = __ffma2_rn(dy, dy, r2);
                 r2 = __ffma2_rn(dz, dz, r2);
                 const float2 ri = make_float2(rsqrt_mufu(r2.x), rsqrt_mufu(r2.y));
-                float2 s = __fmul2_rn(ri, __fmul2_rn(ri, ri));
-                if (!UM) s = __fmul2_rn(mm, s);
+                // the mass on one factor first: 1 / r^3 alone leaves the float
+                // range (r > 4e12) where m / r^3 and m d / r^3 do not
+                float2 s = UM ? __fmul2_rn(ri, __fmul2_rn(ri, ri))
+                              : __fmul2_rn(__fmul2_rn(mm, ri), __fmul2_rn(ri, ri));
                 if (MASK) {
                     const int j = j0 + jj;
                     if (j == ibase + 2 * p * TILE) s.x = 0.f;

@@ -2,7 +2,7 @@
 // close pairs are corrected by near.cu).  The frame is pairsym.cuh.
 //
 // The FP32 FMA pipe bounds it: 14 operations per unordered pair with equal
-// masses (16 with a mass spectrum) cap it at 5.75e12 interactions/s.  At N =
+// masses (17 with a mass spectrum) cap it at 5.75e12 interactions/s.  At N =
 // 65536 it runs 4.1e12 (1.047 ms; the full kernel 1.451 ms at 82% of its cap of
 // 3.66e12), at N = 15360 3.1e12 (76 us).  What is lost is operand supply: a
 // packed FMA with three different register pairs takes the register file more
@@ -152,17 +152,20 @@ struct Sp {
                 r2 = __ffma2_rn(dy, dy, r2);
                 r2 = __ffma2_rn(dz, dz, r2);
                 const float2 ri = make_float2(rsqrt_mufu(r2.x), rsqrt_mufu(r2.y));
-                float2 sp = __fmul2_rn(ri, __fmul2_rn(ri, ri));
+                const float2 q2 = __fmul2_rn(ri, ri);
+                // the masses on one factor first (pair.cu): a shared 1 / r^3 would
+                // save a multiplication, but not its range
+                float2 si = __fmul2_rn(UM ? ri : __fmul2_rn(mm, ri), q2);
                 if (MASK) {
-                    if (t == 0 && kd == p) sp.x = 0.f;
-                    if (t == 0 && kd + 1 == p) sp.y = 0.f;
+                    if (t == 0 && kd == p) si.x = 0.f;
+                    if (t == 0 && kd + 1 == p) si.y = 0.f;
                 }
-                const float2 si = UM ? sp : __fmul2_rn(mm, sp);
                 is.ax[p] = __ffma2_rn(dx, si, is.ax[p]);
                 is.ay[p] = __ffma2_rn(dy, si, is.ay[p]);
                 is.az[p] = __ffma2_rn(dz, si, is.az[p]);
                 if (SYM) {
-                    const float2 sj = UM ? sp : __fmul2_rn(make_float2(is.mi[p], is.mi[p]), sp);
+                    const float2 sj =
+                        UM ? si : __fmul2_rn(__fmul2_rn(make_float2(is.mi[p], is.mi[p]), ri), q2);
                     js.x = __ffma2_rn(dx, sj, js.x);
                     js.y = __ffma2_rn(dy, sj, js.y);
                     js.z = __ffma2_rn(dz, sj, js.z);

@@ -230,8 +230,8 @@ __global__ void __launch_bounds__(SMT, 1) small_step_kernel(const __grid_constan
                             r2 = __ffma2_rn(dy, dy, r2);
                             r2 = __ffma2_rn(dz, dz, r2);
                             const float2 ri = make_float2(rsqrt_mufu(r2.x), rsqrt_mufu(r2.y));
-                            float2 sp = __fmul2_rn(ri, __fmul2_rn(ri, ri));
-                            if (!UM) sp = __fmul2_rn(make_float2(A.w, A.w), sp);
+                            float2 sp = __fmul2_rn(
+                                UM ? ri : __fmul2_rn(make_float2(A.w, A.w), ri), __fmul2_rn(ri, ri));
                             if (d.mask_self) {
                                 if (j == i) sp.x = 0.f;
                                 if (j == i + 1) sp.y = 0.f;
