@@ -79,7 +79,7 @@ enum nb_status {
     NB_ENOMEM = -2,     /* device or host allocation failed */
     NB_ECUDA = -3,      /* a CUDA runtime call failed (message has details) */
     NB_ESTATE = -4,     /* call not valid in the context's state (e.g. step
-                           before load) */
+                           before load, or after one that failed) */
     NB_ETIMEOUT = -5,   /* a bounded device-side wait gave up */
     NB_ENONFINITE = -6  /* result contains NaN/Inf (e.g. coincident particles
                            with eps = 0) */
@@ -171,7 +171,11 @@ void nb_params_default(nb_params *p);
  * body and slot; the kernels that evaluate each pair once use about N / 1024
  * slots, up to 4 GB in all, beyond which, or where the device has no room, the
  * N x N kernels run with a few dozen).  Nothing is allocated by a step or an
- * evaluation.
+ * evaluation.  Where that memory is not to be had (NB_ENOMEM), the context
+ * goes on with the system, precision and parameters that it had; should their
+ * plan not fit again either, or the new system be in place already, it has no
+ * plan, and every call that reads or advances the state returns NB_ESTATE
+ * until a load or change succeeds.
  * *out receives the context.  Errors: NB_EINVAL (bad parameters),
  * NB_ENOMEM, NB_ECUDA. */
 int nb_create(const nb_params *p, int64_t n_capacity, nb_ctx **out);
@@ -193,7 +197,7 @@ int nb_create_batch(const nb_params *p, int64_t n_clusters, const int64_t *sizes
 /* Per-cluster softening eps[k] >= 0 (eq. 4-5) and step scale dt_scale[k] > 0
  * (cluster k advances by dt * dt_scale[k] per nb_step); either array may be
  * NULL to keep the current values.  Arrays have nb_clusters() entries.
- * Errors: NB_EINVAL, NB_ECUDA. */
+ * Errors: NB_EINVAL, NB_ENOMEM, NB_ECUDA. */
 int nb_set_cluster_params(nb_ctx *ctx, const double *eps, const double *dt_scale);
 
 /* Number of clusters (1 for nb_create), or NB_EINVAL for NULL. */
@@ -201,7 +205,7 @@ int64_t nb_clusters(const nb_ctx *ctx);
 
 /* Load a particle system (initial conditions of eq. 3): n rows of positions
  * and velocities, n masses (>= 0, finite).  1 <= n <= capacity.  Host
- * pointers.  Errors: NB_EINVAL, NB_ECUDA. */
+ * pointers.  Errors: NB_EINVAL, NB_ENOMEM, NB_ECUDA. */
 int nb_load(nb_ctx *ctx, int64_t n, const double *pos, const double *vel,
             const double *mass);
 
@@ -252,7 +256,7 @@ int nb_get_state_device(nb_ctx *ctx, double *d_pos, double *d_vel);
 int64_t nb_size(const nb_ctx *ctx);
 
 /* Switch the pair-force arithmetic (enum nb_precision) of a context
- * without reloading; the state is untouched.  Errors: NB_EINVAL. */
+ * without reloading; the state is untouched.  Errors: NB_EINVAL, NB_ENOMEM. */
 int nb_set_precision(nb_ctx *ctx, int precision);
 
 /* Start (on = 1) or stop (on = 0) timing pair-force launches with CUDA

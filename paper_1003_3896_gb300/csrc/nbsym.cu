@@ -130,9 +130,13 @@ void free_graphs(nb_ctx *c)
 }
 
 // (Re)define the cluster set for n bodies and lay it out for the current
-// precision; cached step graphs are dropped.
+// precision.  Cached step graphs are dropped first: a plan may move the set's
+// partial sums.  Where it fails, the context has no plan (ready).
 int replan(nb_ctx *c, int64_t n)
 {
+    free_graphs(c);
+    c->planned = false;
+    c->small = false;
     std::vector<int64_t> boff, nk;
     if (c->batch) {
         int64_t off = 0;
@@ -157,9 +161,35 @@ int replan(nb_ctx *c, int64_t n)
     rc = plan_make(c->pool, c->set, c->p.precision, c->stream, c->plan);
     if (rc) return rc;
     c->small = small_ok(c->set, c->plan);
-    free_graphs(c);
     c->planned = true;
     c->split_stale = true;
+    return NB_OK;
+}
+
+// The same for a loaded context whose state is still that of its c->n bodies:
+// where it fails, `back` puts the parameters back and the context plans again as
+// before, so that it goes on with what it had.
+template <class Back>
+int replan_or_back(nb_ctx *c, int64_t n, Back back)
+{
+    const int rc = replan(c, n);
+    if (rc && c->n > 0) {
+        const std::string why = last_error();
+        back();
+        replan(c, c->n);
+        return set_error(rc, "%s", why.c_str());
+    }
+    return rc;
+}
+
+// Whether `what` may read or launch anything: a system is loaded and its last
+// plan succeeded.
+int ready(const nb_ctx *c, const char *what)
+{
+    if (c->n == 0) return set_error(NB_ESTATE, "%s before nb_load", what);
+    if (!c->planned)
+        return set_error(NB_ESTATE, "%s: the context has no plan (its last load or change of "
+                                    "parameters failed; repeat it)", what);
     return NB_OK;
 }
 
@@ -376,7 +406,7 @@ static int load_common(nb_ctx *c, int64_t n, const double *pos, const double *ve
                          (long long)c->pool.cap);
     DeviceGuard dg(c->p.device);
     if (!c->planned || n != c->n) {
-        int rc = replan(c, n);
+        int rc = replan_or_back(c, n, [] {});
         if (rc) return rc;
     }
     c->n = n;
@@ -434,6 +464,8 @@ int nb_set_cluster_params(nb_ctx *c, const double *eps, const double *dt_scale)
         if (dt_scale && !finite_pos(dt_scale[k]))
             return set_error(NB_EINVAL, "dt_scale[%lld] must be finite and > 0", (long long)k);
     }
+    const std::vector<double> eps0 = c->eps_k, dts0 = c->dts_k;
+    const double e0 = c->p.eps;
     if (eps) {
         c->eps_k.assign(eps, eps + K);
         if (!c->batch) c->p.eps = eps[0];
@@ -441,7 +473,11 @@ int nb_set_cluster_params(nb_ctx *c, const double *eps, const double *dt_scale)
     if (dt_scale) c->dts_k.assign(dt_scale, dt_scale + K);
     if (c->n > 0) {
         DeviceGuard dg(c->p.device);
-        return replan(c, c->n);
+        return replan_or_back(c, c->n, [&] {
+            c->eps_k = eps0;
+            c->dts_k = dts0;
+            c->p.eps = e0;
+        });
     }
     return NB_OK;
 }
@@ -450,7 +486,7 @@ static int accel_common(nb_ctx *c, double *out, bool host)
 {
     if (!c) return set_error(NB_EINVAL, "ctx is NULL");
     if (!out) return set_error(NB_EINVAL, "acc_out is NULL");
-    if (c->n == 0) return set_error(NB_ESTATE, "nb_accel before nb_load");
+    if (const int st = ready(c, "nb_accel")) return st;
     DeviceGuard dg(c->p.device);
     int rc = refresh_split(c);
     if (rc) return rc;
@@ -485,7 +521,7 @@ int nb_accel_device(nb_ctx *c, double *d_acc_out) { return accel_common(c, d_acc
 int nb_accel_range(nb_ctx *c, int64_t i0, int64_t i1, double *acc_out)
 {
     if (!c || !acc_out) return set_error(NB_EINVAL, "NULL argument");
-    if (c->n == 0) return set_error(NB_ESTATE, "nb_accel_range before nb_load");
+    if (const int st = ready(c, "nb_accel_range")) return st;
     if (c->set.K != 1) return set_error(NB_EINVAL, "nb_accel_range takes one cluster");
     if (i0 < 0 || i1 > c->n || i0 >= i1)
         return set_error(NB_EINVAL, "range [%lld, %lld) outside [0, %lld)", (long long)i0,
@@ -528,7 +564,7 @@ int nb_accel_range(nb_ctx *c, int64_t i0, int64_t i1, double *acc_out)
 int nb_substep_range(nb_ctx *c, int64_t i0, int64_t i1, double kick, double drift)
 {
     if (!c) return set_error(NB_EINVAL, "ctx is NULL");
-    if (c->n == 0) return set_error(NB_ESTATE, "nb_substep_range before nb_load");
+    if (const int st = ready(c, "nb_substep_range")) return st;
     if (c->set.K != 1) return set_error(NB_EINVAL, "nb_substep_range takes one cluster");
     if (i0 < 0 || i1 > c->n || i0 >= i1)
         return set_error(NB_EINVAL, "range [%lld, %lld) outside [0, %lld)", (long long)i0,
@@ -574,7 +610,7 @@ int nb_substep_range(nb_ctx *c, int64_t i0, int64_t i1, double kick, double drif
 static int set_state_common(nb_ctx *c, const double *pos, const double *vel, bool host)
 {
     if (!c) return set_error(NB_EINVAL, "ctx is NULL");
-    if (c->n == 0) return set_error(NB_ESTATE, "nb_set_state before nb_load");
+    if (const int st = ready(c, "nb_set_state")) return st;
     if (!pos && !vel) return NB_OK;
     DeviceGuard dg(c->p.device);
     const int64_t n = c->n;
@@ -612,7 +648,7 @@ int nb_step(nb_ctx *c, int order, double dt, int64_t nsteps)
     if (order != 2 && order != 6) return set_error(NB_EINVAL, "order must be 2 or 6");
     if (!finite_pos(dt)) return set_error(NB_EINVAL, "dt must be finite and > 0");
     if (nsteps < 0) return set_error(NB_EINVAL, "nsteps must be >= 0");
-    if (c->n == 0) return set_error(NB_ESTATE, "nb_step before nb_load");
+    if (const int st = ready(c, "nb_step")) return st;
     if (nsteps == 0) return NB_OK;
     DeviceGuard dg(c->p.device);
     if (c->small && small_order(c->set, c->plan, order) && !c->prof_on) {
@@ -667,7 +703,7 @@ int nb_step(nb_ctx *c, int order, double dt, int64_t nsteps)
 
 static int energy_common(nb_ctx *c, std::vector<double> &d)
 {
-    if (c->n == 0) return set_error(NB_ESTATE, "nb_energy before nb_load");
+    if (const int st = ready(c, "nb_energy")) return st;
     DeviceGuard dg(c->p.device);
     NB_TRY(cudaMemsetAsync(c->set.flag, 0, sizeof(int), c->stream));
     int64_t k = 0;
@@ -719,7 +755,7 @@ int nb_torque(nb_ctx *c, double *out)
 {
     if (!c) return set_error(NB_EINVAL, "ctx is NULL");
     if (!out) return set_error(NB_EINVAL, "out is NULL");
-    if (c->n == 0) return set_error(NB_ESTATE, "nb_torque before nb_load");
+    if (const int st = ready(c, "nb_torque")) return st;
     out[0] = out[1] = out[2] = 0.0;
     if (!c->p.ext_on) return NB_OK;
     DeviceGuard dg(c->p.device);
@@ -737,7 +773,7 @@ int nb_torque(nb_ctx *c, double *out)
 static int state_common(nb_ctx *c, double *pos, double *vel, bool host)
 {
     if (!c) return set_error(NB_EINVAL, "ctx is NULL");
-    if (c->n == 0) return set_error(NB_ESTATE, "nb_get_state before nb_load");
+    if (const int st = ready(c, "nb_get_state")) return st;
     if (!pos && !vel) return NB_OK;
     DeviceGuard dg(c->p.device);
     const int64_t n = c->n;
@@ -784,15 +820,16 @@ int nb_set_precision(nb_ctx *c, int precision)
     if (precision < NB_FP64 || precision > NB_DS_NEAR)
         return set_error(NB_EINVAL, "bad precision");
     DeviceGuard dg(c->p.device);
+    const int old = c->p.precision;
     c->p.precision = precision;
-    if (c->n > 0) return replan(c, c->n);
+    if (c->n > 0) return replan_or_back(c, c->n, [&] { c->p.precision = old; });
     return NB_OK;
 }
 
 int nb_accel_symmetric(nb_ctx *c, double *acc_out, double *pair_ms)
 {
     if (!c || !acc_out) return set_error(NB_EINVAL, "NULL argument");
-    if (c->n == 0) return set_error(NB_ESTATE, "nb_accel_symmetric before nb_load");
+    if (const int st = ready(c, "nb_accel_symmetric")) return st;
     if (c->set.K != 1) return set_error(NB_EINVAL, "nb_accel_symmetric takes one cluster");
     DeviceGuard dg(c->p.device);
     const int64_t n = c->n;
@@ -843,7 +880,7 @@ int nb_tune(nb_ctx *c, int reps, nb_tune_t *out)
 {
     if (!c) return set_error(NB_EINVAL, "ctx is NULL");
     if (reps < 1 || reps > 1000) return set_error(NB_EINVAL, "reps must be in [1, 1000]");
-    if (c->n == 0) return set_error(NB_ESTATE, "nb_tune before nb_load");
+    if (const int st = ready(c, "nb_tune")) return st;
     DeviceGuard dg(c->p.device);
     int rc = refresh_split(c);
     if (rc) return rc;

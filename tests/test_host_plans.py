@@ -1,0 +1,111 @@
+"""What a context does when a plan cannot get its device memory, on a stand-in
+for the CUDA runtime (hostcuda.py): no captured graph outlives the memory it was
+captured with, a context whose plan failed goes on with the plan it had or, where
+that fails too, refuses every call that would launch until a plan succeeds."""
+import numpy as np
+import pytest
+
+from hostcuda import Host
+from paper_1003_3896_gb300 import ics
+
+N = 40000   # the double-precision plan's partial sums outgrow those of the others
+
+
+@pytest.fixture(scope="module")
+def host(tmp_path_factory):
+    return Host(tmp_path_factory.mktemp("hostcuda"))
+
+
+@pytest.fixture()
+def ctx(host):
+    host.fail_from()
+    c = host.nbsym.Context(N, eps=1e-2, precision="fp32")
+    c.load(*ics.plummer(N, 1))
+    host.clear()
+    yield c
+    host.fail_from()
+    c.close()
+
+
+def refused(host, f):
+    """f() is NB_ESTATE before any launch."""
+    host.clear()
+    with pytest.raises(host.nbsym.NBError) as e:
+        f()
+    assert e.value.code == host.nbsym.NB_ESTATE
+    assert not host.launches() and host.graphs == 0
+
+
+def test_graphs_do_not_outlive_the_storage(host, ctx):
+    """A change of precision that moves the partial sums, with and without room."""
+    ctx.step(2, 1e-3, 1)
+    ctx.set_precision("fp64")
+    ctx.step(2, 1e-3, 1)
+    ctx.set_precision("fp32")
+    ctx.step(2, 1e-3, 1)
+    assert host.stale == 0
+    ctx.set_precision("ds")
+    ctx.step(6, 1e-3, 2)
+    assert host.stale == 0 and host.ran("pair_sym")
+
+
+def test_no_room_for_symmetric_slots_takes_the_full_kernels(host, ctx):
+    host.fail_from(80 << 20)   # the full kernels' 69 MB still fit
+    ctx.set_precision("fp64")
+    ctx.step(2, 1e-3, 1)
+    assert host.ran("pair_fp64_kernel") and not host.ran("pair_sym")
+    assert host.stale == 0
+
+
+@pytest.mark.parametrize("change", ["precision", "load", "params"])
+def test_failed_plan_leaves_a_usable_or_refusing_context(host, ctx, change):
+    nb = host.nbsym
+    if change == "load":
+        ctx.load(*ics.plummer(N // 4, 1))   # small sums, to outgrow
+    ctx.step(2, 1e-3, 1)
+
+    def again():
+        if change == "precision":
+            ctx.set_precision("fp64")
+        elif change == "load":
+            ctx.set_precision("fp64")
+            ctx.load(*ics.plummer(N, 1))
+        else:
+            ctx.set_precision("fp64")
+            ctx.set_cluster_params(eps=[1e-3])
+
+    host.fail_from(1 << 20)
+    with pytest.raises(nb.NBError) as e:
+        again()
+    assert e.value.code == nb.NB_ENOMEM
+    out = np.empty((ctx.n, 3))
+    for f in (lambda: ctx.step(2, 1e-3, 1), ctx.accel, ctx.energy, ctx.get_state, ctx.torque,
+              lambda: ctx.set_state(pos=out), lambda: ctx.tune(1), ctx.accel_symmetric,
+              lambda: ctx.accel_range(0, 10), lambda: ctx.substep_range(0, 10, 0.1, 0.1)):
+        refused(host, f)
+    host.fail_from()
+    again()
+    host.clear()
+    ctx.step(2, 1e-3, 1)
+    assert host.ran("pair_sym_kernel") and host.stale == 0
+
+
+def test_failed_load_keeps_the_old_system(host):
+    """Room for what the context has (5000 bodies: 15 MB of partial sums), none for
+    what it asks for."""
+    nb = host.nbsym
+    with nb.Context(N, eps=1e-2, precision="fp32") as c:
+        c.load(*ics.plummer(5000, 1))
+        c.step(2, 1e-3, 1)
+        shape = c.pair_shape()
+        host.clear()
+        host.fail_from(20 << 20)
+        try:
+            with pytest.raises(nb.NBError) as e:
+                c.load(*ics.plummer(N, 1))
+            assert e.value.code == nb.NB_ENOMEM
+            assert c.n == 5000 and c.pair_shape() == shape
+            c.step(2, 1e-3, 1)
+            assert host.graphs == 1 and host.stale == 0
+        finally:
+            host.fail_from()
