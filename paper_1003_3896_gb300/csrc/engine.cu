@@ -668,6 +668,31 @@ DevState view(const Pool &P, const ClusterSet &C, const Plan &pl)
     return s;
 }
 
+// A symmetric plan's shape is no measure for these launches: its i-blocks are
+// wider where each unordered pair is evaluated once (float-float from 6144 bodies,
+// double precision from 32768), which here halves the blocks.  The first eighth of
+// 65536 bodies in float-float takes 10.6 ms with 2 bodies per thread, 21.1 with
+// 4; of 32768 in double precision 19.3 with 1, 33.0 with 2.  In the mixed mode the
+// symmetric shape is the narrower one from 2048 to 18432 bodies, and the faster.
+PairLaunch range_launch(const Pool &P, const ClusterSet &C, const Plan &pl, int64_t i0, int64_t i1,
+                        int64_t &W)
+{
+    PairLaunch r = pl.pl;
+    if (pl.pl.d.sym) {
+        r.I = std::min(full_default_I(C, r.mode), sym_default_I(C, r.mode));
+        r.blocks_per_sm = DEFAULT_WAVES * std::max(1, pair_occupancy(r.mode, r.I));
+    }
+    const int ipb = TILE * r.I;
+    const int64_t b0 = i0 / ipb, b1 = (i1 + ipb - 1) / ipb;
+    W = b1 - b0;
+    const int64_t G = std::min((int64_t)P.num_sms * r.blocks_per_sm, W);
+    r.d = make_decomp(W, C.max_ntiles, ipb, G, part_slot_cap(C), TILE, 1);
+    r.d.b0 = b0;
+    r.d.mask_self = pl.pl.d.mask_self;
+    r.d.fpart = pl.pl.d.fpart;
+    return r;
+}
+
 int64_t part_slot_cap(const ClusterSet &C)
 {
     const int64_t per = C.n > 0 ? C.part_elems / (3 * C.n) : MAX_PART_SLOTS;

@@ -193,6 +193,11 @@ struct Phys {
 // plan, when the plan runs the near-pair pass).
 DevState view(const Pool &P, const ClusterSet &C, int precision);
 DevState view(const Pool &P, const ClusterSet &C, const Plan &pl);
+// Launch of the full kernel over the i-block rows of bodies [i0, i1) of a set of
+// one cluster, one block per run of rows (W of them): the sum of a row is done in
+// j order by one block, whatever the range.
+PairLaunch range_launch(const Pool &P, const ClusterSet &C, const Plan &pl, int64_t i0, int64_t i1,
+                        int64_t &W);
 // Pair-kernel family of a plan: the precision's, except that NB_DS on a set
 // of at most DS_FULL_MAX_PAIRS pairs forms the double-single difference on
 // every pair (no near-pair pass).

@@ -529,18 +529,9 @@ int nb_accel_range(nb_ctx *c, int64_t i0, int64_t i1, double *acc_out)
     DeviceGuard dg(c->p.device);
     int rc = refresh_split(c);
     if (rc) return rc;
-    // whole i-block rows of the range, one block per run of rows: each row's
-    // j sum is done in order by one block, as in any other range launch
     const Plan &pl = c->plan;
-    PairLaunch rl = pl.pl;
-    const int ipb = TILE * rl.I;
-    const int64_t b0 = i0 / ipb, b1 = (i1 + ipb - 1) / ipb, W = b1 - b0;
-    int64_t G = (int64_t)c->pool.num_sms * rl.blocks_per_sm;
-    if (G > W) G = W;
-    rl.d = make_decomp(W, c->set.max_ntiles, ipb, G, part_slot_cap(c->set), TILE, 1);
-    rl.d.b0 = b0;
-    rl.d.mask_self = pl.pl.d.mask_self;
-    rl.d.fpart = pl.pl.d.fpart;
+    int64_t W = 0;
+    const PairLaunch rl = range_launch(c->pool, c->set, pl, i0, i1, W);
     const DevState s = view(c->pool, c->set, pl);
     const int64_t uoff[2] = {0, W};
     HostTab ht;
@@ -573,15 +564,8 @@ int nb_substep_range(nb_ctx *c, int64_t i0, int64_t i1, double kick, double drif
         return set_error(NB_EINVAL, "kick and drift must be finite");
     DeviceGuard dg(c->p.device);
     const Plan &pl = c->plan;
-    PairLaunch rl = pl.pl;
-    const int ipb = TILE * rl.I;
-    const int64_t b0 = i0 / ipb, b1 = (i1 + ipb - 1) / ipb, W = b1 - b0;
-    int64_t G = (int64_t)c->pool.num_sms * rl.blocks_per_sm;
-    if (G > W) G = W;
-    rl.d = make_decomp(W, c->set.max_ntiles, ipb, G, part_slot_cap(c->set), TILE, 1);
-    rl.d.b0 = b0;
-    rl.d.mask_self = pl.pl.d.mask_self;
-    rl.d.fpart = pl.pl.d.fpart;
+    int64_t W = 0;
+    const PairLaunch rl = range_launch(c->pool, c->set, pl, i0, i1, W);
     const DevState s = view(c->pool, c->set, pl);
     if (kick != 0.0) {
         // the force evaluation of nb_accel_range (whole i-block rows, each

@@ -109,3 +109,21 @@ def test_failed_load_keeps_the_old_system(host):
             assert host.graphs == 1 and host.stale == 0
         finally:
             host.fail_from()
+
+
+@pytest.mark.parametrize("prec,n,kernel,ipb", [
+    ("dd", 65536, "pair_ff_kernelILi1E", 256), ("dd", 5000, "pair_ff_kernelILi1E", 256),
+    ("fp64", 32768, "pair_fp64_kernelILi1E", 128), ("fp64", 700, "pair_fp64_kernelILi1E", 128),
+    ("ds_near", 15360, "pair_sp_kernelILi2E", 512), ("ds_near", 65536, "pair_sp_kernelILi4E", 1024),
+    ("fp32", 65536, "pair_sp_kernelILi4E", 1024)])
+def test_range_launches_take_the_full_kernels_shape(host, prec, n, kernel, ipb):
+    """An eighth of the bodies: a block per i-block row of the full kernel's own
+    width, not of the symmetric plan's."""
+    host.fail_from()
+    with host.nbsym.Context(n, eps=1e-2, precision=prec) as c:
+        c.load(*ics.plummer(n, 1))
+        for f in (lambda: c.accel_range(0, n // 8), lambda: c.substep_range(0, n // 8, 0.1, 0.1)):
+            host.clear()
+            f()
+            assert [k[1] for k in host.ran(kernel)] == [-(-(n // 8) // ipb)]
+            assert not host.ran("pair_sym")
