@@ -450,32 +450,37 @@ void block_order(ClusterSet &C, const Decomp &d, int I, bool partial)
 }
 
 // Whether a set takes the symmetric kernels, where their slots fit.  The modes
-// of FP64-class accuracy do: the order of their sums moves results by 1e-14.
-// So does the two-pass mixed mode on one system: there the order moves
+// of FP64-class accuracy do: the order of their sums moves results by 1e-14 at
+// most.  So does the two-pass mixed mode on one system: there the order moves
 // velocities by 1e-10 a step (bodies in an encounter apart, Heavy).  On many
 // small clusters it is 1e-9 (fewer, larger float partial sums) with encounters
 // in every cluster, and the modes without the near-pair pass do not find their
 // encounters: those keep the full kernels and their results.
 //
-// A small system in double precision and many small clusters in float-float keep
-// the full kernels too: their units (a j range against every body of one row)
-// spread over the GPU where the symmetric ones leave SMs without a unit or run
-// mostly diagonal tiles.  Double precision, one leapfrog (us, full / symmetric):
-// 512 bodies 23.6 / 28.2, 720 25.0 / 36.4, 768 23.6 / 28.3, 800 33.4 / 28.3, 1300
-// 61.9 / 50.1.  Float-float: 100 clusters of 100 to 300 bodies 52.5 / 66.9, 40 and
-// 200 of 100 to 600 53.5 / 56.1 and 134 / 139, 400 of them 230 / 213, 48 of 100 to
-// 800 68 / 68.  (One system of up to 1600 bodies in float-float would gain 4 us of
-// 37 too, but the two kernels' sums differ by 1.2e-14 there, more than a system
-// may differ from itself in a batch.)
+// Small systems and sets of small clusters keep the full kernels too: a unit of
+// the symmetric kernels (a j range against every body of one row) lasts longer by
+// both sides' sums, and their tiles of an i-block with itself save nothing, which
+// counts until every SM has several units.  Measured, full / symmetric (us):
+//   double precision, one leapfrog: 512 bodies 23.6 / 28.2, 720 25.0 / 36.4, 768
+//   23.6 / 28.3, 800 33.4 / 28.3, 1300 61.9 / 50.1
+//   float-float, one SI6A step: 200 bodies 104 / 133, 1024 110 / 139, 1280 147 /
+//   139; clusters of 400 to 700 bodies, 2 of them 119 / 145; of 600 to 1000, 2
+//   144 / 151; of 300 to 1000, 8 243 / 223; of 300 to 600, 12 183 / 218, 40 396 /
+//   414; of 100 to 900, 40 458 / 434; of 100 to 600, 40 315 / 350, 100 590 / 584,
+//   800 4040 / 3464; of 300 to 400, 400 1909 / 1502; of 100 to 300, 200 433 / 482,
+//   800 1528 / 1659
+//   mixed, explicitly two-pass, one SI6A step: 500 bodies 230 / 279, 4096 324 /
+//   346, 8192 418 / 465, 11000 537 / 544, 12000 593 / 550: from the size on where
+//   NB_DS takes that form
 static bool use_sym(const ClusterSet &C, int mode)
 {
-    if (mode == PM_DS_NEAR) return C.K == 1;
-    if (mode != PM_FP64 && mode != PM_DD) return false;
     double n2 = 0;
     for (int32_t k = 0; k < C.K; ++k) n2 += (double)C.nk[k] * (double)C.nk[k];
+    if (mode == PM_DS_NEAR) return C.K == 1 && n2 > (double)DS_FULL_MAX_PAIRS;
     if (mode == PM_FP64) return n2 > 784.0 * 784.0;
-    const double wn = n2 / (double)C.n;
-    return C.K == 1 || (wn > 250 && (wn > 380 || n2 > 5000.0 * 5000.0));
+    if (mode != PM_DD) return false;
+    const double wn = n2 / (double)C.n;   // mean size, by work
+    return n2 > 1200.0 * 1200.0 && wn > 250 && (wn > 700 || n2 > 3300.0 * 3300.0);
 }
 
 // Bodies per thread without a tuned entry, full decomposition.
@@ -672,16 +677,16 @@ DevState view(const Pool &P, const ClusterSet &C, const Plan &pl)
 // wider where each unordered pair is evaluated once (float-float from 6144 bodies,
 // double precision from 32768), which here halves the blocks.  The first eighth of
 // 65536 bodies in float-float takes 10.6 ms with 2 bodies per thread, 21.1 with
-// 4; of 32768 in double precision 19.3 with 1, 33.0 with 2.  In the mixed mode the
-// symmetric shape is the narrower one from 2048 to 18432 bodies, and the faster.
+// 4; of 32768 in double precision 19.3 with 1, 33.0 with 2.  The mixed mode takes
+// the symmetric kernel's choice where that is the narrower, 2048 to 18432 bodies.
 PairLaunch range_launch(const Pool &P, const ClusterSet &C, const Plan &pl, int64_t i0, int64_t i1,
                         int64_t &W)
 {
     PairLaunch r = pl.pl;
-    if (pl.pl.d.sym) {
-        r.I = std::min(full_default_I(C, r.mode), sym_default_I(C, r.mode));
+    if (pl.pl.d.sym) r.I = full_default_I(C, r.mode);
+    if (r.mode == PM_DS_NEAR) r.I = std::min(r.I, sym_default_I(C, r.mode));
+    if (pl.pl.d.sym || r.I != pl.pl.I)
         r.blocks_per_sm = DEFAULT_WAVES * std::max(1, pair_occupancy(r.mode, r.I));
-    }
     const int ipb = TILE * r.I;
     const int64_t b0 = i0 / ipb, b1 = (i1 + ipb - 1) / ipb;
     W = b1 - b0;

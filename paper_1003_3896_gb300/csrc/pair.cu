@@ -435,6 +435,16 @@ __global__ void __launch_bounds__(TILE, sp_min_blocks(P, MODE)) pair_sp_kernel(
 // operation sum; signed sums keep Knuth's six (ordering them by magnitude
 // costs more issue slots than it saves).  UM (all masses of the cluster
 // equal): 1 / r^3 without m, the caller scales by m.
+//
+// A chunk's 32 terms round their float-float sum at 1e-14 of it in an order of
+// their own; everything after that is double.  So that results do not depend on
+// which kernel a set takes (a system alone the full one, in a batch the symmetric
+// one), the terms are added here in the order of the symmetric kernel: bodies lie
+// over lanes as there (rows of 32 kw consecutive bodies per warp), and lane l
+// takes the chunk's bodies l, l + 1, ... where the symmetric kernel has its row on
+// the i side and l, l - 1, ... where it has it on the j side (the travelling
+// sums).  The two agree to 1e-16 relative; with the bodies of a chunk in index
+// order they differed by 1e-14 to 3e-14.
 
 template <int P>
 struct FFI {
@@ -442,15 +452,18 @@ struct FFI {
     float2 axh[P], axl[P], ayh[P], ayl[P], azh[P], azl[P];   // running sums
 };
 
+// dir: 1 or 31, the step from one of a lane's chunk bodies to the next, mod 32.
+// MASK: the chunk is the thread's own body kd of each lane (met first).
 template <int P, bool MASK, bool UM>
-__device__ __forceinline__ void chunk_pass_ff(const float4 (*cb)[4], int j0, int ibase,
+__device__ __forceinline__ void chunk_pass_ff(const float4 (*cb)[CH], int lane, int dir, int kd,
                                               FFI<P> &q, float2 e2h, float2 e2l)
 {
+    int e = lane;
     const float2 one = make_float2(1.f, 1.f);
     const float2 c32 = make_float2(1.5f, 1.5f), c158 = make_float2(1.875f, 1.875f);
 #pragma unroll 2
-    for (int jj = 0; jj < CH; ++jj) {
-        const float4 A = cb[jj][0], B = cb[jj][1], Cl = cb[jj][2], D = cb[jj][3];
+    for (int t = 0; t < CH; ++t, e = (e + dir) & (CH - 1)) {
+        const float4 A = cb[0][e], B = cb[1][e], Cl = cb[2][e], D = cb[3][e];
         const float2 xjh = make_float2(A.x, A.y), yjh = make_float2(A.z, A.w);
         const float2 zjh = make_float2(B.x, B.y), mjh = make_float2(B.z, B.w);
         const float2 xjl = make_float2(Cl.x, Cl.y), yjl = make_float2(Cl.z, Cl.w);
@@ -497,23 +510,22 @@ __device__ __forceinline__ void chunk_pass_ff(const float4 (*cb)[4], int j0, int
                 ff_mul(mjh, mjl, c3, __ffma2_rn(c3, kv, ce), sh, sl);
             }
             if (MASK) {
-                const int j = j0 + jj;
-                if (j == ibase + 2 * p * TILE) sh.x = sl.x = 0.f;
-                if (j == ibase + (2 * p + 1) * TILE) sh.y = sl.y = 0.f;
+                if (t == 0 && kd == 2 * p) sh.x = sl.x = 0.f;
+                if (t == 0 && kd == 2 * p + 1) sh.y = sl.y = 0.f;
             }
             // a += s d
-            float2 fh, fl, t, te;
+            float2 fh, fl, ts, te;
             ff_mul(sh, sl, dxh, dxl, fh, fl);
-            two_sum2(q.axh[p], fh, t, te);
-            q.axh[p] = t;
+            two_sum2(q.axh[p], fh, ts, te);
+            q.axh[p] = ts;
             q.axl[p] = __fadd2_rn(q.axl[p], __fadd2_rn(te, fl));
             ff_mul(sh, sl, dyh, dyl, fh, fl);
-            two_sum2(q.ayh[p], fh, t, te);
-            q.ayh[p] = t;
+            two_sum2(q.ayh[p], fh, ts, te);
+            q.ayh[p] = ts;
             q.ayl[p] = __fadd2_rn(q.ayl[p], __fadd2_rn(te, fl));
             ff_mul(sh, sl, dzh, dzl, fh, fl);
-            two_sum2(q.azh[p], fh, t, te);
-            q.azh[p] = t;
+            two_sum2(q.azh[p], fh, ts, te);
+            q.azh[p] = ts;
             q.azl[p] = __fadd2_rn(q.azl[p], __fadd2_rn(te, fl));
         }
     }
@@ -528,11 +540,11 @@ __global__ void __launch_bounds__(TILE) pair_ff_kernel(
     double *__restrict__ part, int64_t ps)
 {
     constexpr int I = 2 * P;
-    __shared__ __align__(16) float4 cbuf[WARPS][CH][4];
+    __shared__ __align__(16) float4 cbuf[WARPS][4][CH];
     const int tid = threadIdx.x;
     const int lane = tid & 31;
     const int w = tid >> 5;
-    const float4(*cb)[4] = cbuf[w];
+    const float4(*cb)[CH] = cbuf[w];
     const int64_t g = block_of(tab);
     int64_t u = d.U(g);
     const int64_t uend = d.U(g + 1);
@@ -549,7 +561,16 @@ __global__ void __launch_bounds__(TILE) pair_ff_kernel(
         const float2 e2h = make_float2(e2hf, e2hf), e2l = make_float2(e2lf, e2lf);
         const bool mask_self = d.mask_self != 0;
         const int ib0 = sg.b * d.ipb;
-        const int ibase = ib0 + tid;
+        // the warp's row of 32 kw bodies, as in the symmetric kernel
+        const int rem = n - ib0 < d.ipb ? n - ib0 : d.ipb;
+        const int kw = (rem + TILE - 1) / TILE, rw = 32 * kw;
+        const int r0 = ib0 + w * rw;
+        const bool live = r0 < n;
+        // tiles that have block b on the i side (SymRows::row_tiles, i-blocks being
+        // powers of two)
+        const int ish = __ffs(d.ipb) - 1;
+        const int nb = (n + d.ipb - 1) >> ish;
+        const int ahead = nb / 2 + ((nb & 1) || sg.b < nb / 2 ? 1 : 0);
         const float4 *jdk = jd + 2 * base;
         const float4 *jlk = jl + 2 * base;
 
@@ -562,7 +583,7 @@ __global__ void __launch_bounds__(TILE) pair_ff_kernel(
         for (int k = 0; k < I; ++k) dax[k] = day[k] = daz[k] = 0.0;
 #pragma unroll
         for (int p = 0; p < P; ++p) {
-            const int ia = ibase + 2 * p * TILE, ib = ia + TILE;
+            const int ia = r0 + lane + 64 * p, ib = ia + 32;
             const int64_t ca = base + (ia < n ? ia : n - 1), cb2 = base + (ib < n ? ib : n - 1);
             q.xh[p] = make_float2(xh[ca], xh[cb2]);
             q.yh[p] = make_float2(yh[ca], yh[cb2]);
@@ -583,7 +604,7 @@ __global__ void __launch_bounds__(TILE) pair_ff_kernel(
         }
         for (int jc = J0; jc < J1; jc += CH) {
 #pragma unroll
-            for (int v = 0; v < 4; ++v) cbuf[w][lane][v] = pf[v];
+            for (int v = 0; v < 4; ++v) cbuf[w][v][lane] = pf[v];
             __syncwarp();
             if (jc + CH < J1) {
                 const int j = jc + CH + lane;
@@ -592,11 +613,23 @@ __global__ void __launch_bounds__(TILE) pair_ff_kernel(
                 pf[2] = j < n ? jlk[2 * j] : zero4;
                 pf[3] = j < n ? jlk[2 * j + 1] : zero4;
             }
-            const bool diag = mask_self && jc < ib0 + d.ipb && jc + CH > ib0;
-            if (diag)
-                chunk_pass_ff<P, true, UM>(cb, jc, ibase, q, e2h, e2l);
-            else
-                chunk_pass_ff<P, false, UM>(cb, jc, ibase, q, e2h, e2l);
+            if (live) {
+                // the side that the symmetric kernel has this warp's row on
+                const int bj = jc >> ish;
+                bool iside, own = false;
+                if (bj != sg.b) {
+                    iside = (bj > sg.b ? bj - sg.b : bj - sg.b + nb) < ahead;
+                } else {
+                    const int q = (jc - ib0) / 32;
+                    const int rel = ((P == 1 ? q >> (kw - 1) : q / kw) - w) & (WARPS - 1);
+                    own = rel == 0;
+                    iside = rel <= 1 || (rel == 2 && w < 2);
+                }
+                if (own && mask_self)
+                    chunk_pass_ff<P, true, UM>(cb, lane, 1, (jc - r0) / 32, q, e2h, e2l);
+                else
+                    chunk_pass_ff<P, false, UM>(cb, lane, iside ? 1 : CH - 1, 0, q, e2h, e2l);
+            }
             __syncwarp();
 #pragma unroll
             for (int p = 0; p < P; ++p) {
@@ -613,8 +646,8 @@ __global__ void __launch_bounds__(TILE) pair_ff_kernel(
         const double Gm = UM ? G * (KC > 0 ? tab.mu[sg.k] : c.mu[sg.k]) : G;
 #pragma unroll
         for (int k = 0; k < I; ++k) {
-            const int i = ibase + k * TILE;
-            if (i < n) {
+            const int i = r0 + lane + 32 * k;
+            if (k < kw && i < n) {
                 double *o = part + (sg.slot * 3) * ps + sg.lbase + i;
                 o[0] = Gm * dax[k];
                 o[ps] = Gm * day[k];

@@ -127,3 +127,33 @@ def test_range_launches_take_the_full_kernels_shape(host, prec, n, kernel, ipb):
             f()
             assert [k[1] for k in host.ran(kernel)] == [-(-(n // 8) // ipb)]
             assert not host.ran("pair_sym")
+
+
+def _chosen(host, prec, sizes):
+    host.fail_from()
+    kw = dict(capacity=sizes[0]) if len(sizes) == 1 else dict(sizes=sizes)
+    with host.nbsym.Context(eps=1e-2, precision=prec, **kw) as c:
+        n = sum(sizes)
+        c.load(np.zeros((n, 3)), np.zeros((n, 3)), np.ones(n))
+        host.clear()
+        c.accel()
+        return bool(host.ran("pair_sym"))
+
+
+def test_sizes_of_the_symmetric_kernels_tests_take_them(host):
+    import test_gpu_sym_sizes as t
+    for prec, n in t.SINGLE:
+        assert _chosen(host, prec, [n]), (prec, n)
+    for prec, sizes in t.CLUSTERS:
+        assert _chosen(host, prec, sizes), (prec, len(sizes))
+
+
+@pytest.mark.parametrize("prec,sizes,sym", [
+    ("dd", [64], False), ("dd", [700], False), ("dd", [1200], False), ("dd", [1201], True),
+    ("dd", [400, 700], False), ("dd", [450] * 12, False), ("dd", [450] * 100, True),
+    ("dd", [100] * 1000, False), ("dd", [300, 4100], True), ("fp64", [784], False),
+    ("fp64", [785], True), ("ds_near", [11585], False), ("ds_near", [11586], True), ("ds", [11586], True),
+    ("ds_near", [20000, 3], False), ("fp32", [40000], False), ("ds_full", [40000], False)])
+def test_which_sets_take_the_symmetric_kernels(host, prec, sizes, sym):
+    """Both sides of the lines drawn in use_sym, where each side measured faster."""
+    assert _chosen(host, prec, sizes) == sym
