@@ -806,24 +806,28 @@ __device__ __forceinline__ void put_accel(const DevState &s, const ExtField &ext
     if (!isfinite(ax) || !isfinite(ay) || !isfinite(az)) atomicOr(s.flag, 1);
 }
 
-template <bool FP>
-__global__ void accel_out_kernel(DevState s, Decomp d, ExtField ext, double *__restrict__ out,
+template <bool FP, bool SYM>
+__global__ void accel_out_kernel(DevState s, Decomp dd, ExtField ext, double *__restrict__ out,
                                  int64_t t0, int64_t t1)
 {
     const int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     const int64_t t = t0 + q;
     if (t >= t1) return;
+    Decomp d = dd;
+    d.sym = SYM ? 1 : 0;   // as in kick_drift_kernel
     const BodyRef r = body_at(s.cl, t);
     double ax, ay, az;
     sum_slots<8, FP>(s, d, r, t, ax, ay, az);
     put_accel(s, ext, r.gi, q, ax, ay, az, out);
 }
 
-template <int NP, bool FP>
+template <int NP, bool FP, bool SYM>
 __global__ void __launch_bounds__(32 * NP, SUM_WARPS / NP) accel_split_kernel(
-    DevState s, Decomp d, ExtField ext, double *__restrict__ out, int64_t t0, int64_t t1)
+    DevState s, Decomp dd, ExtField ext, double *__restrict__ out, int64_t t0, int64_t t1)
 {
     const int64_t q = blockIdx.x * (int64_t)32 + (threadIdx.x & 31);
+    Decomp d = dd;
+    d.sym = SYM ? 1 : 0;
     BodyRef r{};
     double ax, ay, az;
     if (split_sum<NP, FP>(s, d, t0 + q, t1, r, [](const BodyRef &) {}, ax, ay, az))
@@ -842,20 +846,27 @@ cudaError_t launch_accel_out_range(const DevState &s, const Decomp &d, const Ext
     const int parts = slot_parts(d, s.n);
     if (parts > 1) {
         const unsigned ns = blocks_for(t1 - t0, 32);
-#define NB_AS(P, F) accel_split_kernel<P, F><<<ns, 32 * P, 0, st>>>(s, d, ext, out_aos, t0, t1)
+#define NB_AS(P, F, S) accel_split_kernel<P, F, S><<<ns, 32 * P, 0, st>>>(s, d, ext, out_aos, t0, t1)
+#define NB_AP(F, S) \
+    if (parts == 8) NB_AS(8, F, S); else if (parts == 4) NB_AS(4, F, S); else NB_AS(2, F, S)
         if (d.fpart) {
-            if (parts == 8) NB_AS(8, true); else if (parts == 4) NB_AS(4, true); else NB_AS(2, true);
+            if (d.sym) { NB_AP(true, true); } else { NB_AP(true, false); }
         } else {
-            if (parts == 8) NB_AS(8, false); else if (parts == 4) NB_AS(4, false); else NB_AS(2, false);
+            if (d.sym) { NB_AP(false, true); } else { NB_AP(false, false); }
         }
+#undef NB_AP
 #undef NB_AS
         return cudaGetLastError();
     }
     const int t = ot_for(t1 - t0);
-    if (d.fpart)
-        accel_out_kernel<true><<<blocks_for(t1 - t0, t), t, 0, st>>>(s, d, ext, out_aos, t0, t1);
-    else
-        accel_out_kernel<false><<<blocks_for(t1 - t0, t), t, 0, st>>>(s, d, ext, out_aos, t0, t1);
+    const unsigned nb = blocks_for(t1 - t0, t);
+#define NB_AO(F, S) accel_out_kernel<F, S><<<nb, t, 0, st>>>(s, d, ext, out_aos, t0, t1)
+    if (d.fpart) {
+        if (d.sym) NB_AO(true, true); else NB_AO(true, false);
+    } else {
+        if (d.sym) NB_AO(false, true); else NB_AO(false, false);
+    }
+#undef NB_AO
     return cudaGetLastError();
 }
 
