@@ -461,7 +461,9 @@ __device__ __forceinline__ void chunk_pass_ff(const float4 (*cb)[CH], int lane, 
     int e = lane;
     const float2 one = make_float2(1.f, 1.f);
     const float2 c32 = make_float2(1.5f, 1.5f), c158 = make_float2(1.875f, 1.875f);
-#pragma unroll 2
+// (four steps: two clusters of 100 to 200 bodies, SI6A step 113.8 us with two of
+// them unrolled, 111.5 with four; from 300 bodies on equal)
+#pragma unroll 4
     for (int t = 0; t < CH; ++t, e = (e + dir) & (CH - 1)) {
         const float4 A = cb[0][e], B = cb[1][e], Cl = cb[2][e], D = cb[3][e];
         const float2 xjh = make_float2(A.x, A.y), yjh = make_float2(A.z, A.w);
