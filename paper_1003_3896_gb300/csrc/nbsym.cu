@@ -21,6 +21,7 @@ struct StepGraph {
     int prof = 0;
     int steps = 1;                 // steps in the graph
     bool ahead = false, next = false;   // half drifts shared with its neighbours (enq_step)
+    int64_t ran = 0;               // steps run by it
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
     std::vector<cudaEvent_t> ev;   // (start, stop) per pair launch when prof
@@ -78,6 +79,17 @@ namespace {
 // more to capture (second order, up to GRAPH_PAIRS pairs).
 constexpr int GRAPH_STEPS = 16;
 constexpr int64_t GRAPH_PAIRS = (int64_t)1 << 26;
+// A graph belongs to one step length, and a program may change it at every call.
+// So the kinds that cost more to capture wait until the steps run at a length, this
+// call's included, have about paid for them: 16-step graphs cost 200 to 290 us and
+// save 2.7 to 4 us a step (300 to 4000 bodies), the two further kinds of shared
+// half drifts 30 (second order) or 90 us (sixth) and save 3.  A new length at every
+// call of 16 steps of 2000 bodies, mixed mode: 618 us with the 16-step graph
+// captured at once, 557 with one step a graph before the symmetric kernels.
+constexpr int64_t LONG_STEPS = 96;
+constexpr int64_t join_steps(int order) { return order == 2 ? 24 : 48; }
+// Step lengths (with their order) whose graphs a context keeps.
+constexpr size_t GRAPH_LENGTHS = 8;
 
 // Largest context whose near-pair pass goes first (create_common).
 constexpr int64_t SIDE_FIRST_CAP = 28672;
@@ -119,13 +131,16 @@ Phys phys_of(const nb_params &p)
     return ph;
 }
 
+void free_graph(StepGraph &g)
+{
+    if (g.exec) cudaGraphExecDestroy(g.exec);
+    if (g.graph) cudaGraphDestroy(g.graph);
+    for (auto e : g.ev) cudaEventDestroy(e);
+}
+
 void free_graphs(nb_ctx *c)
 {
-    for (auto &g : c->graphs) {
-        if (g.exec) cudaGraphExecDestroy(g.exec);
-        if (g.graph) cudaGraphDestroy(g.graph);
-        for (auto e : g.ev) cudaEventDestroy(e);
-    }
+    for (auto &g : c->graphs) free_graph(g);
     c->graphs.clear();
 }
 
@@ -204,6 +219,34 @@ int refresh_split(nb_ctx *c)
     return NB_OK;
 }
 
+bool same_length(const StepGraph &a, const StepGraph &b)
+{
+    return a.order == b.order && a.dt == b.dt && a.prof == b.prof;
+}
+
+// Before the first graph of a further step length: the graphs of the length that
+// came first go, where there are as many as are kept.
+void drop_oldest_length(nb_ctx *c, const StepGraph &add)
+{
+    std::vector<const StepGraph *> lengths;
+    for (const StepGraph &g : c->graphs) {
+        if (same_length(g, add)) return;
+        bool seen = false;
+        for (const StepGraph *q : lengths) seen = seen || same_length(*q, g);
+        if (!seen) lengths.push_back(&g);
+    }
+    if (lengths.size() < GRAPH_LENGTHS) return;
+    const StepGraph old = c->graphs.front();
+    std::vector<StepGraph> keep;
+    for (StepGraph &g : c->graphs) {
+        if (same_length(g, old))
+            free_graph(g);
+        else
+            keep.push_back(std::move(g));
+    }
+    c->graphs.swap(keep);
+}
+
 int get_graph(nb_ctx *c, int order, double h, int steps, bool ahead, bool next, StepGraph **out)
 {
     const int prof = c->prof_on ? 1 : 0;
@@ -247,13 +290,7 @@ int get_graph(nb_ctx *c, int order, double h, int steps, bool ahead, bool next, 
         for (auto ev : g.ev) cudaEventDestroy(ev);
         return set_error(NB_ECUDA, "graph instantiate failed: %s", cudaGetErrorString(e));
     }
-    if (c->graphs.size() >= 16) {
-        auto &old = c->graphs.front();
-        cudaGraphExecDestroy(old.exec);
-        cudaGraphDestroy(old.graph);
-        for (auto ev : old.ev) cudaEventDestroy(ev);
-        c->graphs.erase(c->graphs.begin());
-    }
+    drop_oldest_length(c, g);
     c->graphs.push_back(g);
     *out = &c->graphs.back();
     return NB_OK;
@@ -644,10 +681,14 @@ int nb_step(nb_ctx *c, int order, double dt, int64_t nsteps)
     }
     int64_t pairs = 0;
     for (int64_t q = 0; q < c->set.K; ++q) pairs += c->set.nk[q] * c->set.nk[q];
+    int64_t ran = nsteps;   // steps at this length, this call's included
+    for (const StepGraph &q : c->graphs)
+        if (q.order == order && q.dt == dt && q.prof == (c->prof_on ? 1 : 0)) ran += q.ran;
     // consecutive steps of a call share a half drift where no frame is taken
     // between them (the same two roundings, one kernel fewer)
-    const bool join = ahead_ok(c->plan);
-    const bool several = !c->prof_on && order == 2 && pairs <= GRAPH_PAIRS;
+    const bool join = ahead_ok(c->plan) && ran >= join_steps(order);
+    const bool several =
+        !c->prof_on && order == 2 && pairs <= GRAPH_PAIRS && ran >= LONG_STEPS;
     auto run_of = [&](int64_t k) {
         return several && nsteps - k >= GRAPH_STEPS ? GRAPH_STEPS : 1;
     };
@@ -667,6 +708,7 @@ int nb_step(nb_ctx *c, int order, double dt, int64_t nsteps)
         const int rc = get_graph(c, order, dt, run, join && k > 0, join && k + run < nsteps, &g);
         if (rc) return rc;
         NB_TRY(cudaGraphLaunch(g->exec, c->stream));
+        g->ran += run;
         k += run;
         if (c->prof_on) {
             NB_TRY(cudaStreamSynchronize(c->stream));

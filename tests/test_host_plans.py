@@ -157,3 +157,36 @@ def test_sizes_of_the_symmetric_kernels_tests_take_them(host):
 def test_which_sets_take_the_symmetric_kernels(host, prec, sizes, sym):
     """Both sides of the lines drawn in use_sym, where each side measured faster."""
     assert _chosen(host, prec, sizes) == sym
+
+
+def test_new_step_lengths_capture_one_small_graph_each(host):
+    """A program that changes dt at every call; one that keeps it; several in turn."""
+    host.fail_from()
+    for prec, n in (("fp64", 300), ("fp64", 1024), ("ds", 2000), ("dd", 2000)):
+        with host.nbsym.Context(n, eps=1e-2, precision=prec) as c:
+            c.load(*ics.plummer(n, 1))
+            for order, steps in ((2, 2), (2, 16), (2, 17), (6, 1), (6, 4)):
+                host.clear()
+                for k in range(5):
+                    c.step(order, 1e-3 * (1 + k + 10 * steps), steps)
+                assert host.captures == 5 and host.graphs == 5 * steps
+            # kept: from 96 steps on in graphs of 16
+            host.clear()
+            c.step(2, 1e-4, 64)
+            assert host.graphs == 64
+            host.clear()
+            c.step(2, 1e-4, 64)
+            assert host.graphs == 4
+            host.clear()
+            c.step(2, 1e-4, 64)
+            assert host.graphs == 4 and host.captures == 0
+            host.clear()
+            c.step(2, 2e-4, 100)
+            assert host.graphs == 6 + 4
+            # eight lengths in turn: captured for good
+            for r in range(6):
+                if r == 5:
+                    host.clear()
+                for k in range(8):
+                    c.step(2, 3e-4 * (1 + k), 33)
+            assert host.captures == 0
