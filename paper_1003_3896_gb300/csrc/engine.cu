@@ -161,30 +161,36 @@ int set_create(ClusterSet &C, int32_t kcap, int64_t body_cap, int priority)
     return NB_OK;
 }
 
+// Storage of at least need elements at p (have of them there), grown by half or
+// more: freed and allocated on the stream (ordered) or by the plain calls, which
+// wait for all work of the device.
+template <typename T>
+static int reserve(T *&p, int64_t &have, int64_t need, bool ordered, cudaStream_t st)
+{
+    if (have >= need) return NB_OK;
+    const int64_t want = p ? std::max(need, have * 3 / 2) : need;
+    if (p) {
+        NB_TRY(ordered ? cudaFreeAsync(p, st) : cudaFree(p));
+        p = nullptr;
+        have = 0;
+    }
+    for (const int64_t e : {want, need}) {
+        void *q = nullptr;
+        const size_t bytes = (size_t)e * sizeof(T);
+        if ((ordered ? cudaMallocAsync(&q, bytes, st) : cudaMalloc(&q, bytes)) == cudaSuccess) {
+            p = static_cast<T *>(q);
+            have = e;
+            return NB_OK;
+        }
+        cudaGetLastError();
+    }
+    return set_error(NB_ENOMEM, "partial-sum storage: %lld bytes not available",
+                     (long long)(need * (int64_t)sizeof(T)));
+}
+
 int set_reserve_part(ClusterSet &C, int64_t elems, cudaStream_t st)
 {
-    if (C.part && C.part_elems >= elems) return NB_OK;
-    const int64_t want = C.part ? (elems > C.part_elems * 3 / 2 ? elems : C.part_elems * 3 / 2)
-                                : elems;
-    if (C.part) {
-        NB_TRY(C.part_ordered ? cudaFreeAsync(C.part, st) : cudaFree(C.part));
-        C.part = nullptr;
-        C.part_elems = 0;
-    }
-    void *q = nullptr;
-    for (const int64_t e : {want, elems})
-        if (!q && (C.part_ordered ? cudaMallocAsync(&q, (size_t)e * 8, st)
-                                  : cudaMalloc(&q, (size_t)e * 8)) == cudaSuccess) {
-            C.part_elems = e;
-        } else if (!q) {
-            cudaGetLastError();
-            q = nullptr;
-        }
-    if (!q)
-        return set_error(NB_ENOMEM, "partial-sum storage: %lld bytes not available",
-                         (long long)elems * 8);
-    C.part = static_cast<double *>(q);
-    return NB_OK;
+    return reserve(C.part, C.part_elems, elems, C.part_ordered, st);
 }
 
 void set_destroy(ClusterSet &C)
@@ -513,6 +519,31 @@ static int sym_default_I(const ClusterSet &C, int mode)
     return wn < 6144 ? 2 : 4;   // measured: pairsym_wide.cu
 }
 
+// The search for bodies in a close encounter (Heavy) of a symmetric plan in the
+// mixed mode: the full kernels' untuned decomposition of the set, and storage for
+// the sums.
+static int plan_heavy(const Pool &P, ClusterSet &C, int mode, int waves, cudaStream_t st, Heavy &h)
+{
+    const int fI = full_default_I(C, mode);
+    const int64_t resident = (int64_t)P.num_sms * std::max(1, pair_occupancy(mode, fI));
+    const int64_t ib = (C.n + TILE * fI - 1) / (TILE * fI), tiles = (C.n + TILE - 1) / TILE;
+    int j = TILE;
+    while (j > 32 && ib * tiles * (TILE / j) < resident) j /= 2;
+    const int64_t W = ib * tiles * (TILE / j);
+    const int64_t G = resident * (waves > 0 ? std::min(waves, MAX_WAVES) : DEFAULT_WAVES);
+    const int64_t cap = std::min<int64_t>(part_elems_for(P.num_sms, C.n) / (3 * C.n),
+                                          MAX_PART_SLOTS);
+    h = Heavy{};
+    h.full = make_decomp(W, tiles, TILE * fI, std::min(G, W), cap, j);
+    h.mu = C.mu[0];
+    const int64_t groups = C.n / 512 + h.full.slots + 1;
+    if (groups > HV_GROUPS) return NB_OK;
+    h.parts = (int)((groups + HV_PART - 1) / HV_PART);
+    h.blocks = (int)std::min<int64_t>(hv_limit(C.n) * h.parts, 2 * P.num_sms);
+    return reserve(C.hv_sum, C.hv_sum_elems, hv_limit(C.n) * h.parts * HV_PART * 3,
+                   C.part_ordered, st);
+}
+
 int plan_make(const Pool &P, ClusterSet &C, int precision, cudaStream_t st, Plan &out,
               const PairShape *force, bool use_table, int waves)
 {
@@ -585,45 +616,14 @@ int plan_make(const Pool &P, ClusterSet &C, int precision, cudaStream_t st, Plan
         const int64_t limit = C.part_limit / 24;
         if (make_sym_decomp(C.nk.data(), C.K, C.uoff.data(), TILE * I, j, G, limit, true, pl.pl.d,
                             C.poff.data(), &rows) &&
-            set_reserve_part(C, 3 * rows > full ? 3 * rows : full, st) == NB_OK)
+            set_reserve_part(C, 3 * rows > full ? 3 * rows : full, st) == NB_OK &&
+            (pl.pl.mode != PM_DS_NEAR ||
+             plan_heavy(P, C, pl.pl.mode, waves, st, pl.heavy) == NB_OK))
             break;
+        pl.heavy = Heavy{};
         sym = false;   // the slots do not fit: the full kernels
     }
     pl.pl.d.fpart = sp_family(pl.pl.mode) ? 1 : 0;
-    if (sym && pl.pl.mode == PM_DS_NEAR) {
-        // the full kernels' untuned decomposition of the set
-        const int fI = full_default_I(C, pl.pl.mode);
-        const int fo = std::max(1, pair_occupancy(pl.pl.mode, fI));
-        const int64_t resident = (int64_t)P.num_sms * fo;
-        const int64_t ib = (C.n + TILE * fI - 1) / (TILE * fI), tiles = (C.n + TILE - 1) / TILE;
-        int j = TILE;
-        while (j > 32 && ib * tiles * (TILE / j) < resident) j /= 2;
-        const int64_t W = ib * tiles * (TILE / j);
-        const int64_t G = resident * (waves > 0 ? std::min(waves, MAX_WAVES) : DEFAULT_WAVES);
-        const int64_t cap = std::min<int64_t>(part_elems_for(P.num_sms, C.n) / (3 * C.n),
-                                              MAX_PART_SLOTS);
-        pl.heavy.full = make_decomp(W, tiles, TILE * fI, std::min(G, W), cap, j);
-        const int64_t groups = C.n / 512 + pl.heavy.full.slots + 1;
-        if (groups <= HV_GROUPS) {
-            pl.heavy.parts = (int)((groups + HV_PART - 1) / HV_PART);
-            pl.heavy.blocks = (int)std::min<int64_t>(hv_limit(C.n) * pl.heavy.parts,
-                                                     2 * P.num_sms);
-            const int64_t need = hv_limit(C.n) * pl.heavy.parts * HV_PART * 3;
-            if (C.hv_sum_elems < need) {
-                if (C.hv_sum) NB_TRY(cudaFree(C.hv_sum));
-                C.hv_sum = nullptr;
-                C.hv_sum_elems = 0;
-                if (cudaMalloc(&C.hv_sum, (size_t)need * 4) == cudaSuccess) {
-                    C.hv_sum_elems = need;
-                } else {
-                    cudaGetLastError();
-                    return set_error(NB_ENOMEM, "partial-sum storage: %lld bytes not available",
-                                     (long long)need * 4);
-                }
-            }
-        }
-        pl.heavy.mu = C.mu[0];
-    }
     // several clusters by value: launch the blocks largest-work first.  Not
     // with the near-pair pass beside the pair kernel: its kernels get SMs as
     // the pair kernel's blocks drain, and on the 512-cluster ensemble the

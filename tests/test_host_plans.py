@@ -129,6 +129,34 @@ def test_range_launches_take_the_full_kernels_shape(host, prec, n, kernel, ipb):
             assert not host.ran("pair_sym")
 
 
+def test_no_room_for_the_encounter_sums_takes_the_full_kernels(host, ctx):
+    """The partial sums are there (they serve every precision), 1 MB more is not."""
+    host.fail_from(100 << 10)
+    ctx.set_precision("ds")
+    ctx.step(2, 1e-3, 1)
+    assert host.ran("pair_sp_kernel") and not host.ran("pair_sym") and not host.ran("encounter")
+    host.fail_from()
+    ctx.set_precision("ds")
+    host.clear()
+    ctx.step(2, 1e-3, 1)
+    assert host.ran("pair_sym") and host.ran("encounter") and host.stale == 0
+
+
+def test_serving_groups_grow_without_stopping_the_device(host):
+    """Jobs of growing size in the mixed mode's large groups: neither cudaMalloc nor
+    cudaFree, which wait for every group's work, once the server stands."""
+    host.fail_from()
+    nb = host.nbsym
+    with nb.Server(hbm_budget_bytes=1e8) as srv:
+        host.clear()
+        for n in (12000, 20000, 30000, 40000):
+            pos, vel, m = ics.plummer(n, 1)
+            jid = srv.submit(pos, vel, m, 6, 1e-3, 2, precision="ds", eps=1e-2)
+            assert srv.wait(jid, 60)["state"] == nb.JOB_DONE
+        assert len(host.ran("encounter")) == 4 * 2 * 7
+        assert host.syncing == 0
+
+
 def _chosen(host, prec, sizes):
     host.fail_from()
     kw = dict(capacity=sizes[0]) if len(sizes) == 1 else dict(sizes=sizes)
