@@ -552,6 +552,7 @@ int plan_make(const Pool &P, ClusterSet &C, int precision, cudaStream_t st, Plan
     pl.pl.mode = plan_mode(C, precision);
     bool sym = use_sym(C, pl.pl.mode);
     int I, bps = 0, jt = 0;
+    bool untuned = false;
     PairShape tuned;
     if (force) {
         I = force->I;
@@ -564,6 +565,7 @@ int plan_make(const Pool &P, ClusterSet &C, int precision, cudaStream_t st, Plan
         jt = tuned.jt;
     } else {
         I = sym ? sym_default_I(C, pl.pl.mode) : full_default_I(C, pl.pl.mode);
+        untuned = true;
     }
     if (!pair_variant_exists(pl.pl.mode, I))
         return set_error(NB_EINVAL, "no pair kernel with %d bodies per thread for this precision",
@@ -621,7 +623,8 @@ int plan_make(const Pool &P, ClusterSet &C, int precision, cudaStream_t st, Plan
              plan_heavy(P, C, pl.pl.mode, waves, st, pl.heavy) == NB_OK))
             break;
         pl.heavy = Heavy{};
-        sym = false;   // the slots do not fit: the full kernels
+        sym = false;   // the slots do not fit: the full kernels, in their own shape
+        if (untuned) pl.pl.I = I = full_default_I(C, pl.pl.mode);
     }
     pl.pl.d.fpart = sp_family(pl.pl.mode) ? 1 : 0;
     // several clusters by value: launch the blocks largest-work first.  Not

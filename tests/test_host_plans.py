@@ -53,8 +53,20 @@ def test_no_room_for_symmetric_slots_takes_the_full_kernels(host, ctx):
     host.fail_from(80 << 20)   # the full kernels' 69 MB still fit
     ctx.set_precision("fp64")
     ctx.step(2, 1e-3, 1)
-    assert host.ran("pair_fp64_kernel") and not host.ran("pair_sym")
+    assert host.ran("pair_fp64_kernelILi1E") and not host.ran("pair_sym")
     assert host.stale == 0
+
+
+@pytest.mark.parametrize("prec,n,kernel", [("dd", 440000, "pair_ff_kernelILi1E"),
+                                           ("fp64", 320000, "pair_fp64_kernelILi1E")])
+def test_slots_beyond_the_limit_take_the_full_kernels_shape(host, prec, n, kernel):
+    """More than the 4 GB that symmetric slots may take."""
+    host.fail_from()
+    with host.nbsym.Context(n, eps=1e-2, precision=prec) as c:
+        c.load(np.zeros((n, 3)), np.zeros((n, 3)), np.ones(n))
+        host.clear()
+        c.accel()
+        assert host.ran(kernel) and not host.ran("pair_sym")
 
 
 @pytest.mark.parametrize("change", ["precision", "load", "params"])
