@@ -453,9 +453,9 @@ typedef struct {
     double hbm_budget_bytes;  /* device memory for resident state (> 0);
                                  about 436 bytes per body slot, plus the
                                  groups' partial sums beyond that share (at
-                                 most ~67 MB or a 32nd of the budget,
-                                 whichever is more, per group of the twelve;
-                                 17 MB each from the start) */
+                                 most ~67 MB for each of the twelve groups,
+                                 805 MB in all; a twentieth of the budget, at
+                                 most 201 MB, of it from the start) */
     int max_jobs;             /* resident jobs at most, 1..65536 */
     double G;                 /* as nb_params */
     int ext_on;

@@ -162,13 +162,14 @@ int set_create(ClusterSet &C, int32_t kcap, int64_t body_cap, int priority)
 }
 
 // Storage of at least need elements at p (have of them there), grown by half or
-// more: freed and allocated on the stream (ordered) or by the plain calls, which
+// more, within most where that is enough: freed and allocated on the stream (ordered) or by the plain calls, which
 // wait for all work of the device.
 template <typename T>
-static int reserve(T *&p, int64_t &have, int64_t need, bool ordered, cudaStream_t st)
+static int reserve(T *&p, int64_t &have, int64_t need, int64_t most, bool ordered,
+                   cudaStream_t st)
 {
     if (have >= need) return NB_OK;
-    const int64_t want = p ? std::max(need, have * 3 / 2) : need;
+    const int64_t want = p ? std::max(need, std::min(have * 3 / 2, most)) : need;
     if (p) {
         NB_TRY(ordered ? cudaFreeAsync(p, st) : cudaFree(p));
         p = nullptr;
@@ -190,7 +191,7 @@ static int reserve(T *&p, int64_t &have, int64_t need, bool ordered, cudaStream_
 
 int set_reserve_part(ClusterSet &C, int64_t elems, cudaStream_t st)
 {
-    return reserve(C.part, C.part_elems, elems, C.part_ordered, st);
+    return reserve(C.part, C.part_elems, elems, C.part_limit / 8, C.part_ordered, st);
 }
 
 void set_destroy(ClusterSet &C)
@@ -540,7 +541,7 @@ static int plan_heavy(const Pool &P, ClusterSet &C, int mode, int waves, cudaStr
     if (groups > HV_GROUPS) return NB_OK;
     h.parts = (int)((groups + HV_PART - 1) / HV_PART);
     h.blocks = (int)std::min<int64_t>(hv_limit(C.n) * h.parts, 2 * P.num_sms);
-    return reserve(C.hv_sum, C.hv_sum_elems, hv_limit(C.n) * h.parts * HV_PART * 3,
+    return reserve(C.hv_sum, C.hv_sum_elems, hv_limit(C.n) * h.parts * HV_PART * 3, INT64_MAX,
                    C.part_ordered, st);
 }
 

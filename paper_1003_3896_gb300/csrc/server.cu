@@ -90,10 +90,16 @@ constexpr size_t PAIR_IV_CAP = (size_t)1 << 20;
 constexpr int64_t SMALL_JOB = 16384;
 constexpr int NGROUPS = 12;               // (FP64, NB_DS, NB_DD) x (order 2, 6) x (small, large)
 
-// A group's partial sums for the symmetric kernels: a 32nd of the budget, or
-// this many bytes (the full kernels' fixed part) where that is more.
-constexpr double GROUP_PART_LEAST = 67.0e6;
-constexpr int64_t GROUP_PART_WARM = 1 << 24;   // of it at creation
+// Partial sums.  The full kernels of a group of n bodies reserve at most this fixed
+// part and 48 bytes per body, which the body's slot counts (BYTES_PER_BODY); the
+// budget is understood to come with the fixed part of every group.  The symmetric
+// kernels' slots may be more: groups share what others leave of that allowance
+// (with fp64_via_dd the double-precision groups have no jobs) and what the budget
+// itself leaves (part_limit).
+constexpr double GROUP_PART = 67.0e6;
+// Of it at creation (warm), in all at most this share of the budget.
+constexpr int64_t GROUP_PART_WARM = 1 << 24;
+constexpr double WARM_SHARE = 1.0 / 20;
 
 // Bytes of device memory the pool and the group scratch use per body slot:
 // state, float planes, j-stream, near-pair correction, staging, near-pair
@@ -301,6 +307,25 @@ bool can_enqueue_ahead(const nb_server *s, const Group &g)
     return true;
 }
 
+bool unused(const nb_server *s, const Group &g)
+{
+    return g.precision == NB_FP64 && s->p.fp64_via_dd;
+}
+
+// Bytes that the symmetric kernels' slots of group g may take (its set defined).
+int64_t part_limit(const nb_server *s, const Group &g)
+{
+    const auto own = [](const Group &q) { return GROUP_PART + 48.0 * (double)q.set.n; };
+    double spare = std::max(0.0, s->p.hbm_budget_bytes - (double)s->cap * BYTES_PER_BODY);
+    for (const Group &q : s->groups) {
+        if (unused(s, q))
+            spare += GROUP_PART;
+        else if (&q != &g)
+            spare -= std::max(0.0, (double)q.set.part_elems * 8.0 - own(q));
+    }
+    return (int64_t)(own(g) + std::max(0.0, spare));
+}
+
 // Enqueue the next step of group g (lock held: the tables are rebuilt from
 // the job records when the membership changed, which happens only with no
 // step of the group in flight).
@@ -321,7 +346,7 @@ int launch_step(nb_server *s, Group &g)
         int rc = set_define(g.set, (int32_t)nk.size(), boff.data(), nk.data(), eps.data(),
                             dts.data());
         g.set.mu = mu;
-        // the group's own partial sums: groups step concurrently
+        g.set.part_limit = part_limit(s, g);
         // the large jobs' groups: the most waves, so their blocks are short
         // and free SM slots for the small jobs' kernels sooner
         const bool large = ((&g - s->groups) & 1) != 0;
@@ -345,7 +370,7 @@ int launch_step(nb_server *s, Group &g)
     return NB_OK;
 }
 
-// A step of one body of no mass in every group, and its upload and download,
+// A step of one body of no mass in every group that may get jobs, and its upload and download,
 // before the scheduler starts: what a first use costs (partial sums of jobs of a
 // few thousand bodies, allocator, launch paths; 2.3 ms for the first of them in a
 // process) otherwise holds up the first admissions.
@@ -361,8 +386,11 @@ int warm(nb_server *s)
     int rc = upload(s, j);
     const int64_t off = 0, n = 1;
     const double one = 1.0;
+    const int64_t part = std::min<int64_t>(
+        GROUP_PART_WARM, (int64_t)(WARM_SHARE * s->p.hbm_budget_bytes / NGROUPS));
     for (Group &g : s->groups) {
-        if (!rc) rc = set_reserve_part(g.set, GROUP_PART_WARM / 8, g.stream);
+        if (unused(s, g)) continue;
+        if (!rc) rc = set_reserve_part(g.set, part / 8, g.stream);
         if (!rc) rc = set_define(g.set, 1, &off, &n, &one, &one);
         g.set.mu.assign(1, 0.0);
         Plan pl;
@@ -503,7 +531,6 @@ int nb_server_create(const nb_server_params *p, nb_server **out)
         const int prio = (g & 1) ? least : greatest;   // the small jobs' groups first
         rc = set_create(gr.set, p->max_jobs, cap, prio);
         gr.set.part_ordered = true;
-        gr.set.part_limit = (int64_t)std::max(GROUP_PART_LEAST, p->hbm_budget_bytes / 32.0);
         if (!rc && cudaStreamCreateWithPriority(&gr.stream, cudaStreamNonBlocking, prio) != cudaSuccess)
             rc = set_error(NB_ECUDA, "stream creation failed");
         for (StepSlot &sl : gr.slot) {

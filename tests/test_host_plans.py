@@ -169,6 +169,50 @@ def test_serving_groups_grow_without_stopping_the_device(host):
         assert host.syncing == 0
 
 
+def _server_growth(host, jobs, **kw):
+    """Device bytes that a server of the default budget takes for these jobs."""
+    nb = host.nbsym
+    with nb.Server(hbm_budget_bytes=4e9, **kw) as srv:
+        host.clear()
+        start = host.live
+        for n, order, prec in jobs:
+            pos, vel, m = ics.plummer(n, 1)
+            jid = srv.submit(pos, vel, m, order, 1e-3, 1, precision=prec, eps=1e-2)
+            assert srv.wait(jid, 60)["state"] == nb.JOB_DONE
+        return host.live - start, bool(host.ran("pair_sym_kernel"))
+
+
+def test_server_partial_sums_stay_within_the_groups_allowance(host):
+    """Large jobs of every group: the symmetric slots of 65536 bodies take 119 MB where
+    the allowance of unused groups covers them, else what is left; in all at most
+    67 MB for each of the twelve groups and 48 bytes per body of each."""
+    host.fail_from()
+    n = 65536
+    grown, sym = _server_growth(host, [(n, 6, "ds")])
+    assert sym and grown <= 140e6
+    # all groups may have jobs: no group beyond its own 67 MB
+    grown, _ = _server_growth(host, [(n, 6, "ds")], fp64_via_dd=0)
+    assert grown <= 67e6 + 60 * n
+    jobs = [(m, order, prec) for m in (4000, n, 2 * n) for order in (2, 6) for prec in ("ds", "dd")]
+    grown, _ = _server_growth(host, jobs)
+    assert grown <= 12 * 67e6 + 60 * sum(j[0] for j in jobs)
+
+
+def test_server_takes_little_at_creation_with_a_small_budget(host):
+    """What creation takes beyond its share per budget byte."""
+    host.fail_from()
+    live = []
+    for budget in (1e8, 2e8):
+        before = host.live
+        with host.nbsym.Server(hbm_budget_bytes=budget):
+            live.append(host.live - before)
+    assert 2 * live[0] - live[1] <= 8e6
+    before = host.live
+    with host.nbsym.Server(hbm_budget_bytes=4e9, max_jobs=4):
+        pass
+    assert host.live == before
+
+
 def _chosen(host, prec, sizes):
     host.fail_from()
     kw = dict(capacity=sizes[0]) if len(sizes) == 1 else dict(sizes=sizes)
