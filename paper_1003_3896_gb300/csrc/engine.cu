@@ -141,10 +141,6 @@ int set_create(ClusterSet &C, int32_t kcap, int64_t body_cap, int priority)
     A((void **)&C.ng_spos, (size_t)body_cap * 16);
     A((void **)&C.ng_slo, (size_t)body_cap * 16);
     A((void **)&C.ng_slot, (size_t)C.ng_hcap * sizeof(NgSlot));
-    A((void **)&C.hv_flag, (size_t)body_cap);
-    A((void **)&C.hv_list, (size_t)hv_limit(body_cap) * 4);
-    A((void **)&C.hv_count, sizeof(int));
-    A((void **)&C.hv_done, (size_t)hv_limit(body_cap) * 4);
     if (!ok) {
         cudaGetLastError();
         set_destroy(C);
@@ -198,11 +194,10 @@ void set_destroy(ClusterSet &C)
 {
     void *ptrs[] = {C.dmem,    C.red,   C.ng_bucket, C.ng_entry, C.ng_total, C.flag,
                     C.cid,     C.ng_spos, C.ng_slo,  C.ng_slot,  C.ng_rank,
-                    C.hv_flag, C.hv_list, C.hv_count, C.hv_done};
+                    C.hv_mem};
     for (void *q : ptrs)
         if (q) cudaFree(q);
     if (C.part) cudaFree(C.part);
-    if (C.hv_sum) cudaFree(C.hv_sum);
     if (C.fork) cudaEventDestroy(C.fork);
     if (C.join) cudaEventDestroy(C.join);
     if (C.side) cudaStreamDestroy(C.side);
@@ -284,53 +279,36 @@ int set_layout(ClusterSet &C, cudaStream_t st)
     }
     const int64_t S = (int64_t)C.seg_k.size();
     if (S > C.scap) return set_error(NB_EINVAL, "too many reduction segments");
-    // device layout (must match set_create's size computation)
-    const size_t k8 = (size_t)C.kcap * 8, k81 = (size_t)(C.kcap + 1) * 8;
-    char *p = C.dmem;
-    auto take = [&](size_t bytes) {
-        char *q = p;
-        p += al(bytes);
-        return q;
-    };
-    int64_t *d_boff = (int64_t *)take(k8);
-    int64_t *d_nk = (int64_t *)take(k8);
-    int64_t *d_noff = (int64_t *)take(k81);
-    int64_t *d_uoff = (int64_t *)take(k81);
-    int64_t *d_uoffp = (int64_t *)take(k81);
-    int32_t *d_ntiles = (int32_t *)take((size_t)C.kcap * 4);
-    float *d_eps2f = (float *)take((size_t)C.kcap * 4);
-    double *d_eps2d = (double *)take(k8);
-    double *d_dts = (double *)take(k8);
-    int32_t *d_segk = (int32_t *)take((size_t)C.scap * 4);
-    int64_t *d_seglo = (int64_t *)take((size_t)C.scap * 8);
-    int64_t *d_seghi = (int64_t *)take((size_t)C.scap * 8);
-    int32_t *d_segoff = (int32_t *)take((size_t)(C.kcap + 1) * 4);
-    C.frame = (Frame *)take((size_t)C.kcap * sizeof(Frame));
-    C.diag = (double *)take((size_t)C.kcap * DIAG_STRIDE * 8);
-    double *d_mu = (double *)take(k8);
-    int64_t *d_poff = (int64_t *)take(k8);
-    int64_t *d_poffp = (int64_t *)take(k8);
+    // frames and diagnostics at fixed places, then the tables, gathered on the host
+    // and copied at once (a copy each took 2 us); set_create's size covers them
+    C.frame = (Frame *)C.dmem;
+    C.diag = (double *)(C.dmem + al((size_t)C.kcap * sizeof(Frame)));
+    char *const dev = (char *)C.diag + al((size_t)C.kcap * DIAG_STRIDE * 8);
     if ((int32_t)C.mu.size() != K) C.mu.assign(K, 0.0);
-    auto up = [&](void *dst, const void *src, size_t bytes) {
-        return bytes ? cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, st)
-                     : cudaSuccess;
+    std::vector<char> host;
+    auto put = [&](const auto &v, size_t count) {
+        const size_t at = (host.size() + 15) / 16 * 16, bytes = count * sizeof(v[0]);
+        host.resize(at + bytes);
+        if (bytes) std::memcpy(host.data() + at, v.data(), bytes);
+        return dev + at;
     };
-    NB_TRY(up(d_boff, C.boff.data(), K * 8));
-    NB_TRY(up(d_nk, C.nk.data(), K * 8));
-    NB_TRY(up(d_noff, C.noff.data(), (K + 1) * 8));
-    NB_TRY(up(d_uoff, C.uoff.data(), (K + 1) * 8));
-    NB_TRY(up(d_uoffp, C.uoff_pot.data(), (K + 1) * 8));
-    NB_TRY(up(d_ntiles, C.ntiles.data(), K * 4));
-    NB_TRY(up(d_eps2f, C.eps2f.data(), K * 4));
-    NB_TRY(up(d_eps2d, C.eps2d.data(), K * 8));
-    NB_TRY(up(d_dts, C.dts.data(), K * 8));
-    NB_TRY(up(d_mu, C.mu.data(), K * 8));
-    NB_TRY(up(d_poff, C.poff.data(), K * 8));
-    NB_TRY(up(d_poffp, C.poff_pot.data(), K * 8));
-    NB_TRY(up(d_segk, C.seg_k.data(), S * 4));
-    NB_TRY(up(d_seglo, C.seg_lo.data(), S * 8));
-    NB_TRY(up(d_seghi, C.seg_hi.data(), S * 8));
-    NB_TRY(up(d_segoff, C.seg_off.data(), (K + 1) * 4));
+    int64_t *d_boff = (int64_t *)put(C.boff, K);
+    int64_t *d_nk = (int64_t *)put(C.nk, K);
+    int64_t *d_noff = (int64_t *)put(C.noff, K + 1);
+    int64_t *d_uoff = (int64_t *)put(C.uoff, K + 1);
+    int64_t *d_uoffp = (int64_t *)put(C.uoff_pot, K + 1);
+    int32_t *d_ntiles = (int32_t *)put(C.ntiles, K);
+    float *d_eps2f = (float *)put(C.eps2f, K);
+    double *d_eps2d = (double *)put(C.eps2d, K);
+    double *d_dts = (double *)put(C.dts, K);
+    int32_t *d_segk = (int32_t *)put(C.seg_k, S);
+    int64_t *d_seglo = (int64_t *)put(C.seg_lo, S);
+    int64_t *d_seghi = (int64_t *)put(C.seg_hi, S);
+    int32_t *d_segoff = (int32_t *)put(C.seg_off, K + 1);
+    double *d_mu = (double *)put(C.mu, K);
+    int64_t *d_poff = (int64_t *)put(C.poff, K);
+    int64_t *d_poffp = (int64_t *)put(C.poff_pot, K);
+    NB_TRY(cudaMemcpyAsync(dev, host.data(), host.size(), cudaMemcpyHostToDevice, st));
     Clusters &c = C.cl;
     c.K = K;
     c.boff = d_boff;
@@ -541,8 +519,16 @@ static int plan_heavy(const Pool &P, ClusterSet &C, int mode, int waves, cudaStr
     if (groups > HV_GROUPS) return NB_OK;
     h.parts = (int)((groups + HV_PART - 1) / HV_PART);
     h.blocks = (int)std::min<int64_t>(hv_limit(C.n) * h.parts, 2 * P.num_sms);
-    return reserve(C.hv_sum, C.hv_sum_elems, hv_limit(C.n) * h.parts * HV_PART * 3, INT64_MAX,
-                   C.part_ordered, st);
+    const int64_t listed = hv_limit(C.n), sums = listed * h.parts * HV_PART * 3;
+    const int rc = reserve(C.hv_mem, C.hv_bytes, 4 * (sums + 2 * listed + 1) + C.n, INT64_MAX,
+                           C.part_ordered, st);
+    if (rc) return rc;
+    C.hv_sum = (float *)C.hv_mem;
+    C.hv_list = (int *)(C.hv_sum + sums);
+    C.hv_done = C.hv_list + listed;
+    C.hv_count = C.hv_done + listed;
+    C.hv_flag = (unsigned char *)(C.hv_count + 1);
+    return NB_OK;
 }
 
 int plan_make(const Pool &P, ClusterSet &C, int precision, cudaStream_t st, Plan &out,

@@ -71,10 +71,12 @@ struct ClusterSet {
     int32_t *cid = nullptr;    // linear body -> cluster map
     float4 *ng_spos = nullptr, *ng_slo = nullptr;
     NgSlot *ng_slot = nullptr;
-    unsigned char *hv_flag = nullptr;   // bodies in a close encounter (DevState)
+    // bodies in a close encounter (DevState), in storage of a plan that looks for them
+    unsigned char *hv_flag = nullptr;
     int *hv_list = nullptr, *hv_count = nullptr, *hv_done = nullptr;
-    float *hv_sum = nullptr;            // reserved by a plan that needs it
-    int64_t hv_sum_elems = 0;
+    float *hv_sum = nullptr;
+    char *hv_mem = nullptr;
+    int64_t hv_bytes = 0;
     Frame *frame = nullptr;    // [kcap]
     double *diag = nullptr;    // [kcap][DIAG_STRIDE]
     Clusters cl, cl_pot;       // device views (pair units / potential units)
@@ -231,7 +233,7 @@ int stage_weights(int order, double *w);
 // (the bits of enq_step).
 constexpr int SMALL_MAX = 1024;
 constexpr int SMALL_SLOTS = 40;
-bool small_ok(const ClusterSet &C, const Plan &pl);
+bool small_ok(const ClusterSet &C, const Plan &pl, const Phys &ph);
 bool small_order(const ClusterSet &C, const Plan &pl, int order);
 int small_steps(const Pool &P, const ClusterSet &C, const Plan &pl, const Phys &ph, int order,
                 double h, int64_t steps, cudaStream_t st);

@@ -175,7 +175,7 @@ int replan(nb_ctx *c, int64_t n)
         c->set.mu.assign(nk.size(), 0.0);
     rc = plan_make(c->pool, c->set, c->p.precision, c->stream, c->plan);
     if (rc) return rc;
-    c->small = small_ok(c->set, c->plan);
+    c->small = small_ok(c->set, c->plan, c->phys);
     c->planned = true;
     c->split_stale = true;
     return NB_OK;
@@ -921,7 +921,7 @@ int nb_tune(nb_ctx *c, int reps, nb_tune_t *out)
         return set_error(rc, "%s", why.c_str());
     }
     c->plan = pl;
-    c->small = small_ok(c->set, c->plan);
+    c->small = small_ok(c->set, c->plan, c->phys);
     if (out) {
         out->precision = rep.precision;
         out->bodies_per_thread = rep.shape.I;

@@ -397,7 +397,7 @@ bool fits(Kernel kernel)
 
 }  // namespace
 
-bool small_ok(const ClusterSet &C, const Plan &pl)
+bool small_ok(const ClusterSet &C, const Plan &pl, const Phys &ph)
 {
     const Decomp &d = pl.pl.d;
     if (C.K != 1 || C.n > SMALL_MAX || d.sym || d.rows || d.b0 || d.slots > SMALL_SLOTS)
@@ -405,8 +405,7 @@ bool small_ok(const ClusterSet &C, const Plan &pl)
     // a block's bodies lie in at most two rows
     if (d.ipb < OWN || !d.fpart) return false;
     if (pl.pl.mode != PM_DS_FULL && pl.pl.mode != PM_FP32) return false;
-    return fits(kernel_of(pl.pl.mode == PM_DS_FULL, pl.pl.um, false)) &&
-           fits(kernel_of(pl.pl.mode == PM_DS_FULL, pl.pl.um, true));
+    return fits(kernel_of(pl.pl.mode == PM_DS_FULL, pl.pl.um, ph.ext.on));
 }
 
 bool small_order(const ClusterSet &C, const Plan &pl, int order)
