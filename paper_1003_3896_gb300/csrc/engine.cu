@@ -190,6 +190,15 @@ int set_reserve_part(ClusterSet &C, int64_t elems, cudaStream_t st)
     return reserve(C.part, C.part_elems, elems, C.part_limit / 8, C.part_ordered, st);
 }
 
+int set_release_part(ClusterSet &C, cudaStream_t st)
+{
+    double *const p = C.part;
+    C.part = nullptr;
+    C.part_elems = 0;
+    if (p) NB_TRY(C.part_ordered ? cudaFreeAsync(p, st) : cudaFree(p));
+    return NB_OK;
+}
+
 void set_destroy(ClusterSet &C)
 {
     void *ptrs[] = {C.dmem,    C.red,   C.ng_bucket, C.ng_entry, C.ng_total, C.flag,

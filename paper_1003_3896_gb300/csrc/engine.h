@@ -110,6 +110,8 @@ void block_order(ClusterSet &C, const Decomp &d, int I, bool partial);
 // smaller (part_ordered: by stream-ordered allocation on st); none of the
 // set's work may be in flight.
 int set_reserve_part(ClusterSet &C, int64_t elems, cudaStream_t st);
+// Give it back (the next plan reserves what it needs).
+int set_release_part(ClusterSet &C, cudaStream_t st);
 void set_destroy(ClusterSet &C);
 // Clusters k = 0..K-1 at pool slots [boff[k], boff[k] + nk[k]), softening
 // eps[k] and step scale dts[k] (NULL: 1).  Host only; set_layout uploads.

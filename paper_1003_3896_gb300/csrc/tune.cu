@@ -277,8 +277,12 @@ int tune_pair(const Pool &P, ClusterSet &C, int precision, const Phys &ph, cudaS
         rep.pair_ms = best_ms;
         rep.cost_ms = best_cost;
         tune_store(tune_key(P, C, precision), best);
-        rc = plan_make(P, C, precision, st, out, &best, false);
     } while (0);
+    // the candidates' largest partial sums go back (262144 bodies in the mixed mode
+    // hold 3.2 GB for the narrowest i-blocks, 0.8 for the default's)
+    const int rel = set_release_part(C, st);
+    if (!rc) rc = rel;
+    if (!rc) rc = plan_make(P, C, precision, st, out, &best, false);
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     return rc;

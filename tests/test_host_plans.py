@@ -274,3 +274,30 @@ def test_new_step_lengths_capture_one_small_graph_each(host):
                 for k in range(8):
                     c.step(2, 3e-4 * (1 + k), 33)
             assert host.captures == 0
+
+
+@pytest.mark.parametrize("prec", ["ds", "fp64"])
+def test_tuning_gives_its_partial_sums_back(host, prec):
+    """The candidates reach the narrowest i-blocks' slots; what stays is what the chosen
+    shape takes in a fresh context."""
+    host.fail_from()
+    n = 60000
+    nb = host.nbsym
+    body = ics.plummer(n, 1)
+    before = host.live
+    try:
+        with nb.Context(n, eps=1e-2, precision=prec) as c:
+            c.load(*body)
+            c.step(2, 1e-3, 1)
+            host.clear()
+            c.tune(1)
+            shape, held = c.pair_shape(), host.live - before
+            assert host.peak - before > 1.5 * held
+            c.step(2, 1e-3, 1)
+            assert host.stale == 0
+        with nb.Context(n, eps=1e-2, precision=prec) as c:   # takes the tuned shape
+            c.load(*body)
+            assert c.pair_shape() == shape
+            assert host.live - before == held
+    finally:
+        nb.tune_clear()
