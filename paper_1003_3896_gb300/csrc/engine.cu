@@ -525,7 +525,9 @@ static int plan_heavy(const Pool &P, ClusterSet &C, int mode, int waves, cudaStr
     h.full = make_decomp(W, tiles, TILE * fI, std::min(G, W), cap, j);
     h.mu = C.mu[0];
     const int64_t groups = C.n / 512 + h.full.slots + 1;
-    if (groups > HV_GROUPS) return NB_OK;
+    if (groups > HV_GROUPS)
+        return set_error(NB_EINVAL, "%lld bodies: too many for the search for encounters",
+                         (long long)C.n);
     h.parts = (int)((groups + HV_PART - 1) / HV_PART);
     h.blocks = (int)std::min<int64_t>(hv_limit(C.n) * h.parts, 2 * P.num_sms);
     const int64_t listed = hv_limit(C.n), sums = listed * h.parts * HV_PART * 3;

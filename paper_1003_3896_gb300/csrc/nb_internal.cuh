@@ -297,7 +297,10 @@ __host__ __device__ __forceinline__ int slot_parts(const Decomp &d, int64_t n)
 // close binaries) all keep their sums.
 constexpr float HV_X = 8.f;
 __host__ __device__ __forceinline__ int64_t hv_limit(int64_t n) { return n / 64 + 64; }
-constexpr int HV_GROUPS = 1024;   // float partial sums of a body's row, at most
+// Float partial sums of a body's row, at most (above it the full kernels run): more
+// than the largest system has whose symmetric slots fit a context's 4 GB, about
+// 620000 bodies.
+constexpr int HV_GROUPS = 1536;
 constexpr int HV_PART = 64;       // of them per block
 struct Heavy {
     Decomp full;    // the full kernels' default decomposition of the set

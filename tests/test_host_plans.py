@@ -301,3 +301,15 @@ def test_tuning_gives_its_partial_sums_back(host, prec):
             assert host.live - before == held
     finally:
         nb.tune_clear()
+
+
+@pytest.mark.parametrize("n", [520000, 530000, 600000, 700000])
+def test_symmetric_mixed_plans_look_for_encounters(host, n):
+    """Also near the size where the symmetric slots no longer fit."""
+    host.fail_from()
+    with host.nbsym.Context(n, eps=1e-2, precision="ds") as c:
+        c.load(np.zeros((n, 3)), np.zeros((n, 3)), np.ones(n))
+        host.clear()
+        c.accel()
+        assert bool(host.ran("pair_sym")) == bool(host.ran("encounter"))
+        assert bool(host.ran("pair_sym")) == (n <= 600000)
