@@ -152,6 +152,18 @@ def code_digest(text: str) -> str:
     return hashlib.sha256(" ".join(text.split()).encode()).hexdigest()[:16]
 
 
+def pipe_ops(precision: str, n: int, once: bool) -> float:
+    """Lane operations per interaction that the pair kernel issues to the pipe that
+    bounds it (FP32 FMA; FP64 in double precision), equal masses.  For an unordered
+    pair of the mixed mode: 3 differences, 3 for r^2, 2 for r^-3, 3 for each body's
+    sum.  `once`: each unordered pair, two interactions, is evaluated once."""
+    if once:
+        return {"ds": 14, "dd": 131, "fp64": 15}[precision] / 2
+    if precision == "ds":   # every pair in double-single up to 2^27 pairs
+        precision = "ds_full" if n * n <= 1 << 27 else "fp32"
+    return {"fp32": 11, "ds_full": 17, "dd": 107, "fp64": 12}[precision]
+
+
 def pair_source_digest() -> str | None:
     """code_digest of the pair kernel's sources: the recorded traffic stays valid
     across comment edits and lapses with any change of the kernel's code."""
@@ -443,6 +455,7 @@ def main():
     wall = time.perf_counter() - wall0
     prof = ctx.prof_read()
     shape = ctx.pair_shape()
+    once = ctx.pair_symmetric
     ctx.prof_enable(False)
     step_ms = [s.elapsed_time(e) for s, e in zip(starts, ends)]
     t_ms = max_over_ranks(sum(step_ms), dev)
@@ -487,20 +500,15 @@ def main():
 
     clocks = clk.summary()
     peaks = nbsym.measure_peaks(local)
-    achieved = FLOPS_PER_PAIR * prof["interactions"] / (prof["pair_ms"] * 1e-3) / 1e12
     sustained_mhz = clocks.get("sm_mhz") or 2070.0
-    # the symmetric kernels evaluate each unordered pair once and use it for both
-    # bodies, so the rate over the N^2 interactions (20 flops each by the paper's
-    # count) can pass the pipe's peak; pipe_busy counts what they issue
-    once = {"ds": n * n > 1 << 27, "dd": True, "fp64": n > 784}.get(args.precision, False)
-    kernel = "pair_sym_kernel" if once else {"fp64": "pair_fp64_kernel"}.get(args.precision,
-                                                                             "pair_sp_kernel")
-    pipe_busy = None
-    if once and args.precision == "ds":
-        # 14 FMA-pipe lane operations for an unordered pair of equal masses (3
-        # differences, 3 for r^2, 2 for r^-3, 3 for each body's sum)
-        pipe_busy = (14 * prof["interactions"] / 2 / (prof["pair_ms"] * 1e-3)
-                     / (fp32_peak_tflops(sms, 2070.0) * 1e12 / 2))
+    # achieved counts the lane operations that the pair kernel issues to the pipe
+    # that bounds it, two flops each as in the peak; the rate over all N^2
+    # interactions at the paper's 20 flops (the symmetric kernels evaluate each
+    # unordered pair once, for both bodies) is reported beside it
+    rate = prof["interactions"] / (prof["pair_ms"] * 1e-3) / 1e12
+    achieved = 2 * pipe_ops(args.precision, n, once) * rate
+    kernel = "pair_sym_kernel" if once else {"fp64": "pair_fp64_kernel", "dd": "pair_ff_kernel"}.get(
+        args.precision, "pair_sp_kernel")
     if args.precision == "fp64":
         # the FP64 pipe: the DFMA rate measured in the same run is the
         # ceiling (this GPU's DFMA issue measures ~83% of the nominal 1.25
@@ -528,7 +536,8 @@ def main():
                      "kernel": f"{kernel} ({args.precision})",
                      "peak_basis": peak_basis,
                      "pairs_evaluated": "each unordered pair once" if once else "every pair",
-                     "frac_of_issued_fma_lanes": pipe_busy,
+                     "pipe_ops_per_interaction": pipe_ops(args.precision, n, once),
+                     "effective_tflops_20_per_interaction": FLOPS_PER_PAIR * rate,
                      "frac_at_sampled_clock": frac_clock,
                      ("frac_of_nominal_fp64" if args.precision == "fp64"
                       else "frac_of_measured_fp32"): frac_meas,

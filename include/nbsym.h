@@ -423,6 +423,12 @@ int64_t nb_tune_load(const char *path);
 int nb_pair_shape(nb_ctx *ctx, int *bodies_per_thread, int *blocks_per_sm, int *j_tile,
                   int64_t *grid);
 
+/* 1 when the current plan's pair kernel evaluates each unordered pair once and
+ * adds its force to both bodies, 0 when it evaluates every pair for each body
+ * (nb_accel_range and nb_substep_range always do).  Errors: NB_EINVAL (NULL
+ * ctx), NB_ESTATE (nothing loaded). */
+int nb_pair_symmetric(nb_ctx *ctx);
+
 /* Number of entries in the table. */
 int64_t nb_tune_entries(void);
 

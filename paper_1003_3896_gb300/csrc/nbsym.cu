@@ -949,6 +949,13 @@ int nb_pair_shape(nb_ctx *c, int *bodies_per_thread, int *blocks_per_sm, int *j_
     return NB_OK;
 }
 
+int nb_pair_symmetric(nb_ctx *c)
+{
+    if (!c) return set_error(NB_EINVAL, "ctx is NULL");
+    if (c->n == 0 || !c->planned) return set_error(NB_ESTATE, "nothing loaded");
+    return c->plan.pl.d.sym;
+}
+
 int nb_tune_save(const char *path)
 {
     if (!path) return set_error(NB_EINVAL, "path is NULL");

@@ -112,6 +112,7 @@ nb_tune_load = _sig("nb_tune_load", C.c_int64, C.c_char_p)
 nb_tune_entries = _sig("nb_tune_entries", C.c_int64)
 nb_pair_shape = _sig("nb_pair_shape", C.c_int, _ctxp, C.POINTER(C.c_int), C.POINTER(C.c_int),
                      C.POINTER(C.c_int), C.POINTER(C.c_int64))
+nb_pair_symmetric = _sig("nb_pair_symmetric", C.c_int, _ctxp)
 nb_tune_clear = _sig("nb_tune_clear", None)
 
 
@@ -372,6 +373,11 @@ class Context:
         check(nb_pair_shape(self._h, C.byref(i), C.byref(b), C.byref(j), C.byref(g)))
         return {"bodies_per_thread": i.value, "blocks_per_sm": b.value, "j_tile": j.value,
                 "grid": g.value}
+
+    @property
+    def pair_symmetric(self) -> bool:
+        """Whether the plan's pair kernel evaluates each unordered pair once."""
+        return bool(check(nb_pair_symmetric(self._h)))
 
     def prof_enable(self, on: bool = True):
         check(nb_prof_enable(self._h, int(bool(on))))

@@ -42,6 +42,7 @@ def test_one_system(nbs, orc, prec, n):
         pos, vel, m = bodies(n, equal)
         with nbs.Context(n, eps=eps, precision=prec) as c:
             c.load(pos, vel, m)
+            assert c.pair_symmetric
             a = c.accel()
         assert rel_rms(a, orc.accel_int(pos, m, 1.0, eps)) <= TOL[prec], (equal, eps)
 
@@ -52,6 +53,7 @@ def test_clusters(nbs, orc, prec, sizes):
     pos, vel, m = (np.concatenate([c[q] for c in cl]) for q in range(3))
     with nbs.Context(sizes=sizes, precision=prec, eps=0.01) as b:
         b.load(pos, vel, m)
+        assert b.pair_symmetric
         a = b.accel()
     off = np.concatenate([[0], np.cumsum(sizes)])
     for k in [*range(min(20, len(sizes))), len(sizes) - 1]:
@@ -73,9 +75,11 @@ def test_float_float_sums_do_not_depend_on_the_kernel(nbs, n, equal):
         pos, vel, m = (np.concatenate([c[q] for c in cl]) for q in range(3))
         with nbs.Context(sizes=[n, 4100], precision="dd", eps=1e-3) as b:
             b.load(pos, vel, m)
+            assert b.pair_symmetric
             got = b.accel()[:n]
         with nbs.Context(n, precision="dd", eps=1e-3) as c:
             c.load(*cl[0])
+            assert not c.pair_symmetric
             alone = c.accel()
             parts = np.concatenate([c.accel_range(0, n // 2), c.accel_range(n // 2, n)])
         assert rel_rms(got, alone) <= 2e-15

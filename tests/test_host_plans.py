@@ -221,7 +221,8 @@ def _chosen(host, prec, sizes):
         c.load(np.zeros((n, 3)), np.zeros((n, 3)), np.ones(n))
         host.clear()
         c.accel()
-        return bool(host.ran("pair_sym"))
+        assert c.pair_symmetric == bool(host.ran("pair_sym"))
+        return c.pair_symmetric
 
 
 def test_sizes_of_the_symmetric_kernels_tests_take_them(host):
@@ -313,3 +314,32 @@ def test_symmetric_mixed_plans_look_for_encounters(host, n):
         c.accel()
         assert bool(host.ran("pair_sym")) == bool(host.ran("encounter"))
         assert bool(host.ran("pair_sym")) == (n <= 600000)
+
+
+def test_pair_symmetric_without_a_plan(host):
+    host.fail_from()
+    nb = host.nbsym
+    assert nb.nb_pair_symmetric(None) == nb.NB_EINVAL
+    with nb.Context(10) as c, pytest.raises(nb.NBError) as e:
+        c.pair_symmetric
+    assert e.value.code == nb.NB_ESTATE
+
+
+@pytest.mark.parametrize("prec,n,order,one", [
+    ("ds", 1, 2, True), ("ds", 480, 2, True), ("ds", 1024, 2, True), ("ds", 1025, 2, False),
+    ("ds", 704, 6, True), ("ds", 705, 6, False), ("fp32", 832, 6, True), ("fp32", 833, 6, False),
+    ("fp64", 480, 2, False), ("dd", 480, 2, False), ("ds_near", 480, 2, False)])
+def test_which_steps_run_in_one_kernel(host, prec, n, order, one):
+    """The sizes of the small-step tests that compare it with the separate kernels take
+    it, and a profiled context, the other side of that comparison, does not."""
+    host.fail_from()
+    with host.nbsym.Context(n, eps=1e-2, precision=prec) as c:
+        c.load(*ics.plummer(n, 1))
+        host.clear()
+        c.step(order, 1e-3, 3)
+        assert bool(host.ran("small_step_kernel")) == one
+        assert host.graphs == (0 if one else 3)
+        c.prof_enable(True)
+        host.clear()
+        c.step(order, 1e-3, 3)
+        assert not host.ran("small_step_kernel") and host.graphs == 3
