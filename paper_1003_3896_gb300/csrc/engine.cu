@@ -573,7 +573,7 @@ int plan_make(const Pool &P, ClusterSet &C, int precision, cudaStream_t st, Plan
     for (int32_t k = 0; k < C.K && pl.pl.um; ++k) pl.pl.um = C.mu[k] > 0;
     int64_t rows = 0;   // partial sums needed
     for (;;) {
-        int occ = sym ? sym_occupancy(pl.pl.mode, I) : pair_occupancy(pl.pl.mode, I);
+        int occ = sym ? sym_occupancy(pl.pl.mode, I, pl.pl.um) : pair_occupancy(pl.pl.mode, I);
         if (occ < 1) occ = 1;
         int b = bps;
         if (waves > 0) b = (waves < MAX_WAVES ? waves : MAX_WAVES) * occ;

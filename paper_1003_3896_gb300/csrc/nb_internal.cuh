@@ -372,7 +372,7 @@ constexpr int64_t MAX_PART_SLOTS = 128;
 int pair_occupancy(int mode, int I);
 bool pair_variant_exists(int mode, int I);
 // The same of the symmetric kernels (pairsym.cu); 0: no such variant.
-int sym_occupancy(int mode, int I);
+int sym_occupancy(int mode, int I, bool um);
 int potential_occupancy();
 // Narrowest unit: the kernels' chunk of j bodies.
 inline int sym_jt_least(int mode) { return mode == PM_DS_NEAR ? 64 : 32; }

@@ -58,9 +58,9 @@ cudaError_t launch_pair_sym(const DevState &s, const PairLaunch &pl, const HostT
                               : launch_sym_wide(s, pl, ht, G, st);
 }
 
-int sym_occupancy(int mode, int I)
+int sym_occupancy(int mode, int I, bool um)
 {
-    return sp_family(mode) ? occupancy_sym_sp(mode, I) : occupancy_sym_wide(mode, I);
+    return sp_family(mode) ? occupancy_sym_sp(mode, I, um) : occupancy_sym_wide(mode, I);
 }
 
 }  // namespace nb

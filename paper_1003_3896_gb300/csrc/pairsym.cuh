@@ -440,7 +440,7 @@ int occupancy_sym_any()
 // the variants (pairsym_sp.cu, pairsym_wide.cu)
 cudaError_t launch_sym_sp(const DevState &s, const PairLaunch &pl, const HostTab &ht, double G,
                           cudaStream_t st);
-int occupancy_sym_sp(int mode, int I);
+int occupancy_sym_sp(int mode, int I, bool um);
 cudaError_t launch_sym_wide(const DevState &s, const PairLaunch &pl, const HostTab &ht, double G,
                             cudaStream_t st);
 int occupancy_sym_wide(int mode, int I);

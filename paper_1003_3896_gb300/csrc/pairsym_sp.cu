@@ -27,7 +27,11 @@ struct Sp {
     static constexpr bool UM = UM_, JSUM = true, SELF = false;
     static constexpr int ACC = 6 * I;           // double-single running sums
     static constexpr int FOLD_CHUNKS = 8;       // 512 j bodies, 256 per float partial sum
-    static constexpr int MINB = I == 8 ? 3 : 4;
+    // resident blocks: the mass spectrum's registers (each i body's mass as both
+    // halves) do not fit those of one block more; spilled, an evaluation's kernel
+    // took 19.8 instead of 19.1 ms at N = 262144 (I = 8), 65 instead of 61 us at
+    // 12000 (I = 4)
+    static constexpr int MINB = I == 8 ? (UM ? 3 : 2) : UM ? 4 : 3;
     typedef float Slab;
     typedef float2 Part;
     typedef WideDS Wide;
@@ -210,13 +214,11 @@ cudaError_t launch_sym_sp(const DevState &s, const PairLaunch &pl, const HostTab
     return cudaErrorInvalidValue;
 }
 
-int occupancy_sym_sp(int mode, int I)
+int occupancy_sym_sp(int mode, int I, bool um)
 {
 #define NB_O(II)                                                                          \
-    if (mode == PM_DS_NEAR && I == II) {                                                  \
-        const int a = occupancy_sym<Sp<II, true>, 1>(), b = occupancy_sym<Sp<II, false>, 1>(); \
-        return a < b ? a : b;                                                             \
-    }
+    if (mode == PM_DS_NEAR && I == II)                                                    \
+        return um ? occupancy_sym<Sp<II, true>, 1>() : occupancy_sym<Sp<II, false>, 1>();
     NB_O(2) NB_O(4) NB_O(8)
 #undef NB_O
     return 0;

@@ -550,7 +550,8 @@ int nb_server_create(const nb_server_params *p, nb_server **out)
         for (int I : {1, 2, 4, 8}) {
             if (!rc && pair_variant_exists(mode, I)) {
                 pair_occupancy(mode, I);
-                if (mode != PM_DS_FULL) sym_occupancy(mode, I);
+                for (bool um : {true, false})
+                    if (mode != PM_DS_FULL) sym_occupancy(mode, I, um);
             }
         }
     if (!rc) potential_occupancy();

@@ -210,7 +210,7 @@ int tune_pair(const Pool &P, ClusterSet &C, int precision, const Phys &ph, cudaS
         const int Is[] = {1, 2, 4, 8};
         for (int I : Is) {
             if (!pair_variant_exists(mode, I)) continue;
-            const int occ = def.pl.d.sym ? sym_occupancy(mode, I) : pair_occupancy(mode, I);
+            const int occ = def.pl.d.sym ? sym_occupancy(mode, I, def.pl.um) : pair_occupancy(mode, I);
             // finer j-ranges only pay when full-width units are scarce
             int64_t w_full = 0;
             for (int32_t k = 0; k < C.K; ++k)
