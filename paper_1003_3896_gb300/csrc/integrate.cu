@@ -449,10 +449,10 @@ __device__ __forceinline__ bool is_heavy(const DevState &s, const Decomp &d, int
     return FP && d.sym && s.hv_flag && s.hv_flag[t] && *s.hv_count <= hv_limit(s.n);
 }
 
-// One thread per body (slot_parts = 1).  SB: slots loaded together (a grid run in waves gives an i-block tens of
-// slots; an ensemble of small clusters a few, where a narrower batch keeps
-// registers, and so resident warps, for the memory latency)
-// Float-pair partial sums in slot order.
+// One thread per body (slot_parts = 1): float-pair partial sums in slot order.  SB:
+// slots loaded together (a grid run in waves gives an i-block tens of slots; an
+// ensemble of small clusters a few, where a narrower batch keeps registers, and so
+// resident warps, for the memory latency).
 template <int SB>
 __device__ __forceinline__ void sum_slots_ff(const DevState &s, const SlotRun &run,
                                              double &ax, double &ay, double &az)

@@ -22,10 +22,10 @@
 // is fixed by the decomposition: results are bit-reproducible.
 //
 // The warps' j sums of a unit meet in a slab in shared memory, one unit later
-// (three slabs; phase_wait, so no warp stops for the others); each j body's
-// four are added in warp order and go to the partial slot of the tile's delta.  The i sums go to a slot per (row,
-// block).  The consumers (the kick, the acceleration output) add a body's
-// slots in order.
+// (three slabs; phase_wait, so no warp stops for the others); each j body's four
+// are added in warp order and go to the partial slot of the tile's delta.  The i
+// sums go to a slot per (row, block).  The consumers (the kick, the acceleration
+// output) add a body's slots in order.
 //
 // The tile of a block with itself: the chunk's bodies lie in the row of one
 // warp r.  That warp sums them without the j side (so its own row is a full

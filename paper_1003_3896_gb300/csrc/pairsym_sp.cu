@@ -12,7 +12,10 @@
 // slots).  Packing two j bodies of a lane, not two i bodies of a thread, halves
 // the shuffles and staged reads per pair at the same registers and i-block
 // width: 1.047 against 1.092 ms; eight i bodies against four 1.047 : 1.098, with
-// four steps unrolled (one 1.059, two 1.094, eight 1.140).
+// four steps unrolled (one 1.059, two 1.094, eight 1.140).  With a mass spectrum
+// 1.276 ms at N = 65536 (FMA pipe 76% busy), 19.1 at 262144; with the cube of the
+// inverse distance shared by both sides, one operation fewer, 18.9 at 262144, but
+// that cube leaves the float range beyond 4e12 length units.
 #include "pairsym.cuh"
 
 namespace nb {

@@ -73,11 +73,11 @@ __device__ __forceinline__ double widen(float f)
 //        R^(-3/2) = y0^3 (1 + m), m = 3 v / 2 + v^2 (15/8 + 35/16 v + O(v^2)): the
 //        dropped terms are below 2^-62, and the v^2 term, below 2^-30.8, needs
 //        only float precision.
-// Within 1.1 and 1.4 units of 2^-53 of the exact powers (emulated); before, with y0 to 24 bits, y0^2
-// and y0^3 and the whole series in double, five and six operations and 1.5 and
-// 3.3 units.  N = 16384 FP64 evaluation 4.65 -> 3.83 ms, energy of N = 32768
-// 11.8 -> 9.7 ms.  R outside the float range (the padding's 1e300, R = 0,
-// non-finite R) takes the library rsqrt.
+// Within 1.1 and 1.4 units of 2^-53 of the exact powers (emulated).  The form with
+// y0 to 24 bits and its powers and the whole series in double takes five and six
+// operations and is within 1.5 and 3.3 units: N = 16384 FP64 evaluation 4.65 ms
+// with it, 3.83 with this one; energy of N = 32768 11.8 and 9.7 ms.  R outside the
+// float range (the padding's 1e300, R = 0, non-finite R) takes the library rsqrt.
 template <bool POT>
 __device__ __forceinline__ double rsqrt_pow(double R)
 {
