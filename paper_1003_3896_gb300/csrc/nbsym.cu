@@ -169,10 +169,12 @@ int replan(nb_ctx *c, int64_t n)
     int rc = set_define(c->set, (int32_t)nk.size(), boff.data(), nk.data(), c->eps_k.data(),
                         c->dts_k.data());
     if (rc) return rc;
+    // masses not seen yet: the equal-mass kernels' plan, which reserves the most (the
+    // load plans again for the masses it finds)
     if (c->mu_k.size() == nk.size())
         c->set.mu = c->mu_k;
     else
-        c->set.mu.assign(nk.size(), 0.0);
+        c->set.mu.assign(nk.size(), 1.0);
     rc = plan_make(c->pool, c->set, c->p.precision, c->stream, c->plan);
     if (rc) return rc;
     c->small = small_ok(c->set, c->plan, c->phys);
@@ -447,6 +449,7 @@ static int load_common(nb_ctx *c, int64_t n, const double *pos, const double *ve
         if (rc) return rc;
     }
     c->n = n;
+    c->planned = false;   // until the system is in place
     const double *dp = pos, *dv = vel, *dm = mass;
     if (kind == cudaMemcpyHostToDevice) {
         double *sp = c->pool.stage, *sv = sp + 3 * c->pool.cap, *sm = sp + 6 * c->pool.cap;
@@ -476,6 +479,7 @@ static int load_common(nb_ctx *c, int64_t n, const double *pos, const double *ve
         int rc = replan(c, n);
         if (rc) return rc;
     }
+    c->planned = true;
     c->split_stale = true;
     return NB_OK;
 }

@@ -343,3 +343,14 @@ def test_which_steps_run_in_one_kernel(host, prec, n, order, one):
         host.clear()
         c.step(order, 1e-3, 3)
         assert not host.ran("small_step_kernel") and host.graphs == 3
+
+
+@pytest.mark.parametrize("prec", ["ds", "fp64", "dd"])
+def test_first_load_reserves_once(host, prec):
+    """The plan before the masses are known takes no less than the one after: no large
+    storage is freed and allocated again."""
+    host.fail_from()
+    with host.nbsym.Context(N, eps=1e-2, precision=prec) as c:
+        host.clear()
+        c.load(*ics.plummer(N, 1))
+        assert host.syncing <= 2   # partial sums, encounter sums
