@@ -68,7 +68,11 @@ typedef struct nb_ctx nb_ctx;
  *             sets; lets a caller (or a test) run that form on systems small
  *             enough to check step by step against a slow reference.
  * In every mode the state (positions, velocities), the kick/drift update,
- * the external field and the energy diagnostic are double precision. */
+ * the external field and the energy diagnostic are double precision.
+ * Units: in all modes but NB_FP64 a pair's r^2 + eps^2 and m / r^3 have to lie
+ * in the range of floats (1.2e-38 to 3.4e38); where all masses of a cluster are
+ * equal, and in NB_DD, 1 / r^3 as well, that is distances (softened) between
+ * 1.5e-13 and 4e12 length units. */
 enum nb_precision { NB_FP64 = 0, NB_DS = 1, NB_FP32 = 2, NB_DS_FULL = 3, NB_DD = 4,
                     NB_DS_NEAR = 5 };
 
